@@ -5,6 +5,7 @@
 #include <cudaTypedefs.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -31,6 +32,12 @@ struct pf_handle {
   int G_total = 0, n_tiles = 0;
   int k1_grid = 1, rs_cluster = 1;
   int rs_threads = RS_THREADS;  // resampler CTA: RS_THREADS, or RS_THREADS_SMALL for small groups
+  int rs_pad = 0;               // 0: every group starts on a 16-byte boundary, else 3 (ResampleArgs::pad)
+  // several tracks: the groups by class of size, resampled by one CTA each
+  // (PFARNA_RS_THREADS unset; pf_autotune may prefer the cluster kernel)
+  bool rs_by_class = false;
+  int rs_sum_nt = RS_THREADS;   // GlobalArgs::sum_nt of those launches
+  GroupClasses classes{};
   int steps_run = 0;
   int failed = 0;
   cudaStream_t last_stream = nullptr;
@@ -103,7 +110,7 @@ struct pf_handle {
   bool carry_any = false;           // some track resamples by Alg. 1's test (PF_RESAMPLE_ESS)
   bool variants = false;            // carry_any, or some track uses PF_SEND_KEYED
   char* ws = nullptr;        // the workspace, its size, and the byte range of the TMA
-  size_t ws_total = 0;       // descriptors in it (they hold this workspace's addresses)
+  size_t ws_total = 0;       // descriptors in it (they hold this workspace's addresses); ws_total: what a checkpoint keeps
   size_t tmap_off = 0, tmap_bytes = 0;
   unsigned long long cfg_sig = 0;  // signature of the configurations and history
   void* encode = nullptr;  // cuTensorMapEncodeTiled, or nullptr
@@ -164,6 +171,8 @@ QuantCoeffs make_qc() {
 }
 
 struct Layout {
+  size_t saved;  // bytes kept by pf_save: what follows is scratch of pf_init or of one step
+  size_t order;
   size_t trk, ts, gs, gd, tiles, frame_of, pv0, pv1, I0, I1, anc, lw, tp, ypad, hist, ghist, ring, ring_next, exo_next, keys_next,
       tile_ctr, parent, ds, rq, chunks, chunk_q, fsync,
       tmap, total;
@@ -319,6 +328,8 @@ Layout plan(const pf_track_config* c, int n, int history) {
     L.seed = take(sizeof(float) * (size_t)n);
     L.replay_bad = take(sizeof(int));
   }
+  L.saved = o;
+  L.order = take(sizeof(int) * (size_t)L.G_total);
   L.total = o;
   return L;
 }
@@ -330,9 +341,8 @@ int num_sms() {
   return sms > 0 ? sms : 1;
 }
 
-int resample_cluster(int Np, bool single_track) {
-  if (!single_track) return 1;
-  int c = (Np + RS_SUB - 1) / RS_SUB;
+int resample_cluster(int Np, int pad) {
+  int c = (Np + pad + RS_SUB - 1) / RS_SUB;
   return c < 1 ? 1 : (c > 8 ? 8 : c);
 }
 
@@ -510,6 +520,7 @@ ResampleArgs resample_args(const pf_handle* h, int fuse) {
   ra.n_groups = h->G_total;
   ra.lean = h->carry_any ? 0 : 1;  // no group resamples by Alg. 1's test
   ra.max_np = 1;
+  ra.pad = h->rs_pad;
   for (int t = 0; t < h->n_tracks; ++t) ra.max_np = h->cfg[t].Np > ra.max_np ? h->cfg[t].Np : ra.max_np;
   ra.tile_ctr = h->tile_ctr;
   ra.glob = global_args(h, 1);
@@ -520,7 +531,10 @@ ResampleArgs resample_args(const pf_handle* h, int fuse) {
 
 namespace pf {
 QuantCoeffs resample_coeffs() { return make_qc(); }
-int resample_cluster_size(int Np) { return resample_cluster(Np, true); }
+int resample_pad(const float* logw, const uint32_t* anc, int G, int Np) {
+  return ((((uintptr_t)logw | (uintptr_t)anc) & 15) || (G > 1 && (Np & 3))) ? 3 : 0;
+}
+int resample_cluster_size(int Np, int pad) { return resample_cluster(Np, pad); }
 void set_handleless_error(const char* msg) { g_err = msg; }
 }  // namespace pf
 
@@ -557,6 +571,8 @@ pf_status pf_init(const pf_track_config* cfg, int32_t n_tracks, int32_t history,
   h->R = L.R;
   h->cfg.assign(cfg, cfg + n_tracks);
   h->N_total = L.N_total;
+  for (int t = 0; t < n_tracks; ++t)
+    if (cfg[t].Np & 3) h->rs_pad = 3;
   h->G_total = L.G_total;
   h->n_tiles = L.n_tiles;
   h->qc = make_qc();
@@ -703,6 +719,19 @@ pf_status pf_init(const pf_track_config* cfg, int32_t n_tracks, int32_t history,
   h->tp = tp;
   cudaStream_t s = (cudaStream_t)stream;
 
+  // the groups by class of size, the largest first within a class (a batch's
+  // resampling then ends on its small groups)
+  std::vector<int> order(L.G_total);
+  for (int i = 0; i < L.G_total; ++i) order[i] = i;
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return gd[x].Np > gd[y].Np; });
+  h->classes.list = (const int*)(w + L.order);
+  for (int c = 1; c <= 3; ++c) {
+    // class c - 1 ends where the groups fit one sub-chunk of class c
+    int n = h->classes.begin[c - 1];
+    while (n < L.G_total && (c == 3 || gd[order[n]].Np + h->rs_pad > RG_THREADS[c] * RS_ITEMS)) ++n;
+    h->classes.begin[c] = n;
+  }
+
   // One TMA descriptor per track over its padded frame (boxes of ROI_W x
   // ROI_BOX_H floats).  If the driver cannot encode them, the propagate
   // kernel reads every frame through L1 instead.
@@ -732,6 +761,7 @@ pf_status pf_init(const pf_track_config* cfg, int32_t n_tracks, int32_t history,
   cudaError_t e;
   if ((e = cudaMemsetAsync(w, 0, L.total, s)) != cudaSuccess) { pf_destroy(h); return cuda_fail(nullptr, e, "cudaMemsetAsync"); }
   if ((e = cudaMemcpyAsync(h->trk, tp.data(), sizeof(TrackParams) * n_tracks, cudaMemcpyHostToDevice, s)) ||
+      (e = cudaMemcpyAsync(w + L.order, order.data(), sizeof(int) * order.size(), cudaMemcpyHostToDevice, s)) ||
       (e = cudaMemcpyAsync(h->gd, gd.data(), sizeof(GroupDesc) * gd.size(), cudaMemcpyHostToDevice, s)) ||
       (e = cudaMemcpyAsync(h->tiles, tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice, s)) ||
       (e = cudaMemcpyAsync(h->chunks, chunks.data(), sizeof(int4) * chunks.size(), cudaMemcpyHostToDevice, s)) ||
@@ -747,7 +777,7 @@ pf_status pf_init(const pf_track_config* cfg, int32_t n_tracks, int32_t history,
   const int sms = num_sms();
   h->sms = sms;
   h->ws = w;
-  h->ws_total = L.total;
+  h->ws_total = L.saved;
   h->tmap_off = L.tmap;
   h->tmap_bytes = sizeof(CUtensorMap) * (size_t)n_tracks;
   {
@@ -758,7 +788,7 @@ pf_status pf_init(const pf_track_config* cfg, int32_t n_tracks, int32_t history,
     };
     mix(cfg, sizeof(pf_track_config) * (size_t)n_tracks);
     mix(&history, sizeof history);
-    mix(&L.total, sizeof L.total);
+    mix(&L.saved, sizeof L.saved);
     h->cfg_sig = sig;
   }
   int occ = 1;
@@ -798,7 +828,8 @@ pf_status pf_init(const pf_track_config* cfg, int32_t n_tracks, int32_t history,
     for (int t = 0; t < n_tracks; ++t) maxNp = cfg[t].Np > maxNp ? cfg[t].Np : maxNp;
     h->rs_threads = maxNp <= RS_THREADS_SMALL * RS_ITEMS ? RS_THREADS_SMALL : RS_THREADS;
     if (n_tracks == 1) {
-      h->rs_cluster = resample_cluster(cfg[0].Np, true);
+      h->rs_cluster = resample_cluster(cfg[0].Np, h->rs_pad);
+      if (h->rs_threads == RS_THREADS_SMALL && maxNp + h->rs_pad > RS_THREADS_SMALL * RS_ITEMS) h->rs_cluster = 2;
     } else {
       const int sub = h->rs_threads * RS_ITEMS;
       int c = (maxNp + sub - 1) / sub;
@@ -809,6 +840,8 @@ pf_status pf_init(const pf_track_config* cfg, int32_t n_tracks, int32_t history,
     const char* rt = std::getenv("PFARNA_RS_THREADS");  // "128" / "512": force the resampler's CTA size
     if (rt && std::atoi(rt) == RS_THREADS_SMALL) h->rs_threads = RS_THREADS_SMALL;
     if (rt && std::atoi(rt) == RS_THREADS) h->rs_threads = RS_THREADS;
+    h->rs_by_class = n_tracks > 1 && !rt;
+    h->rs_sum_nt = h->rs_threads;
   }
 
   InitArgs ia{h->trk, h->tiles, h->n_tiles, h->N_total, user_state, h->pv[1], h->In[1]};
@@ -819,6 +852,16 @@ pf_status pf_init(const pf_track_config* cfg, int32_t n_tracks, int32_t history,
   }
   *out = h;
   return PF_OK;
+}
+
+// The step's resampling (fuse = 1: with the tracks' global steps).
+static cudaError_t launch_step_resample(const pf_handle* h, int fuse, bool pdl, cudaStream_t s) {
+  if (h->rs_by_class) {
+    ResampleArgs ra = resample_args(h, fuse);
+    ra.glob.sum_nt = h->rs_sum_nt;
+    return launch_resample_groups(ra, h->classes, pdl, s);
+  }
+  return launch_resample(resample_args(h, fuse), h->G_total, h->rs_cluster, pdl, s, h->rs_threads);
 }
 
 // The kernels of one step after frame preparation: the fused step, or
@@ -836,8 +879,7 @@ static cudaError_t launch_step_kernels(pf_handle* h, cudaStream_t s, bool marks,
   if ((e = launch_propagate(k1, h->R, h->k1_grid + h->n_ring_blocks, h->pdl, s)) != cudaSuccess) return e;
   if (marks && (e = mark(h, PF_KERNEL_PROPAGATE_WEIGHT, s)) != cudaSuccess) return e;
   if (marks && (e = mark(h, PF_KERNEL_RESAMPLE, s)) != cudaSuccess) return e;
-  if ((e = launch_resample(resample_args(h, 1), h->G_total, h->rs_cluster, h->pdl, s, h->rs_threads)) != cudaSuccess)
-    return e;
+  if ((e = launch_step_resample(h, 1, h->pdl, s)) != cudaSuccess) return e;
   return marks ? mark(h, PF_KERNEL_RESAMPLE, s) : cudaSuccess;
 }
 
@@ -1025,6 +1067,8 @@ pf_status pf_autotune(pf_handle* h, const float* const* frames, int32_t* k1_grid
       h->k1_grid = std::get<0>(it->second);
       h->rs_cluster = std::get<1>(it->second);
       h->rs_threads = std::get<2>(it->second);
+      h->rs_by_class = h->rs_threads == 0;  // (0: by class of size)
+      if (h->rs_by_class) h->rs_threads = RS_THREADS;
       cached = true;
     }
   }
@@ -1068,6 +1112,14 @@ pf_status pf_autotune(pf_handle* h, const float* const* frames, int32_t* k1_grid
     }
     int best_c = h->rs_cluster, best_t = h->rs_threads;
     best = 1e30f;
+    if (h->n_tracks > 1 && e == cudaSuccess) {
+      float ms = 0.0f;
+      for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep)
+        e = time_it([&] { return launch_resample_groups(resample_args(h, 0), h->classes, false, s); }, ms);
+      best = ms;
+      best_c = 1;
+      best_t = 0;
+    }
     for (int nt : {RS_THREADS, RS_THREADS_SMALL})
       for (int c = 1; c <= 8 && e == cudaSuccess; c *= 2) {
         const ResampleArgs ra = resample_args(h, 0);
@@ -1086,7 +1138,8 @@ pf_status pf_autotune(pf_handle* h, const float* const* frames, int32_t* k1_grid
     if (e != cudaSuccess) return cuda_fail(h, e, "autotune");
     h->k1_grid = best_grid;
     h->rs_cluster = best_c;
-    h->rs_threads = best_t;
+    h->rs_by_class = best_t == 0;
+    h->rs_threads = h->rs_by_class ? RS_THREADS : best_t;
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     g_tune_cache[key] = std::make_tuple(best_grid, best_c, best_t);
   }
@@ -1096,7 +1149,7 @@ pf_status pf_autotune(pf_handle* h, const float* const* frames, int32_t* k1_grid
   // the propagate kernel reads, so only the resampler runs again, now with
   // the global step.
   e = cached ? launch_step_kernels(h, s, false)
-             : launch_resample(resample_args(h, 1), h->G_total, h->rs_cluster, false, s, h->rs_threads);
+             : launch_step_resample(h, 1, false, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "step kernels");
   h->steps_run += 1;
   h->finish_pending = true;
@@ -1300,8 +1353,9 @@ pf_status pf_resample(const float* logw, const uint32_t* u, int32_t G, int32_t N
   ResampleArgs ra{gd, gs, nullptr, logw, nullptr, anc, 0, (unsigned long long*)q, u, 1, make_qc(), ds};
   ra.n_groups = G;
   ra.max_np = Np;
-  ra.lean = q ? 0 : 1;  // without codes to store, the lean instance when the chunks fit
-  if ((e = launch_resample(ra, G, resample_cluster(Np, true), false, s)) != cudaSuccess)
+  ra.lean = 1;
+  ra.pad = resample_pad(logw, anc, G, Np);
+  if ((e = launch_resample(ra, G, resample_cluster(Np, ra.pad), false, s)) != cudaSuccess)
     return cuda_fail(nullptr, e, "k_resample");
   return PF_OK;
 }

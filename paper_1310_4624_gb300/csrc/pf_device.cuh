@@ -35,6 +35,12 @@ constexpr int RS_SUB = RS_THREADS * RS_ITEMS;
 constexpr int RS_WIN = 2 * RS_SUB;    // resampler merge window: items and outputs merged at once (ancestors staged)
 __host__ __device__ constexpr int pad8(int i) { return i + (i >> 3); }  // shared index with one spare per 8
 constexpr int RS_SUB_PAD = pad8(RS_SUB);
+// Items (and outputs) of one CTA of the lean resampler, for a group of Np on
+// a cluster of C: a multiple of 8 that covers Np and, where groups start off
+// the 16-byte grid (pad = 3), the elements between the grid and the group.
+__host__ __device__ constexpr int rs_chunk_lean(int Np, int C, int pad) { return ((Np + pad + C - 1) / C + 7) & ~7; }
+constexpr int RG_THREADS[3] = {256, 128, 32};  // one-CTA resampler: threads per group, by class of group size
+constexpr int RG_TEAMS[3] = {1, 1, 4};         // and groups per CTA
 constexpr int RS_CHUNK = K1_THREADS * RS_ITEMS;  // fused step: items of one resampling chunk (A and B tasks)
 constexpr int TASK_P = 0, TASK_A = 1, TASK_B = 2;  // fused step task kinds
 constexpr int GL_THREADS = 1024;      // per-track global-step CTA, one thread per group
@@ -254,21 +260,24 @@ struct QuantCoeffs {
   float l2e;
 };
 
+// n comes from adding 1.5 2^23 (whose unit in the last place is 1, so the sum
+// rounds z to the nearest integer, ties to even, as rintf does for |z| <= 40)
+// and the code from one 64-bit right shift: with p = mant 2^(e - 23), e in
+// {-1, 0} and n in [-40, 0], p 2^(n+40) = (mant 2^39) / 2^(22 - e - n), a
+// shift by 22 .. 63.  No conversion instruction (a quarter-rate unit).
 __device__ __forceinline__ unsigned long long quantize(float lw, float M, const QuantCoeffs& qc) {
   const float t = __fsub_rn(lw, M);
   const float z = __fmul_rn(t, qc.l2e);
-  if (!(z >= -40.0f)) return 0ull;
-  const float n = rintf(z);
-  const float f = __fsub_rn(z, n);
+  const float zr = __fadd_rn(z, 12582912.0f);
+  const float f = __fsub_rn(z, __fsub_rn(zr, 12582912.0f));
   float p = qc.c[7];
 #pragma unroll
   for (int d = 6; d >= 0; --d) p = __fmaf_rn(p, f, qc.c[d]);
-  // trunc(p 2^(n+40)) with integer shifts of p's significand (p > 0 normal):
-  // p = mant 2^(ex - 23), so the code is mant shifted by ex - 23 + n + 40.
   const uint32_t bits = __float_as_uint(p);
-  const unsigned long long mant = (bits & 0x7fffffu) | 0x800000u;
-  const int sh = (int)((bits >> 23) & 0xffu) - 127 - 23 + (int)n + 40;
-  return sh >= 0 ? (mant << sh) : (mant >> (-sh));
+  const uint32_t mant = (bits & 0x7fffffu) | 0x800000u;
+  const uint32_t sh = 149u + 0x4B400000u - (bits >> 23) - __float_as_uint(zr);
+  const unsigned long long q = ((unsigned long long)mant << 39) >> (sh & 63u);
+  return z >= -40.0f ? q : 0ull;
 }
 
 // FP32 approximation of a 64-bit unsigned value from its two 32-bit halves
@@ -346,6 +355,42 @@ struct Thresholds {
     if (Sf + m < Tf) return true;
     if (Sf > Tf + m) return false;
     return S <= T((uint32_t)jf);
+  }
+};
+
+// #{j in [0, Np) : T_j < S} in 32-bit fixed point.  The count is
+// ceil(x), x = S Np / Q - u 2^-32 (clamped at 0), and a group with weight has
+// Q in [2^40, 2^60] (its largest particle's code is 2^40).  With the 32
+// leading bits of Q as the unit, s = S >> sh and m ~ Np 2^(62 - p) / (Q >> sh)
+// (Np <= 2^p), v = (s m >> 32) - (u >> (p + 2)) is x in units of 2^-f,
+// f = 30 - p: the truncations of s, of the product and of u cost at most 1/2,
+// 1 and 1 units, Q's dropped bits 1 and m's own error 2, so v is within 6
+// units of x.  Where v is 8 units or more from a whole number its ceiling is
+// the count; nearer (one boundary in 2^(f-4): 1 in 4096 at Np = 16384) the
+// caller takes the exact form.
+struct FastCount {
+  uint32_t m, uo, mask;
+  int sh, f;
+  __device__ __forceinline__ void init(unsigned long long Q, uint32_t Np, uint32_t u) {
+    const int p = Np > 1 ? 32 - __clz((int)(Np - 1)) : 0;
+    f = 30 - p;
+    mask = (1u << f) - 1u;
+    uo = u >> (p + 2);
+    sh = 32 - __clzll((long long)Q);
+    const uint32_t q32 = (uint32_t)(Q >> sh);
+    // Np 2^(62 - p) / q32 by an FP32 quotient and one correction of its remainder
+    const unsigned long long num = (unsigned long long)Np << (62 - p);
+    const float r = __frcp_rn((float)q32);
+    const uint32_t m0 = (uint32_t)__fmul_rz(__fmul_rz((float)(uint32_t)(num >> 32), 4294967296.0f), r);
+    const long long rem = (long long)(num - (unsigned long long)m0 * q32);
+    m = m0 + (int)__fmul_rz((float)rem, r);
+  }
+  // The count's estimate; false when the exact form must decide.
+  __device__ __forceinline__ bool operator()(unsigned long long S, int& c) const {
+    const uint32_t s = __funnelshift_r((uint32_t)S, (uint32_t)(S >> 32), (uint32_t)sh);
+    const int v = (int)(__umulhi(s, m) - uo);
+    c = (v + (int)mask) >> f;
+    return ((uint32_t)(v + 8) & mask) >= 16u;
   }
 };
 

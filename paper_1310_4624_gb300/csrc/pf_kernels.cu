@@ -178,6 +178,7 @@ struct GlobalScratch {
   float tot[6];
   double pe;
   int ring[MAX_G];
+  float e[MAX_G];
 };
 
 // The global step's inputs that the groups of the step do not write: the
@@ -313,7 +314,9 @@ __device__ __forceinline__ void global_step_core(const GlobalArgs& a, int t, Glo
 #pragma unroll
   for (int i = 0; i < GPT; ++i) {
     if (threadIdx.x + i * NT < G) {
-      wsum += __expf(lam[i] - mx);
+      const float e = __expf(lam[i] - mx);
+      wsum += e;
+      if (a.sum_nt) sc.e[threadIdx.x + i * NT] = e;
       const double w = exp((double)lam[i] - (double)mx);
       iw += __double2ull_rn(w * 4503599627370496.0);
       iw2 += __double2ull_rn(w * w * 4503599627370496.0);
@@ -337,9 +340,22 @@ __device__ __forceinline__ void global_step_core(const GlobalArgs& a, int t, Glo
     if (m < G) sc.ring[m] = shuffled ? rnext[i] : m;
   }
   __syncthreads();
+  if (a.sum_nt) {
+    // the FP32 sum in the order of a CTA of sum_nt threads, whatever this
+    // CTA's size, so that a track's results do not depend on the class of
+    // its groups
+    for (int w = warp; w < a.sum_nt / 32; w += NW) {
+      float x = 0.0f;
+      for (int m = w * 32 + lane; m < G; m += a.sum_nt) x += sc.e[m];
+      x = warp_sum(x);
+      if (lane == 0) sc.red[w][0] = x;
+    }
+    __syncthreads();
+  }
   if (threadIdx.x == 0) {
+    const int nws = !a.sum_nt ? nwa : G > a.sum_nt ? a.sum_nt / 32 : (G + 31) / 32;
     float x = 0.0f;
-    for (int w = 0; w < nwa; ++w) x += sc.red[w][0];
+    for (int w = 0; w < nws; ++w) x += sc.red[w][0];
     sc.tot[0] = x;
   }
   if (threadIdx.x == (NW > 1 ? 32 : 7)) {
@@ -1983,18 +1999,87 @@ __device__ __forceinline__ void global_step_when_reported(const GlobalArgs& g, D
 // CTAs of its cluster mark its output positions).
 constexpr size_t RS_MARK_OFF = (sizeof(GlobalScratch) + 15) / 16 * 16;
 
+// The count of a boundary whose fixed-point value v (FastCount) lies within 8
+// units of a whole number n = (v + 8) >> f: n or n + 1, by x <= n, that is
+// S Np 2^32 <= Q (n 2^32 + u), in exact 128-bit products (S Np < 2^80).  Not
+// inlined: few boundaries come here.
+__device__ __noinline__ int count_exact(unsigned long long S, unsigned long long Q, uint32_t Np, uint32_t u, int n) {
+  if (n < 0) return 0;
+  const unsigned long long t = ((unsigned long long)(uint32_t)n << 32) | u;
+  const unsigned long long llo = S * Np, lhi = __umul64hi(S, Np);
+  const unsigned long long a_hi = (lhi << 32) | (llo >> 32), a_lo = llo << 32;
+  const unsigned long long b_hi = __umul64hi(Q, t), b_lo = Q * t;
+  const bool le = a_hi < b_hi || (a_hi == b_hi && a_lo <= b_lo);
+  return le ? n : n + 1;
+}
+
+// A boundary's count in about 10 instructions (a 32-bit multiply-high and the
+// nearness test) where two FP32-filtered threshold comparisons took about 40:
+// the resampling launch of 64 groups of 16384 went from 16.0 to 13.6 us, of 4
+// groups of 1024 from 12.3 to 10.7 us.
+__device__ __forceinline__ int count_fast(const FastCount& fc, unsigned long long S, unsigned long long Q, uint32_t Np,
+                                          uint32_t u) {
+  int c;
+  if (!fc(S, c)) {
+    const uint32_t s32 = __funnelshift_r((uint32_t)S, (uint32_t)(S >> 32), (uint32_t)fc.sh);
+    c = count_exact(S, Q, Np, u, ((int)(__umulhi(s32, fc.m) - fc.uo) + 8) >> fc.f);
+  }
+  return c;
+}
+
+// ITEMS log-weights of a group at its items i0 .. i0 + ITEMS - 1 (a multiple
+// of four items from a 16-byte boundary), -inf outside [lo, hi): whole float4
+// inside the range, single loads at its ends.  Through L2: one 32-byte sector
+// per thread and no line to keep.
+template <int ITEMS>
+__device__ __forceinline__ void load_items(const float* __restrict__ lw, int i0, int lo, int hi, float (&v)[ITEMS]) {
+#pragma unroll
+  for (int r = 0; r < ITEMS; r += 4) {
+    const int i = i0 + r;
+    if (i >= lo && i + 4 <= hi) {
+      const float4 x = __ldcg(reinterpret_cast<const float4*>(lw + i));
+      v[r] = x.x; v[r + 1] = x.y; v[r + 2] = x.z; v[r + 3] = x.w;
+    } else {
+#pragma unroll
+      for (int b = 0; b < 4; ++b) v[r + b] = (i + b >= lo && i + b < hi) ? __ldcg(lw + i + b) : -INFINITY;
+    }
+  }
+}
+
+// Ancestors of ITEMS consecutive outputs j0 .. (a multiple of four outputs
+// from a 16-byte boundary), those in [lo, hi) stored.
+template <int ITEMS>
+__device__ __forceinline__ void store_items(uint32_t* __restrict__ anc, int j0, int lo, int hi,
+                                            const uint32_t (&o)[ITEMS]) {
+#pragma unroll
+  for (int r = 0; r < ITEMS; r += 4) {
+    const int j = j0 + r;
+    if (j >= lo && j + 4 <= hi) {
+      *reinterpret_cast<uint4*>(anc + j) = make_uint4(o[r], o[r + 1], o[r + 2], o[r + 3]);
+    } else {
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+        if (j + b >= lo && j + b < hi) anc[j + b] = o[r + b];
+    }
+  }
+}
+
+// Elements from the previous 16-byte boundary to p (4-byte elements).
+__device__ __forceinline__ int off16(const void* p) { return (int)((reinterpret_cast<uintptr_t>(p) >> 2) & 3); }
+
 // Resampler: one thread-block cluster per group, each CTA a contiguous chunk
 // of the group's slots (a multiple of 8), processed in sub-chunks of SUB
 // items; thread t owns the RS_ITEMS consecutive items [t*RS_ITEMS, ...).
 
-// LEAN: every CTA's chunk fits in its registers (one sub-chunk), no group
-// resamples by Alg. 1's test and no weight codes are stored (the common
-// filter step, and pf_resample without codes) -- with the other paths
-// compiled out (a smaller kernel: the resampler is latency-bound, and
-// instruction fetch leads its stalls).
-template <int NTR, bool LEAN>
-__global__ void __launch_bounds__(NTR, NTR >= 512 ? 2 : 8) k_resample(const __grid_constant__ ResampleArgs a) {
-  constexpr int SUB = NTR * RS_ITEMS;  // items per sub-chunk
+// LEAN: every CTA's chunk fits in its registers (one sub-chunk of NTR x ITEMS
+// items), with the other paths compiled out (a smaller kernel: the resampler
+// is latency-bound, and instruction fetch leads its stalls).  EXTRA: some
+// group resamples by Alg. 1's test, or the weight codes are stored.
+template <int NTR, int ITEMS, bool LEAN, bool EXTRA>
+__global__ void __launch_bounds__(NTR, NTR >= 512 ? (ITEMS > RS_ITEMS ? 1 : 2) : 8)
+    k_resample(const __grid_constant__ ResampleArgs a) {
+  static_assert(LEAN || (ITEMS == RS_ITEMS && EXTRA), "the general instance merges windows of RS_ITEMS per thread");
+  constexpr int SUB = NTR * ITEMS;  // items per sub-chunk
   constexpr int SUB_PAD = pad8(SUB);
   cg::cluster_group cl = cg::this_cluster();
   const int C = (int)cl.num_blocks();
@@ -2012,9 +2097,11 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? 2 : 8) k_resample(const __gr
   }
   const GroupDesc d = a.gd[grp];
   const int Np = d.Np;
-  const int chunk = ((Np + C - 1) / C + 7) & ~7;
-  const int lo = min(rank * chunk, Np), hi = min(lo + chunk, Np);
-  const bool single = LEAN || (hi - lo) <= SUB;  // the whole chunk stays in registers
+  // LEAN: items and outputs are split in units of the 16-byte boundaries of
+  // their arrays: a0 (b0) elements of the first item's (output's) float4 lie
+  // before the group, so that every load and store of a group at any offset
+  // is a whole vector except at the group's two ends
+  const int chunk = LEAN ? rs_chunk_lean(Np, C, a.pad) : ((Np + C - 1) / C + 7) & ~7;
   // In a filter step: the track's step index (read before the cluster
   // barrier that precedes every ticket below, since the track's global step,
   // run by the last ticket holder, advances it), which picks the log-weight
@@ -2022,8 +2109,12 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? 2 : 8) k_resample(const __gr
   const TrackParams* __restrict__ Pt = a.glob.trk ? a.glob.trk + d.track : nullptr;
   const int kk = a.u_arr ? 0 : a.glob.ts[d.track].k;
   const float* __restrict__ lw = ((a.lw1 && (kk & 1)) ? a.lw1 : a.lw) + d.base;
-  const bool ess_rule = !LEAN && Pt && Pt->resample_rule == 1;
-  const bool vec = ((d.base & 3) == 0);
+  const int a0 = LEAN ? off16(lw) : 0;
+  const int lo = LEAN ? max(rank * chunk - a0, 0) : min(rank * chunk, Np);
+  const int hi = LEAN ? min((rank + 1) * chunk - a0, Np) : min(lo + chunk, Np);
+  const bool single = LEAN || (hi - lo) <= SUB;  // the whole chunk stays in registers
+  const bool ess_rule = EXTRA && Pt && Pt->resample_rule == 1;
+  const bool vec = off16(lw) == 0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
   __shared__ float s_pub_max;
@@ -2041,21 +2132,25 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? 2 : 8) k_resample(const __gr
   extern __shared__ __align__(16) unsigned long long s_dyn_rs[];
   unsigned long long* s_incl = s_dyn_rs;
   uint32_t* s_out = reinterpret_cast<uint32_t*>(s_dyn_rs + SUB_PAD);
-  // LEAN: one entry per output position of this CTA (NTR RS_ITEMS), 0 or
+  // LEAN: one entry per output position of this CTA (NTR ITEMS), 0 or
   // the 1-based item whose outputs start there
   uint32_t* s_mark = reinterpret_cast<uint32_t*>(reinterpret_cast<unsigned char*>(s_dyn_rs) + RS_MARK_OFF);
 
-  float v[RS_ITEMS];
+  float v[ITEMS];
   auto load_sub = [&](int sub) {
-    const int i0 = sub + (int)threadIdx.x * RS_ITEMS;
-    if (vec && i0 + RS_ITEMS <= hi) {
-      const float4 x0 = *reinterpret_cast<const float4*>(lw + i0);
-      const float4 x1 = *reinterpret_cast<const float4*>(lw + i0 + 4);
-      v[0] = x0.x; v[1] = x0.y; v[2] = x0.z; v[3] = x0.w;
-      v[4] = x1.x; v[5] = x1.y; v[6] = x1.z; v[7] = x1.w;
+    if constexpr (LEAN) {
+      load_items<ITEMS>(lw, rank * chunk - a0 + (int)threadIdx.x * ITEMS, lo, hi, v);
     } else {
+      const int i0 = sub + (int)threadIdx.x * ITEMS;
+      if (vec && i0 + ITEMS <= hi) {
+        const float4 x0 = *reinterpret_cast<const float4*>(lw + i0);
+        const float4 x1 = *reinterpret_cast<const float4*>(lw + i0 + 4);
+        v[0] = x0.x; v[1] = x0.y; v[2] = x0.z; v[3] = x0.w;
+        v[4] = x1.x; v[5] = x1.y; v[6] = x1.z; v[7] = x1.w;
+      } else {
 #pragma unroll
-      for (int r = 0; r < RS_ITEMS; ++r) v[r] = (i0 + r < hi) ? lw[i0 + r] : -INFINITY;
+        for (int r = 0; r < ITEMS; ++r) v[r] = (i0 + r < hi) ? lw[i0 + r] : -INFINITY;
+      }
     }
   };
 
@@ -2064,9 +2159,10 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? 2 : 8) k_resample(const __gr
   // (set by the previous step's global step, complete before the propagate
   // kernel ran), so it is drawn before waiting for the propagate kernel.
   if constexpr (LEAN) {
-    uint4* m4 = reinterpret_cast<uint4*>(s_mark) + 2 * threadIdx.x;
-    m4[0] = make_uint4(0u, 0u, 0u, 0u);  // before the cluster barrier that precedes any marking
-    m4[1] = make_uint4(0u, 0u, 0u, 0u);
+    uint4* m4 = reinterpret_cast<uint4*>(s_mark) + (ITEMS / 4) * threadIdx.x;
+#pragma unroll
+    for (int r = 0; r < ITEMS / 4; ++r)  // before the cluster barrier that precedes any marking
+      m4[r] = make_uint4(0u, 0u, 0u, 0u);
   }
   uint32_t u = 0;
   if (!a.u_arr)
@@ -2094,7 +2190,7 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? 2 : 8) k_resample(const __gr
     for (int sub = lo; sub < hi; sub += SUB) {
       if (!single) load_sub(sub);
 #pragma unroll
-      for (int r = 0; r < RS_ITEMS; ++r) m = fmaxf(m, v[r]);
+      for (int r = 0; r < ITEMS; ++r) m = fmaxf(m, v[r]);
     }
     m = block_max<NTR>(m, s_f);
     if (threadIdx.x == 0) s_pub_max = m;
@@ -2105,11 +2201,13 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? 2 : 8) k_resample(const __gr
   // this CTA's total weight code, then the cluster prefix and group total;
   // under Alg. 1's test also the sums of c = q >> 20 and c^2
   unsigned long long qs = 0, e1 = 0, e2 = 0;
-  unsigned long long qv[RS_ITEMS] = {0, 0, 0, 0, 0, 0, 0, 0};  // 0 on a CTA past the group's end
+  unsigned long long qv[ITEMS];
+#pragma unroll
+  for (int r = 0; r < ITEMS; ++r) qv[r] = 0;  // 0 on a CTA past the group's end
   for (int sub = lo; sub < hi; sub += SUB) {
     if (!single) load_sub(sub);
 #pragma unroll
-    for (int r = 0; r < RS_ITEMS; ++r) {
+    for (int r = 0; r < ITEMS; ++r) {
       qv[r] = quantize(v[r], M, a.qc);
       qs += qv[r];
       if (ess_rule) {
@@ -2140,12 +2238,13 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? 2 : 8) k_resample(const __gr
     }
     pre_cta = wpre + (x - qs);
     qs = tot;
+    if (ess_rule) __syncthreads();  // s_w is free again
   } else {
     qs = block_sum_u64<NTR>(qs, s_w);
-    if (ess_rule) {
-      e1 = block_sum_u64<NTR>(e1, s_w);
-      e2 = block_sum_u64<NTR>(e2, s_w);
-    }
+  }
+  if (ess_rule) {
+    e1 = block_sum_u64<NTR>(e1, s_w);
+    e2 = block_sum_u64<NTR>(e2, s_w);
   }
   if (threadIdx.x == 0) {
     s_pub_q = qs;
@@ -2245,29 +2344,9 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? 2 : 8) k_resample(const __gr
     // no finite weight, or Alg. 1's test keeps the particles: identity
     for (int i = lo + threadIdx.x; i < hi; i += NTR) {
       anc[i] = (uint32_t)(obase + i);
-      if (!LEAN && a.q_out) a.q_out[d.base + i] = 0ull;
+      if (EXTRA && a.q_out) a.q_out[d.base + i] = 0ull;
     }
   } else {
-    // the threshold constants, with the track's precomputed reciprocal of Np
-    // when it has one: every thread's own (LEAN), else one thread's for the
-    // CTA
-    Thresholds th;
-    if constexpr (LEAN) {
-      if (Pt)
-        th.init_magic(Q, (uint32_t)Np, u, Pt->m_Np);
-      else
-        th.init(Q, (uint32_t)Np, u);
-    } else {
-      if (threadIdx.x == 0) {
-        if (a.glob.trk)
-          s_th.init_magic(Q, (uint32_t)Np, u, a.glob.trk[d.track].m_Np);
-        else
-          s_th.init(Q, (uint32_t)Np, u);
-      }
-      __syncthreads();
-      th = s_th;
-    }
-    const float inv_Q = 1.0f / u64_to_float_approx(Q);
     if constexpr (LEAN) {
       // Alg. 3 step 7 by marking: item i takes the outputs O_i .. O_{i+1} - 1,
       // O_i = #{j : T_j < S_i} with S_i the sum of the codes before it.  An
@@ -2277,20 +2356,27 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? 2 : 8) k_resample(const __gr
       // the cluster like items).  A running maximum over each CTA's
       // positions then gives every output its item, with the same work for
       // every CTA however the weight is spread.
-      const int i0 = (int)threadIdx.x * RS_ITEMS;
+      const int i0 = rank * chunk - a0 + (int)threadIdx.x * ITEMS;  // the thread's first item
       unsigned long long S = Sb + pre_cta;  // codes before the thread's first item
       const uint32_t mark_addr = (uint32_t)__cvta_generic_to_shared(s_mark);
 #ifdef PF_DEBUG
-      PF_DBG_INDEX(a.ds, chunk - 1, NTR * RS_ITEMS, 203u);  // the CTA's outputs fit its mark array
+      PF_DBG_INDEX(a.ds, chunk - 1, NTR * ITEMS, 203u);  // the CTA's outputs fit its mark array
 #endif
-      int c = count_below(th, S, inv_Q, Np, u, a.ds);
+      FastCount fc;
+      fc.init(Q, (uint32_t)Np, u);
+      if (EXTRA && a.q_out)
 #pragma unroll
-      for (int r = 0; r < RS_ITEMS; ++r) {
+        for (int r = 0; r < ITEMS; ++r)
+          if (i0 + r >= lo && i0 + r < hi) a.q_out[d.base + i0 + r] = qv[r];
+      const int b0 = off16(anc);  // outputs in units of the ancestors' 16-byte boundaries
+      int c = count_fast(fc, S, Q, (uint32_t)Np, u) + b0;
+#pragma unroll
+      for (int r = 0; r < ITEMS; ++r) {
         if (qv[r] == 0ull) continue;
         S += qv[r];
-        const int c1 = count_below(th, S, inv_Q, Np, u, a.ds);
+        const int c1 = count_fast(fc, S, Q, (uint32_t)Np, u) + b0;
         if (c1 > c) {
-          const uint32_t item = (uint32_t)(lo + i0 + r) + 1u;
+          const uint32_t item = (uint32_t)(i0 + r) + 1u;
           int own = 0;  // c / chunk (C is at most 16)
           for (int b = 1; b < C; ++b) own += c >= b * chunk ? 1 : 0;
           int pos = c - own * chunk;
@@ -2304,23 +2390,34 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? 2 : 8) k_resample(const __gr
         c = c1;
       }
     } else {
+    // the threshold constants, with the track's precomputed reciprocal of Np
+    // when it has one, by one thread for the CTA
+    if (threadIdx.x == 0) {
+      if (a.glob.trk)
+        s_th.init_magic(Q, (uint32_t)Np, u, a.glob.trk[d.track].m_Np);
+      else
+        s_th.init(Q, (uint32_t)Np, u);
+    }
+    __syncthreads();
+    const Thresholds th = s_th;
+    const float inv_Q = 1.0f / u64_to_float_approx(Q);
     unsigned long long carry = Sb;
     for (int sub = lo; sub < hi; sub += SUB) {
       const int n = min(SUB, hi - sub);
-      const int i0 = (int)threadIdx.x * RS_ITEMS;  // first item of this thread (sub-chunk relative)
+      const int i0 = (int)threadIdx.x * ITEMS;  // first item of this thread (sub-chunk relative)
       if (!single) {
         load_sub(sub);
 #pragma unroll
-        for (int r = 0; r < RS_ITEMS; ++r) qv[r] = quantize(v[r], M, a.qc);
+        for (int r = 0; r < ITEMS; ++r) qv[r] = quantize(v[r], M, a.qc);
       }
-      if (!LEAN && a.q_out)
+      if (a.q_out)
 #pragma unroll
-        for (int r = 0; r < RS_ITEMS; ++r)
+        for (int r = 0; r < ITEMS; ++r)
           if (i0 + r < n) a.q_out[d.base + sub + i0 + r] = qv[r];
       // exclusive scan of the thread totals: warp shuffles, then warps
       unsigned long long tsum = 0;
 #pragma unroll
-      for (int r = 0; r < RS_ITEMS; ++r) tsum += qv[r];
+      for (int r = 0; r < ITEMS; ++r) tsum += qv[r];
       unsigned long long x = tsum;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -2340,7 +2437,7 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? 2 : 8) k_resample(const __gr
       {
         unsigned long long S = carry + wpre + (x - tsum);
 #pragma unroll
-        for (int r = 0; r < RS_ITEMS; ++r) {
+        for (int r = 0; r < ITEMS; ++r) {
           S += qv[r];
           s_incl[pad8(i0 + r)] = S;
         }
@@ -2360,16 +2457,18 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? 2 : 8) k_resample(const __gr
   if constexpr (LEAN) {
     cl.sync();  // every mark has landed, and the reads of s_pub_q are done
     if (Q != 0 && resample) {
-      // running maximum over this CTA's positions p0 + 0 .. n_out - 1 (its
-      // first position always holds a mark)
-      const int p0 = rank * chunk, n_out = min(chunk, Np - p0);
-      const int i0 = (int)threadIdx.x * RS_ITEMS;
-      const uint4 m0 = reinterpret_cast<const uint4*>(s_mark)[2 * threadIdx.x];
-      const uint4 m1 = reinterpret_cast<const uint4*>(s_mark)[2 * threadIdx.x + 1];
-      uint32_t m[RS_ITEMS] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
+      // running maximum over this CTA's positions (the first one that holds
+      // an output of the group always holds a mark)
+      const int j0 = rank * chunk - off16(anc) + (int)threadIdx.x * ITEMS;  // the thread's first output
+      uint32_t m[ITEMS];
 #pragma unroll
-      for (int r = 1; r < RS_ITEMS; ++r) m[r] = max(m[r], m[r - 1]);
-      uint32_t x = m[RS_ITEMS - 1];
+      for (int r = 0; r < ITEMS; r += 4) {
+        const uint4 q = reinterpret_cast<const uint4*>(s_mark)[(ITEMS / 4) * threadIdx.x + r / 4];
+        m[r] = q.x; m[r + 1] = q.y; m[r + 2] = q.z; m[r + 3] = q.w;
+      }
+#pragma unroll
+      for (int r = 1; r < ITEMS; ++r) m[r] = max(m[r], m[r - 1]);
+      uint32_t x = m[ITEMS - 1];
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const uint32_t t = __shfl_up_sync(0xffffffffu, x, o);
@@ -2382,19 +2481,12 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? 2 : 8) k_resample(const __gr
 #pragma unroll
       for (int w = 0; w < NTR / 32; ++w)
         if (w < warp) pre = max(pre, (uint32_t)s_w[w]);
-      if (i0 < n_out && max(pre, m[0]) == 0u) set_error(a.ds, ERR_INVARIANT, 12u, (uint32_t)grp, (uint32_t)(p0 + i0));
-      uint32_t o[RS_ITEMS];
+      const int jhi = min((rank + 1) * chunk - off16(anc), Np);
+      if (j0 >= 0 && j0 < jhi && max(pre, m[0]) == 0u) set_error(a.ds, ERR_INVARIANT, 12u, (uint32_t)grp, (uint32_t)j0);
+      uint32_t o[ITEMS];
 #pragma unroll
-      for (int r = 0; r < RS_ITEMS; ++r) o[r] = (uint32_t)(obase + max(max(m[r], pre), 1u) - 1u);
-      uint32_t* out = anc + p0 + i0;
-      if (i0 + RS_ITEMS <= n_out && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
-        reinterpret_cast<uint4*>(out)[0] = make_uint4(o[0], o[1], o[2], o[3]);
-        reinterpret_cast<uint4*>(out)[1] = make_uint4(o[4], o[5], o[6], o[7]);
-      } else {
-#pragma unroll
-        for (int r = 0; r < RS_ITEMS; ++r)
-          if (i0 + r < n_out) out[r] = o[r];
-      }
+      for (int r = 0; r < ITEMS; ++r) o[r] = (uint32_t)(obase + max(max(m[r], pre), 1u) - 1u);
+      store_items<ITEMS>(anc, j0, 0, jhi, o);
     }
   }
 
@@ -2404,6 +2496,301 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? 2 : 8) k_resample(const __gr
 }
 
 
+
+// ======================================================= resample, one CTA per group
+// A batch holds thousands of groups of very different sizes, so there is no
+// need of a cluster per group: TEAM threads (one CTA, or for the smallest
+// groups one warp of a CTA of TEAMS) resample a whole group, in sub-chunks of
+// TEAM x RS_ITEMS items.  A group of one sub-chunk keeps its codes in
+// registers; a larger one is read twice (the total first).  Outputs are found
+// as in the lean cluster kernel, by marking each item's first output and a
+// running maximum, over windows of as many outputs as the sub-chunk has items.
+// Groups come largest first, one launch per class of size.  The class
+// launches overlap: every CTA of a class passes its dependency before it lets
+// the next class start, so a later class finds the propagate kernel complete
+// at its start and waits for the class before it only at its end (which keeps
+// the chain of completions for the kernels after it); its reads of what the
+// propagate kernel wrote go through L2.
+template <int TEAM, int TEAMS>
+__global__ void __launch_bounds__(TEAM* TEAMS, 1024 / (TEAM * TEAMS))
+    k_resample_groups(const __grid_constant__ ResampleArgs a) {
+  constexpr int ITEMS = RS_ITEMS, CAP = TEAM * ITEMS, NW = TEAM / 32;
+  constexpr size_t MARKS = sizeof(uint32_t) * CAP * TEAMS;
+  __shared__ __align__(16) unsigned char s_buf[MARKS > sizeof(GlobalScratch) ? MARKS : sizeof(GlobalScratch)];
+  __shared__ unsigned long long s_w[2][NW];
+  __shared__ uint32_t s_m[NW];
+  __shared__ float s_f[NW];
+  __shared__ float s_stat[NW][8];
+  __shared__ uint32_t s_u;
+  __shared__ int s_last[TEAMS];
+  const int team = (int)threadIdx.x / TEAM, tid = (int)threadIdx.x % TEAM;
+  const int lane = threadIdx.x & 31, warp = tid >> 5;
+  uint32_t* s_mark = reinterpret_cast<uint32_t*>(s_buf) + team * CAP;
+  auto sync = [] {
+    if constexpr (TEAM == 32)
+      __syncwarp();
+    else
+      __syncthreads();
+  };
+  int par = 0;  // s_w's buffer: one barrier per sum, the next sum writes the other
+  auto scan = [&](unsigned long long x, unsigned long long& excl, unsigned long long& tot) {
+    const unsigned long long own = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long t = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += t;
+    }
+    excl = x - own;
+    if constexpr (TEAM == 32) {
+      tot = __shfl_sync(0xffffffffu, x, 31);
+    } else {
+      if (lane == 31) s_w[par][warp] = x;
+      sync();
+      tot = 0;
+#pragma unroll
+      for (int w = 0; w < NW; ++w) {
+        const unsigned long long y = s_w[par][w];
+        if (w < warp) excl += y;
+        tot += y;
+      }
+      par ^= 1;
+    }
+  };
+
+  if (!a.wait_last) grid_dep_wait();
+  grid_dep_launch();
+  if (a.tile_ctr && blockIdx.x == 0 && threadIdx.x == 0) *a.tile_ctr = 0;  // for the next propagate launch
+  const int gi = (int)blockIdx.x * TEAMS + team;
+  // a failed propagate launch left weights that mean nothing: resample nothing
+  const bool failed =
+      (*reinterpret_cast<volatile const unsigned int*>(&a.ds->err) & (ERR_TIMEOUT | ERR_INDEX)) != 0u;
+  int last_track = -1;
+  if (gi < a.n_groups && !failed) {
+    const int grp = a.list ? a.list[gi] : gi;
+    const GroupDesc d = a.gd[grp];
+    const int Np = d.Np;
+    const TrackParams* __restrict__ Pt = a.glob.trk ? a.glob.trk + d.track : nullptr;
+    const int kk = a.u_arr ? 0 : __ldcg(&a.glob.ts[d.track].k);
+    const float* __restrict__ lw = ((a.lw1 && (kk & 1)) ? a.lw1 : a.lw) + d.base;
+    uint32_t* __restrict__ anc = a.anc + (kk & 1) * a.anc_stride + d.base;
+    const bool ess_rule = Pt && Pt->resample_rule == 1;
+    const int a0 = off16(lw), b0 = off16(anc);
+    const int n_sub = (Np + a0 + CAP - 1) / CAP;
+    auto item0 = [&](int sub) { return sub * CAP - a0 + tid * ITEMS; };  // the thread's first item
+#pragma unroll
+    for (int r = 0; r < ITEMS; r += 4) reinterpret_cast<uint4*>(s_mark)[(ITEMS / 4) * tid + r / 4] = make_uint4(0u, 0u, 0u, 0u);
+
+    float v[ITEMS];
+    unsigned long long qv[ITEMS];
+    load_items<ITEMS>(lw, item0(0), 0, Np, v);
+    uint32_t u = 0;
+    if (warp == 0) {
+      u = a.u_arr ? a.u_arr[grp]
+                  : philox(Pt->key0, Pt->key1, make_uint4((uint32_t)d.g, 0u, (uint32_t)kk, Pt->tag | (ST_RESAMPLE << 4))).x;
+      if (TEAM > 32 && tid == 0) s_u = u;
+    }
+    float M = -INFINITY;
+    if (a.tile_part != nullptr) {
+      const uint32_t mk = __ldcg(&a.gs[grp].mkey[kk & 1]);
+      M = mk == 0u ? -INFINITY : key_float((int)(mk ^ 0x80000000u));
+      if (tid == 0) a.gs[grp].mkey[(kk + 1) & 1] = 0u;  // for the next step's tiles
+    } else {
+      float m = -INFINITY;
+      for (int sub = 0; sub < n_sub; ++sub) {
+        if (sub > 0) load_items<ITEMS>(lw, item0(sub), 0, Np, v);
+#pragma unroll
+        for (int r = 0; r < ITEMS; ++r) m = fmaxf(m, v[r]);
+      }
+      M = warp_max(m);
+      if constexpr (TEAM > 32) {
+        if (lane == 0) s_f[warp] = M;
+        sync();
+#pragma unroll
+        for (int w = 0; w < NW; ++w) M = fmaxf(M, s_f[w]);
+      }
+      if (n_sub > 1) load_items<ITEMS>(lw, item0(0), 0, Np, v);
+    }
+
+    // codes and the group's total; under Alg. 1's test also the sums of
+    // c = q >> 20 and c^2
+    unsigned long long tsum = 0, e1 = 0, e2 = 0, excl, Q;
+    for (int sub = 0; sub < n_sub; ++sub) {
+      if (sub > 0) load_items<ITEMS>(lw, item0(sub), 0, Np, v);
+#pragma unroll
+      for (int r = 0; r < ITEMS; ++r) {
+        qv[r] = quantize(v[r], M, a.qc);
+        tsum += qv[r];
+      }
+      if (ess_rule)
+#pragma unroll
+        for (int r = 0; r < ITEMS; ++r) {
+          const unsigned long long c = qv[r] >> 20;
+          e1 += c;
+          e2 += c * c;
+        }
+    }
+    scan(tsum, excl, Q);
+    if constexpr (TEAM > 32) u = s_u;
+    bool resample = true;
+    if (ess_rule) {
+      unsigned long long x, E1, E2;
+      scan(e1, x, E1);
+      scan(e2, x, E2);
+      resample = Q == 0 || ess_below(E1, E2, (uint32_t)Np, Pt->ess_t);
+    }
+
+    if (a.tile_part != nullptr) {
+      // group estimate and ESS from the propagate tiles' partial sums, each
+      // tile's sums rescaled from its own maximum to the group maximum
+      GroupState& G = a.gs[grp];
+      float acc[7] = {0, 0, 0, 0, 0, 0, 0};
+      if (Q != 0) {
+        for (int t = tid; t < d.tile_count; t += TEAM) {
+          const float4* tp = reinterpret_cast<const float4*>(a.tile_part + (long long)(d.tile_begin + t) * 8);
+          const float4 x = __ldcg(tp), y = __ldcg(tp + 1);
+          if (!(x.x - M >= -87.0f)) continue;
+          const float sc = __expf(x.x - M);
+          acc[0] = fmaf(sc, x.y, acc[0]);
+          acc[1] = fmaf(sc, x.z, acc[1]);
+          acc[2] = fmaf(sc, x.w, acc[2]);
+          acc[3] = fmaf(sc, y.x, acc[3]);
+          acc[4] = fmaf(sc, y.y, acc[4]);
+          acc[5] = fmaf(sc, y.z, acc[5]);
+          acc[6] = fmaf(sc * sc, y.w, acc[6]);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 7; ++q) acc[q] = warp_sum(acc[q]);
+      if constexpr (TEAM > 32) {
+        if (lane == 0)
+#pragma unroll
+          for (int q = 0; q < 7; ++q) s_stat[warp][q] = acc[q];
+        sync();
+      }
+      if (tid == 0) {
+        if constexpr (TEAM > 32) {
+#pragma unroll
+          for (int q = 0; q < 7; ++q) {
+            acc[q] = s_stat[0][q];
+#pragma unroll
+            for (int w = 1; w < NW; ++w) acc[q] += s_stat[w][q];
+          }
+        }
+        const bool ok = (Q != 0) && acc[0] > 0.0f;
+        for (int q = 0; q < 5; ++q) G.xs[q] = ok ? acc[1 + q] / acc[0] : 0.0f;
+        G.ess = ok ? acc[0] * acc[0] / acc[6] : 0.0f;
+        G.M = M;
+        G.Q = Q;
+        G.carry_next = resample ? 0 : 1;
+      }
+    }
+
+    const unsigned long long obase = a.local_idx ? 0ull : (unsigned long long)d.g * (unsigned long long)Np;
+    if (Q == 0 || !resample) {
+      // no finite weight, or Alg. 1's test keeps the particles: identity
+      for (int i = tid; i < Np; i += TEAM) {
+        anc[i] = (uint32_t)(obase + i);
+        if (a.q_out) a.q_out[d.base + i] = 0ull;
+      }
+    } else {
+      FastCount fc;
+      fc.init(Q, (uint32_t)Np, u);
+      unsigned long long carry = 0;
+      int jl = 0;  // outputs of the sub-chunks before this one
+      for (int sub = 0; sub < n_sub; ++sub) {
+        unsigned long long tot = Q;
+        if (n_sub > 1) {
+          load_items<ITEMS>(lw, item0(sub), 0, Np, v);
+          tsum = 0;
+#pragma unroll
+          for (int r = 0; r < ITEMS; ++r) {
+            qv[r] = quantize(v[r], M, a.qc);
+            tsum += qv[r];
+          }
+          scan(tsum, excl, tot);
+        }
+        const int i0 = item0(sub);
+        if (a.q_out)
+#pragma unroll
+          for (int r = 0; r < ITEMS; ++r)
+            if (i0 + r >= 0 && i0 + r < Np) a.q_out[d.base + i0 + r] = qv[r];
+        const int jh = sub + 1 < n_sub ? count_fast(fc, carry + tot, Q, (uint32_t)Np, u) : Np;
+        // windows of CAP outputs from a 16-byte boundary of the ancestors
+        for (int w0 = ((jl + b0) & ~3) - b0; w0 < jh; w0 += CAP) {
+          unsigned long long S = carry + excl;
+          int c = count_fast(fc, S, Q, (uint32_t)Np, u) - w0;
+#pragma unroll
+          for (int r = 0; r < ITEMS; ++r) {
+            S += qv[r];
+            const int c1 = count_fast(fc, S, Q, (uint32_t)Np, u) - w0;
+            if (c1 > c && c1 > 0 && c < CAP) {
+              int pos = c > 0 ? c : 0;
+#ifdef PF_DEBUG
+              pos = (int)PF_DBG_INDEX(a.ds, pos, CAP, 204u);
+#endif
+              s_mark[pos] = (uint32_t)(i0 + r) + 1u;
+            }
+            c = c1;
+          }
+          sync();
+          uint32_t m[ITEMS];
+#pragma unroll
+          for (int r = 0; r < ITEMS; r += 4) {
+            uint4& q = reinterpret_cast<uint4*>(s_mark)[(ITEMS / 4) * tid + r / 4];
+            m[r] = q.x; m[r + 1] = q.y; m[r + 2] = q.z; m[r + 3] = q.w;
+            q = make_uint4(0u, 0u, 0u, 0u);  // for the next window
+          }
+#pragma unroll
+          for (int r = 1; r < ITEMS; ++r) m[r] = max(m[r], m[r - 1]);
+          uint32_t x = m[ITEMS - 1];
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x = max(x, t);
+          }
+          uint32_t pre = __shfl_up_sync(0xffffffffu, x, 1);
+          if (lane == 0) pre = 0u;
+          if constexpr (TEAM > 32) {
+            if (lane == 31) s_m[warp] = x;
+            sync();
+#pragma unroll
+            for (int w = 0; w < NW; ++w)
+              if (w < warp) pre = max(pre, s_m[w]);
+          } else {
+            sync();  // the zeroed marks before the next window's
+          }
+          const int j0 = w0 + tid * ITEMS;
+          if (j0 >= jl && j0 < jh && max(pre, m[0]) == 0u) set_error(a.ds, ERR_INVARIANT, 13u, (uint32_t)grp, (uint32_t)j0);
+          uint32_t o[ITEMS];
+#pragma unroll
+          for (int r = 0; r < ITEMS; ++r) o[r] = (uint32_t)(obase + max(max(m[r], pre), 1u) - 1u);
+          store_items<ITEMS>(anc, j0, jl, jh, o);
+        }
+        carry += tot;
+        jl = jh;
+      }
+    }
+    // the group has reported: the last of its track runs the global step
+    if (a.fuse_global && tid == 0) {
+      __threadfence();
+      const unsigned prev = atomicAdd(&a.glob.ts[d.track].ticket, 1u);
+      if (prev + 1u == (unsigned)Pt->G) last_track = d.track;
+      __threadfence();
+    }
+  }
+  if (a.fuse_global) {
+    if (tid == 0) s_last[team] = last_track;
+    __syncthreads();  // (the marks are free for the scratch)
+    for (int t = 0; t < TEAMS; ++t) {
+      const int track = s_last[t];
+      if (track < 0) continue;
+      global_step_call<TEAM * TEAMS>(a.glob, track, *reinterpret_cast<GlobalScratch*>(s_buf));
+      if (threadIdx.x == 0) a.glob.ts[track].ticket = 0u;
+      __syncthreads();
+    }
+  }
+  if (a.wait_last) grid_dep_wait();
+}
 
 // ============================================================ export helpers
 __global__ void k_export_states(const float4* __restrict__ pv, const float* __restrict__ In, long long n,
@@ -2552,30 +2939,63 @@ cudaError_t launch_propagate(const K1Args& a, int R, int grid, bool pdl, cudaStr
   }
 }
 
-template <int NTR, bool LEAN>
+template <int NTR, int ITEMS, bool LEAN, bool EXTRA>
 static cudaError_t launch_resample_t(const ResampleArgs& a, int n_groups, int cluster, bool pdl, cudaStream_t s) {
-  constexpr size_t smem = LEAN ? RS_MARK_OFF + NTR * RS_ITEMS * sizeof(uint32_t)
+  constexpr size_t smem = LEAN ? RS_MARK_OFF + NTR * ITEMS * sizeof(uint32_t)
                               : pad8(NTR * RS_ITEMS) * sizeof(unsigned long long) +
                                     pad8(2 * NTR * RS_ITEMS) * sizeof(uint32_t);
   static_assert(sizeof(GlobalScratch) <= smem, "the global step's scratch lives in the resampler's shared memory");
   static std::once_flag once;
   static cudaError_t attr_err = cudaSuccess;
   std::call_once(once, [] {
-    attr_err = cudaFuncSetAttribute(k_resample<NTR, LEAN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    attr_err = cudaFuncSetAttribute(k_resample<NTR, ITEMS, LEAN, EXTRA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   });
   if (attr_err != cudaSuccess) return attr_err;
   const int clusters = n_groups + (a.fuse_global == 2 ? 1 : 0);  // the global step's extra cluster
-  return launch_ex(k_resample<NTR, LEAN>, dim3((unsigned)(clusters * cluster)), dim3(NTR), cluster, pdl, s, a, smem);
+  return launch_ex(k_resample<NTR, ITEMS, LEAN, EXTRA>, dim3((unsigned)(clusters * cluster)), dim3(NTR), cluster, pdl, s, a, smem);
 }
 
 cudaError_t launch_resample(const ResampleArgs& a, int n_groups, int cluster, bool pdl, cudaStream_t s, int threads) {
-  const long long chunk = (((long long)a.max_np + cluster - 1) / cluster + 7) / 8 * 8;  // as in k_resample
-  if (a.lean && !a.q_out && chunk <= (long long)threads * RS_ITEMS) {
-    if (threads == RS_THREADS_SMALL) return launch_resample_t<RS_THREADS_SMALL, true>(a, n_groups, cluster, pdl, s);
-    return launch_resample_t<RS_THREADS, true>(a, n_groups, cluster, pdl, s);
+  // the lean instances while every CTA's chunk fits their registers: 8 items
+  // per thread, 16 for the largest groups (65536 particles on a cluster of 8)
+  const long long chunk = rs_chunk_lean(a.max_np, cluster, a.pad);
+  const bool small = threads == RS_THREADS_SMALL, extra = !a.lean || a.q_out;
+  if (chunk <= (long long)threads * RS_ITEMS) {
+    if (small)
+      return extra ? launch_resample_t<RS_THREADS_SMALL, RS_ITEMS, true, true>(a, n_groups, cluster, pdl, s)
+                   : launch_resample_t<RS_THREADS_SMALL, RS_ITEMS, true, false>(a, n_groups, cluster, pdl, s);
+    return extra ? launch_resample_t<RS_THREADS, RS_ITEMS, true, true>(a, n_groups, cluster, pdl, s)
+                 : launch_resample_t<RS_THREADS, RS_ITEMS, true, false>(a, n_groups, cluster, pdl, s);
   }
-  if (threads == RS_THREADS_SMALL) return launch_resample_t<RS_THREADS_SMALL, false>(a, n_groups, cluster, pdl, s);
-  return launch_resample_t<RS_THREADS, false>(a, n_groups, cluster, pdl, s);
+  if (!small && !extra && chunk <= (long long)RS_THREADS * 2 * RS_ITEMS)
+    return launch_resample_t<RS_THREADS, 2 * RS_ITEMS, true, false>(a, n_groups, cluster, pdl, s);
+  if (small) return launch_resample_t<RS_THREADS_SMALL, RS_ITEMS, false, true>(a, n_groups, cluster, pdl, s);
+  return launch_resample_t<RS_THREADS, RS_ITEMS, false, true>(a, n_groups, cluster, pdl, s);
+}
+
+template <int C>
+static cudaError_t launch_groups_t(const ResampleArgs& a, bool pdl, cudaStream_t s) {
+  return launch_ex(k_resample_groups<RG_THREADS[C], RG_TEAMS[C]>,
+                   dim3((unsigned)((a.n_groups + RG_TEAMS[C] - 1) / RG_TEAMS[C])), dim3(RG_THREADS[C] * RG_TEAMS[C]), 0,
+                   pdl, s, a);
+}
+
+cudaError_t launch_resample_groups(const ResampleArgs& a0, const GroupClasses& gc, bool pdl, cudaStream_t s) {
+  ResampleArgs a = a0;
+  bool first = true;
+  for (int c = 0; c < 3; ++c) {
+    a.n_groups = gc.begin[c + 1] - gc.begin[c];
+    if (a.n_groups == 0) continue;
+    a.list = gc.list + gc.begin[c];
+    a.wait_last = first ? 0 : 1;
+    const cudaError_t e = c == 0   ? launch_groups_t<0>(a, pdl, s)
+                          : c == 1 ? launch_groups_t<1>(a, pdl, s)
+                                   : launch_groups_t<2>(a, pdl, s);
+    if (e != cudaSuccess) return e;
+    a.tile_ctr = nullptr;
+    first = false;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_global(const GlobalArgs& a, int n_tracks, cudaStream_t s) {

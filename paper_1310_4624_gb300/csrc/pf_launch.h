@@ -133,6 +133,7 @@ struct GlobalArgs {
   int finalize;  // 0: prepare step 0 only
   DevState* ds;
   int keep_k;    // 1: leave the step index to the caller (fused step: advanced when its launch ends)
+  int sum_nt;    // 0, or the CTA size whose order of summation the carried weights' sum follows
 };
 
 struct ResampleArgs {
@@ -152,12 +153,22 @@ struct ResampleArgs {
                                // 2 (one track): an extra cluster after the groups' runs it instead,
                                // once every group has reported, so no group's merge waits behind it
   int n_groups;                // groups of the launch (the extra cluster, if any, comes after them)
-  int lean;                    // 1: no group under Alg. 1's test and no codes stored (a filter step, or
-                               // pf_resample without codes): the lean instance runs if every CTA's chunk
-                               // also fits its registers
+  int lean;                    // 1: no group under Alg. 1's test
   int max_np;                  // the largest group of the launch (for that test)
+  int pad;                     // 0: every group starts on 16 bytes of the log-weights and the ancestors, else 3
   int* tile_ctr;               // propagate kernel's tile counter to reset, or nullptr
   GlobalArgs glob;             // (fuse_global) arguments of that step, finalize = 1
+  // one-CTA resampler (launch_resample_groups): the groups of this launch
+  const int* list;             // global group indices, or nullptr (0 .. n_groups - 1)
+  int wait_last;               // 1: a launch behind another class of the same step, which waits for that one
+                               // at its end instead of its start
+};
+
+// The groups of a batch by class of size (RG_THREADS): list[begin[c] ..
+// begin[c + 1]) are those of class c, the largest first.
+struct GroupClasses {
+  const int* list;             // device
+  int begin[4];
 };
 
 // pf_backward (pf_adjoint.cu)
@@ -241,6 +252,9 @@ cudaError_t fused_occupancy(int R, int* blocks_per_sm);
 // threads: RS_THREADS, or RS_THREADS_SMALL (eight CTAs per SM, for batches of small groups)
 cudaError_t launch_resample(const ResampleArgs& a, int n_groups, int cluster, bool pdl, cudaStream_t s,
                             int threads = RS_THREADS);
+// The resampling of many groups, one CTA (or one warp) per group, a launch
+// per class of group size.
+cudaError_t launch_resample_groups(const ResampleArgs& a, const GroupClasses& gc, bool pdl, cudaStream_t s);
 cudaError_t launch_global(const GlobalArgs& a, int n_tracks, cudaStream_t s);
 cudaError_t launch_finish(const GlobalArgs& a, int n_tracks, cudaStream_t s);
 // launch_finish, then x^ (n_tracks x 5) and log Z (n_tracks) stored through
@@ -254,7 +268,9 @@ const void* propagate_kernel(int R);
 
 // Host helpers shared by the C-ABI entry points (defined in pf_api.cu).
 QuantCoeffs resample_coeffs();             // weight-code coefficients
-int resample_cluster_size(int Np);         // resampler cluster size for one group of Np
+int resample_cluster_size(int Np, int pad);  // resampler cluster size for one group of Np
+// ResampleArgs::pad for G groups of Np in a caller's arrays
+int resample_pad(const float* logw, const uint32_t* anc, int G, int Np);
 void set_handleless_error(const char* msg);  // text for pf_last_error(NULL)
 // The no-allocation resampler's error word on the current device (defined
 // in pf_noalloc.cu); PF_OK and *out set, or an error status.
