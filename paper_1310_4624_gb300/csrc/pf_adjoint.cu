@@ -16,14 +16,16 @@
 // (the softmax terms of lbar cancel because sum_m dL_k,m = s at every k);
 // states back-propagate through the NCV Jacobian to their recorded parents.
 // The forward pass is replayed from the initial population and the recorded
-// parents with the same Philox streams; states are recomputed from
-// checkpoints, not stored per step.
+// parents with the same Philox streams; the replay leaves the log-weights and
+// the likelihood's derivatives of each step (24 bytes a particle), which is
+// all that the reverse sweep needs of it.  Where those of every step would
+// take more than ADJ_STORE_MAX, they are kept for a segment at a time and
+// replayed from checkpoints of the states.
 #include <cuda_runtime.h>
 
 #include <climits>
 #include <cmath>
 #include <cstdint>
-#include <type_traits>
 
 #include "pf_device.cuh"
 #include "pf_launch.h"
@@ -31,107 +33,346 @@
 
 namespace pf {
 
-// ------------------------------------------------------------------ replay
-// Replay of step k for every slot: the state (k >= 1: NCV from the recorded
-// parent and the step's normals) and, when weights != 0, the log-weight and
-// its per-tile (max, sum exp) for the group log-weights.
-template <int R>
-__global__ void __launch_bounds__(256) k_replay(ReplayArgs a) {
-  constexpr int PAD = 2 * R + 1;
-  const int k = a.k;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  __shared__ float s_m[8], s_s[8];
-  for (int tile = blockIdx.x; tile < a.n_tiles; tile += gridDim.x) {
-    const int4 td = a.tiles[tile];
-    const TrackParams& P = a.trk[td.x];
-    const int g = td.y, Np = P.Np;
-    const long long Nt = (long long)P.G * Np;
-    const int hslot = k % a.history;
-    const float log_G = logf((float)P.G), log_Np = logf((float)Np);
-    float mx = -INFINITY, sm = 0.0f;
-    for (int jj = threadIdx.x; jj < td.w; jj += blockDim.x) {
-      const int j = td.z + jj;
-      const long long il = (long long)g * Np + j, i = P.part_off + il;
-      float4 s;
-      float I;
-      int o = g;
-      if (k >= 1) {
-        const long long par = a.parent[P.parent_off + (long long)hslot * Nt + il];
-        o = (int)fastdiv((uint32_t)par, P.m_Np);  // origin group (par < 2^31)
-        s = a.pv_in[P.part_off + par];
-        I = a.I_in[P.part_off + par];
-        uint4 w0 = make_uint4(j, g, k, P.tag | (ST_PROP << 4) | 0u);
-        uint4 w1 = make_uint4(j, g, k, P.tag | (ST_PROP << 4) | 1u);
-        philox2(P.key0, P.key1, w0, w1);
-        float e0, e1, e2, e3, e4, e5;
-        box_muller_fast(w0.x, w0.y, e0, e1);
-        box_muller_fast(w0.z, w0.w, e2, e3);
-        box_muller_fast(w1.x, w1.y, e4, e5);
-        s.x = fmaf(P.spos, e0, s.x + s.z);
-        s.y = fmaf(P.spos, e1, s.y + s.w);
-        s.z = fmaf(P.sv, e2, s.z);
-        s.w = fmaf(P.sv, e3, s.w);
-        I = fmaf(P.sI, e4, I);
-        a.pv_out[i] = s;
-        a.I_out[i] = I;
-      } else {
-        s = a.pv_out[i];
-        I = a.I_out[i];
-      }
-      if (a.ck_pv) {
-        a.ck_pv[i] = s;
-        a.ck_I[i] = I;
-      }
-      if (a.weights) {
-        float gxI[2 * R + 1];
-        const float cxf = floorf(s.x + 0.5f), cyf = floorf(s.y + 0.5f);
-        gauss_row<R>(cxf, s.x, P.c_psf, P.kappa, gxI);
+constexpr int RG_GROUP_THREADS = 1024;
+
+// --------------------------------------------- likelihood and its derivatives
+// Where a tile's pixels come from: the caller's frame (raw: y = z - bg inside,
+// 0 outside) or the track's padded frame (bg = 0, every access inside).
+// Patch coordinates are those of the padded frame; sub converts them.
+struct PixelSource {
+  const float* z;
+  int w, h, sub;
+  float bg;
+  __device__ __forceinline__ float at(int u, int v) const {
+    const int x = u - sub, y = v - sub;
+    return ((unsigned)x < (unsigned)w && (unsigned)y < (unsigned)h) ? __fsub_rn(__ldg(z + (long long)y * w + x), bg)
+                                                                    : 0.0f;
+  }
+};
+
+// Two neighbouring pixels of a patch row: from the staged box (8-byte aligned
+// pairs) or from the frame.
+struct StagedRows {
+  const float* base;
+  __device__ __forceinline__ float2 pair(int b, int p) const {
+    return *reinterpret_cast<const float2*>(base + b * ROI_W + 2 * p);
+  }
+  __device__ __forceinline__ float one(int b, int a) const { return base[b * ROI_W + a]; }
+};
+struct FrameRows {
+  const PixelSource& px;
+  int u, v;
+  __device__ __forceinline__ float2 pair(int b, int p) const {
+    return make_float2(px.at(u + 2 * p, v + b), px.at(u + 2 * p + 1, v + b));
+  }
+  __device__ __forceinline__ float one(int b, int a) const { return px.at(u + a, v + b); }
+};
+
+// Log-likelihood (Sec. V model) and its partial derivatives: d[0..4] = dl/dx,
+// dl/dy, dl/dI, dl/dsigma_psf, dl/db.  One pass over the patch, columns 2p and
+// 2p + 1 as one packed FP32 pair.  With r = y - I gx gy per pixel, what the
+// derivatives need of the columns is A_a = sum_b gy_b r_ab (sum r gx gy (u-x)^n
+// = sum_a gx_a (u_a-x)^n A_a, taken once after the rows) and of the rows
+// R_b = sum_a gx_a r_ab, so a pair costs five packed operations (r, r^2, A, R,
+// sum r) where sums by row of r gx, r gx a and r gx a^2 cost eight a pixel.
+// Pixels outside the frame count as background, so only inside pixels depend
+// on b: a patch over the border (rare) sums those in a pass of its own.
+template <int R, bool FRAME, class Rows>
+__device__ __forceinline__ float loglik_grad(const Rows& rows, int H, int W, float x, float y, float I,
+                                             const TrackParams& P, float (&d)[5]) {
+  constexpr int D = 2 * R + 1;
+  const float cxf = floorf(x + 0.5f), cyf = floorf(y + 0.5f);
+  const float cc = P.c_psf, kappa = P.kappa;
+  float gx[D];
+  gauss_row<R>(cxf, x, cc, kappa, gx);
+  float2 A[R];
 #pragma unroll
-        for (int c = 0; c < 2 * R + 1; ++c) gxI[c] *= I;
-        const int pu = (int)fminf(fmaxf(cxf, -(float)(R + 1)), (float)(P.W + R)) - R + PAD;
-        const int pv = (int)fminf(fmaxf(cyf, -(float)(R + 1)), (float)(P.H + R)) - R + PAD;
-        const float* base = a.ypad + P.ypad_off + (long long)pv * P.pitch + pu;
-        const float ss = P.obs_model == 1 ? patch_ss<R, true, false>(base, P.pitch, gxI, cyf - s.y, P.c_psf, P.kappa)
-                                          : patch_ss<R, false, false>(base, P.pitch, gxI, cyf - s.y, P.c_psf, P.kappa);
-        const float lb = k >= 1 ? (float)a.lbar_prev[P.group_off + o] : -log_G;
-        const float lw = lb - log_Np - ss * P.inv2so2;
-        if (lw == lw && lw > -INFINITY) {
-          if (lw > mx) {
-            sm = sm * __expf(mx - lw) + 1.0f;
-            mx = lw;
-          } else {
-            sm += __expf(lw - mx);
-          }
+  for (int p = 0; p < R; ++p) A[p] = make_float2(0.0f, 0.0f);
+  float Al = 0.0f;  // column 2R
+  float2 ss = make_float2(0.0f, 0.0f), Sb = ss, Y2 = ss, Y1 = ss;
+  float Sy = 0.0f, Sy2 = 0.0f;
+  const float dy = cyf - y;
+  auto row = [&](int b, float gy) {
+    const float nI = -(I * gy);
+    const float2 nI2 = make_float2(nI, nI), gy2 = make_float2(gy, gy);
+    float2 R0 = make_float2(0.0f, 0.0f), Rb = R0;
+#pragma unroll
+    for (int p = 0; p < R; ++p) {
+      const float2 yv = rows.pair(b, p), g2 = make_float2(gx[2 * p], gx[2 * p + 1]);
+      const float2 r = __ffma2_rn(g2, nI2, yv);
+      ss = __ffma2_rn(r, r, ss);
+      A[p] = __ffma2_rn(gy2, r, A[p]);
+      R0 = __ffma2_rn(g2, r, R0);
+      Rb = __fadd2_rn(Rb, r);
+      if constexpr (FRAME) {
+        Y2 = __ffma2_rn(yv, yv, Y2);
+        Y1 = __fadd2_rn(Y1, yv);
+      }
+    }
+    const float yl = rows.one(b, 2 * R);
+    const float r = fmaf(gx[2 * R], nI, yl);
+    ss.x = fmaf(r, r, ss.x);
+    Al = fmaf(gy, r, Al);
+    R0.x = fmaf(gx[2 * R], r, R0.x);
+    Rb.x += r;
+    if constexpr (FRAME) {
+      Y2.x = fmaf(yl, yl, Y2.x);
+      Y1.x += yl;
+    }
+    Sb = __fadd2_rn(Sb, Rb);
+    const float dv = (float)(b - R) + dy;
+    const float t = gy * dv * (R0.x + R0.y);
+    Sy += t;
+    Sy2 = fmaf(t, dv, Sy2);
+  };
+  {
+    const float g = ex2(-cc * dy * dy);
+    float up = ex2(-cc * fmaf(2.0f, dy, 1.0f)), dn = ex2(cc * fmaf(2.0f, dy, -1.0f));
+    row(R, g);
+    float gu = g, gd = g;
+#pragma unroll
+    for (int a = 1; a <= R; ++a) {
+      gu *= up;
+      gd *= dn;
+      up *= kappa;
+      dn *= kappa;
+      row(R + a, gu);
+      row(R - a, gd);
+    }
+  }
+  float SI = 0.0f, S1 = 0.0f, S2 = 0.0f;
+  const float dx = cxf - x;
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    const float t = gx[a] * (a == 2 * R ? Al : (a & 1) ? A[a / 2].y : A[a / 2].x);
+    const float du = (float)(a - R) + dx;
+    SI += t;
+    S1 = fmaf(t, du, S1);
+    S2 = fmaf(t * du, du, S2);
+  }
+  float sb = Sb.x + Sb.y;
+  // inside-the-frame column / row ranges of the (true) patch
+  const float ulo = fmaxf(0.0f, (float)R - cxf), uhi = fminf((float)(2 * R), (float)(W - 1) + (float)R - cxf);
+  const float vlo = fmaxf(0.0f, (float)R - cyf), vhi = fminf((float)(2 * R), (float)(H - 1) + (float)R - cyf);
+  if (!(ulo == 0.0f && uhi == (float)(2 * R) && vlo == 0.0f && vhi == (float)(2 * R))) {
+    sb = 0.0f;
+#pragma unroll 1
+    for (int b = 0; b < D; ++b) {
+      if ((float)b < vlo || (float)b > vhi) continue;
+      const float dv = (float)(b - R) + dy;
+      const float nI = -(I * ex2(-cc * dv * dv));
+      float rb = 0.0f;
+#pragma unroll
+      for (int a = 0; a < D; ++a)
+        rb += ((float)a >= ulo && (float)a <= uhi) ? fmaf(gx[a], nI, rows.one(b, a)) : 0.0f;
+      sb += rb;
+    }
+  }
+  const float iso2 = 2.0f * P.inv2so2;  // 1 / sigma_obs^2
+  const float s2 = P.spsf * P.spsf;
+  const float sq = ss.x + ss.y;
+  d[0] = I * S1 / s2 * iso2;
+  d[1] = I * Sy / s2 * iso2;
+  d[2] = SI * iso2;
+  d[3] = I * (S2 + Sy2) / (s2 * P.spsf) * iso2;
+  d[4] = sb * iso2;
+  if constexpr (FRAME) {
+    // frame likelihood ratio: + sum y^2 / (2 sigma_obs^2), whose only
+    // parameter is b (dy/db = -1 inside the frame, y = 0 outside)
+    d[4] -= (Y1.x + Y1.y) * iso2;
+    return -(sq - (Y2.x + Y2.y)) * P.inv2so2;
+  }
+  return -sq * P.inv2so2;
+}
+
+// The same off the staged box, out of line (rare: a tile whose patches do not
+// fit one box), so that its addressing takes no registers of the main path.
+template <int R>
+__device__ __noinline__ float loglik_grad_frame(const PixelSource& px, int u, int v, float4 s, float I,
+                                                const TrackParams& P, float (&d)[5]) {
+  const FrameRows rows{px, u, v};
+  return P.obs_model == 1 ? loglik_grad<R, true>(rows, P.H, P.W, s.x, s.y, I, P, d)
+                          : loglik_grad<R, false>(rows, P.H, P.W, s.x, s.y, I, P, d);
+}
+
+// ------------------------------------------------------------------ replay
+// Replay of step k for every slot: the state (propagate: NCV from the
+// recorded parent and the step's normals; else as given in pv_out), the
+// log-weights' (max, sum exp) per tile for the group log-weights and, where
+// dl_pv is given, the log-weight and the likelihood's derivatives for the
+// reverse sweep, which then never looks at a frame.
+// One CTA per tile; the box of the tile's patches is staged in shared memory
+// twice (the copy shifted by one float makes every patch row a row of aligned
+// pairs), a tile whose patches do not fit reads the frame through L1.  Bound
+// by FP32 issue.  Gradient of log Z, 16 x 65536 particles, 20 frames: 7.45 ms
+// with scalar L1 reads in two passes, 5.51 ms with this one.
+template <int R>
+__global__ void __launch_bounds__(K1_THREADS, 3) k_replay(ReplayArgs a) {
+  constexpr int D = 2 * R + 1, PAD = 2 * R + 1, NW = K1_THREADS / 32;
+  __shared__ __align__(16) float s_roi[2][ROI_FLOATS + 4];
+  __shared__ int s_box[NW][4];
+  __shared__ float s_m[NW], s_s[NW];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int k = a.k, tile = blockIdx.x;
+  grid_dep_wait();
+  grid_dep_launch();
+  const int4 td = a.tiles[tile];
+  const TrackParams& P = a.trk[td.x];
+  const int g = td.y, Np = P.Np;
+  const long long Nt = (long long)P.G * Np;
+  const uint32_t* __restrict__ par_t = a.parent + P.parent_off + (long long)(k % a.history) * Nt;
+  float4 s[K1_PPT];
+  float I[K1_PPT];
+  int o[K1_PPT], pu[K1_PPT], pv[K1_PPT];
+  int umin = INT_MAX, umax = INT_MIN, vmin = INT_MAX, vmax = INT_MIN;
+#pragma unroll
+  for (int q = 0; q < K1_PPT; ++q) {
+    const int jj = threadIdx.x + q * K1_THREADS, j = td.z + jj;
+    const long long il = (long long)g * Np + j, i = P.part_off + il;
+    o[q] = g;
+    if (jj >= td.w) continue;
+    uint32_t par = 0;
+    if (k >= 1) {
+      par = par_t[il];
+      o[q] = (int)fastdiv(par, P.m_Np);  // origin group
+    }
+    if (a.propagate) {
+      s[q] = a.pv_in[P.part_off + par];
+      I[q] = a.I_in[P.part_off + par];
+      uint4 w0 = make_uint4(j, g, k, P.tag | (ST_PROP << 4) | 0u);
+      uint4 w1 = make_uint4(j, g, k, P.tag | (ST_PROP << 4) | 1u);
+      philox2(P.key0, P.key1, w0, w1);
+      float e0, e1, e2, e3, e4, e5;
+      box_muller_fast(w0.x, w0.y, e0, e1);
+      box_muller_fast(w0.z, w0.w, e2, e3);
+      box_muller_fast(w1.x, w1.y, e4, e5);
+      s[q].x = fmaf(P.spos, e0, s[q].x + s[q].z);
+      s[q].y = fmaf(P.spos, e1, s[q].y + s[q].w);
+      s[q].z = fmaf(P.sv, e2, s[q].z);
+      s[q].w = fmaf(P.sv, e3, s[q].w);
+      I[q] = fmaf(P.sI, e4, I[q]);
+      a.pv_out[i] = s[q];
+      a.I_out[i] = I[q];
+    } else {
+      s[q] = a.pv_out[i];
+      I[q] = a.I_out[i];
+    }
+    if (a.ck_pv) {
+      a.ck_pv[i] = s[q];
+      a.ck_I[i] = I[q];
+    }
+    if (a.zero_pv) {
+      a.zero_pv[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      a.zero_I[i] = 0.0f;
+    }
+    pu[q] = (int)fminf(fmaxf(floorf(s[q].x + 0.5f), -(float)(R + 1)), (float)(P.W + R)) - R + PAD;
+    pv[q] = (int)fminf(fmaxf(floorf(s[q].y + 0.5f), -(float)(R + 1)), (float)(P.H + R)) - R + PAD;
+    umin = min(umin, pu[q]);
+    umax = max(umax, pu[q]);
+    vmin = min(vmin, pv[q]);
+    vmax = max(vmax, pv[q]);
+  }
+
+  // the box of the tile's patches, staged as y values
+  const PixelSource px = a.zraw ? PixelSource{a.zraw, P.W, P.H, PAD, P.bg}
+                                : PixelSource{a.ypad + P.ypad_off, P.pitch, P.H + 2 * PAD, 0, 0.0f};
+  umin = __reduce_min_sync(0xffffffffu, umin);
+  umax = __reduce_max_sync(0xffffffffu, umax);
+  vmin = __reduce_min_sync(0xffffffffu, vmin);
+  vmax = __reduce_max_sync(0xffffffffu, vmax);
+  if (lane == 0) {
+    s_box[warp][0] = umin;
+    s_box[warp][1] = umax;
+    s_box[warp][2] = vmin;
+    s_box[warp][3] = vmax;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < NW; ++w) {
+    umin = min(umin, s_box[w][0]);
+    umax = max(umax, s_box[w][1]);
+    vmin = min(vmin, s_box[w][2]);
+    vmax = max(vmax, s_box[w][3]);
+  }
+  const int cols = umax + D - umin, nrows = vmax + D - vmin;
+  const bool staged = cols <= ROI_W && nrows <= ROI_ROWS;
+  if (staged) {
+    // eight threads a row, 32 rows a pass: sector-sized reads
+    const int c0 = threadIdx.x & 7;
+    for (int r = threadIdx.x >> 3; r < nrows; r += K1_THREADS / 8)
+#pragma unroll
+      for (int i = 0; i < ROI_W / 8; ++i) {
+        const int c = c0 + 8 * i;
+        if (c < cols) {
+          const float v = px.at(umin + c, vmin + r);
+          s_roi[0][r * ROI_W + c] = v;
+          if (r * ROI_W + c > 0) s_roi[1][r * ROI_W + c - 1] = v;
         }
       }
+    __syncthreads();
+  }
+
+  const float log_G = logf((float)P.G), log_Np = logf((float)Np);
+  const bool frame_model = P.obs_model == 1;
+  float mx = -INFINITY, sm = 0.0f;
+#pragma unroll
+  for (int q = 0; q < K1_PPT; ++q) {
+    const int jj = threadIdx.x + q * K1_THREADS;
+    if (jj >= td.w) continue;
+    const long long i = P.part_off + (long long)g * Np + td.z + jj;
+    float d[5];
+    float l;
+    if (staged) {
+      const int c = pu[q] - umin, off = (pv[q] - vmin) * ROI_W + c;
+      const StagedRows rows{(c & 1) ? &s_roi[1][off - 1] : &s_roi[0][off]};
+      l = frame_model ? loglik_grad<R, true>(rows, P.H, P.W, s[q].x, s[q].y, I[q], P, d)
+                      : loglik_grad<R, false>(rows, P.H, P.W, s[q].x, s[q].y, I[q], P, d);
+    } else {
+      l = loglik_grad_frame<R>(px, pu[q], pv[q], s[q], I[q], P, d);
     }
-    if (a.weights) {
-      // block (max, sum exp) of the tile
-      float m2 = warp_max(mx);
-      float s2 = (mx > -INFINITY) ? sm * __expf(mx - m2) : 0.0f;
-      s2 = warp_sum(s2);
-      if (lane == 0) {
-        s_m[warp] = m2;
-        s_s[warp] = s2;
-      }
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        float M = -INFINITY;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) M = fmaxf(M, s_m[w]);
-        float S = 0.0f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
-          if (s_m[w] > -INFINITY) S += s_s[w] * __expf(s_m[w] - M);
-        a.tile_part[(long long)tile * 8 + 0] = M;
-        a.tile_part[(long long)tile * 8 + 1] = S;
-      }
-      __syncthreads();
+    const float lb = k >= 1 ? a.lbar_prev[P.group_off + o[q]] : -log_G;
+    const float lw = lb - log_Np + l;
+    if (a.dl_pv) {
+      a.dl_pv[i] = make_float4(d[0], d[1], d[2], d[3]);
+      a.dl_b[i] = d[4];
+      a.dl_lw[i] = lw;
     }
+    if (lw == lw && lw > -INFINITY) {
+      if (lw > mx) {
+        sm = sm * __expf(mx - lw) + 1.0f;
+        mx = lw;
+      } else {
+        sm += __expf(lw - mx);
+      }
+    }
+  }
+  // block (max, sum exp) of the tile
+  const float m2 = warp_max(mx);
+  const float s2 = warp_sum((mx > -INFINITY) ? sm * __expf(mx - m2) : 0.0f);
+  if (lane == 0) {
+    s_m[warp] = m2;
+    s_s[warp] = s2;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float M = -INFINITY;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) M = fmaxf(M, s_m[w]);
+    float S = 0.0f;
+#pragma unroll
+    for (int w = 0; w < NW; ++w)
+      if (s_m[w] > -INFINITY) S += s_s[w] * __expf(s_m[w] - M);
+    *reinterpret_cast<float2*>(&a.tile_part[(long long)tile * 8]) = make_float2(M, S);
   }
 }
 
 // Per track: the replayed group log-weights of step k, log c_k, lbar_k, and
 // at the last step the seed of the reverse sweep, dL = s pi.  FP64 (G-sized).
-__global__ void __launch_bounds__(256) k_replay_groups(ReplayGroupArgs a) {
+// The sweep's accumulators are prepared here: the gradient's copies and the
+// second dL buffer start at zero at step 0, log Z is set there.
+__global__ void __launch_bounds__(RG_GROUP_THREADS) k_replay_groups(ReplayGroupArgs a) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int t = blockIdx.x;
   const TrackParams& P = a.trk[t];
   const int G = P.G;
@@ -144,13 +385,13 @@ __global__ void __launch_bounds__(256) k_replay_groups(ReplayGroupArgs a) {
   for (int m = warp; m < G; m += nw) {
     const int t0 = a.gd[P.group_off + m].tile_begin, nt = a.gd[P.group_off + m].tile_count;
     float M = -INFINITY;
-    for (int q = lane; q < nt; q += 32) M = fmaxf(M, a.tile_part[(long long)(t0 + q) * 8]);
+    for (int q = lane; q < nt; q += 32) M = fmaxf(M, __ldcg(&a.tile_part[(long long)(t0 + q) * 8]));
     M = warp_max(M);
     float S = 0.0f;
     if (M > -INFINITY)
       for (int q = lane; q < nt; q += 32) {
-        const float Mt = a.tile_part[(long long)(t0 + q) * 8];
-        if (Mt > -INFINITY) S = fmaf(a.tile_part[(long long)(t0 + q) * 8 + 1], expf(Mt - M), S);
+        const float2 ms = __ldcg(reinterpret_cast<const float2*>(&a.tile_part[(long long)(t0 + q) * 8]));
+        if (ms.x > -INFINITY) S = fmaf(ms.y, expf(ms.x - M), S);
       }
     S = warp_sum(S);
     if (lane == 0) s_lam[m] = (M > -INFINITY && S > 0.0f) ? (double)M + log((double)S) : -INFINITY;
@@ -173,254 +414,225 @@ __global__ void __launch_bounds__(256) k_replay_groups(ReplayGroupArgs a) {
     double tot = 0.0;
     for (int w = 0; w < nw; ++w) tot += s_d[w];
     s_lc = mx + log(tot);
-    a.logZ[t] += s_lc;
+    a.logZ[t] = (a.k > 0 ? a.logZ[t] : 0.0) + s_lc;
+  }
+  if (a.k == 0) {
+    for (int i = threadIdx.x; i < GRAD_COPIES * 5; i += blockDim.x)
+      a.grad[((long long)(i / 5) * gridDim.x + t) * GRAD_STRIDE + i % 5] = 0.0;
+    for (int m = threadIdx.x; m < G; m += blockDim.x) a.dlam1[P.group_off + m] = 0.0;
   }
   __syncthreads();
   const double lc = s_lc;
   for (int m = threadIdx.x; m < G; m += blockDim.x) {
     const double lam = s_lam[m];
     const long long gm = P.group_off + m;
-    a.lam_hist[(long long)a.k * a.G_total + gm] = lam;
-    a.lbar_hist[(long long)a.k * a.G_total + gm] = lam - lc;
-    if (a.last) a.dlam[gm] = (double)a.seed[t] * exp(lam - lc);
+    a.lam[(long long)a.k * a.G_total + gm] = (float)lam;
+    a.lbar[(long long)a.k * a.G_total + gm] = (float)(lam - lc);
+    if (a.last) a.dlam[gm] = (double)(a.seed ? a.seed[t] : a.seed0) * exp(lam - lc);
   }
 }
 
 // ------------------------------------------------------------------ adjoint
-// Log-likelihood (Sec. V model) and its partial derivatives for the
-// adjoint: d[0..4] = dl/dx, dl/dy, dl/dI, dl/dsigma_psf, dl/db.  One pass
-// over the patch with separable row sums: per row v with r = y - I gx gy,
-// R0 = sum r gx, R1 = sum r gx a, R2 = sum r gx a^2 (a the column offset), so
-// that sum r gx (u - x) = R1 + du0 R0 and sum r gx (u - x)^2 = R2 + 2 du0 R1
-// + du0^2 R0 with du0 = cx - R - x.  Pixels outside the frame count as
-// background, so only inside pixels depend on b.
-template <int R>
-__device__ __forceinline__ float loglik_grad(const float* __restrict__ yp, int pitch, int H, int W, float x, float y,
-                                             float I, const TrackParams& P, float (&d)[5]) {
-  constexpr int D = 2 * R + 1;
-  constexpr int PAD = 2 * R + 1;
-  const float cxf = floorf(x + 0.5f), cyf = floorf(y + 0.5f);
-  const int cx = (int)fminf(fmaxf(cxf, -(float)(R + 1)), (float)(W + R));
-  const int cy = (int)fminf(fmaxf(cyf, -(float)(R + 1)), (float)(H + R));
-  const float* __restrict__ row = yp + (long long)(cy - R + PAD) * pitch + (cx - R + PAD);
-  float gx[D];
-  gauss_row<R>(cxf, x, P.c_psf, P.kappa, gx);
-  float gy[D];
-  gauss_row<R>(cyf, y, P.c_psf, P.kappa, gy);
-  // inside-the-frame column / row ranges of the (true) patch
-  const float ulo = fmaxf(0.0f, (float)R - cxf), uhi = fminf((float)(2 * R), (float)(W - 1) + (float)R - cxf);
-  const float vlo = fmaxf(0.0f, (float)R - cyf), vhi = fminf((float)(2 * R), (float)(H - 1) + (float)R - cyf);
-  float ss = 0.0f, SI = 0.0f, S1 = 0.0f, Sy = 0.0f, Ss = 0.0f, Sb = 0.0f, Y2 = 0.0f, Y1 = 0.0f;
-  const float du0 = cxf - (float)R - x;
-  // patches wholly inside the frame (almost all) sum the b-derivative's
-  // residuals without per-pixel masks
-  const bool inside = ulo == 0.0f && uhi == (float)(2 * R) && vlo == 0.0f && vhi == (float)(2 * R);
-  auto rows = [&](auto inside_tag) {
-    constexpr bool IN = decltype(inside_tag)::value;
-#pragma unroll
-    for (int b = 0; b < D; ++b) {
-      const float* __restrict__ rp = row + (long long)b * pitch;
-      const float Igy = I * gy[b];
-      float R0 = 0.0f, R1 = 0.0f, R2 = 0.0f, Rb = 0.0f;
-#pragma unroll
-      for (int a = 0; a < D; ++a) {
-        const float yv = __ldg(rp + a);  // y = z - b, 0 outside the frame
-        const float r = fmaf(-gx[a], Igy, yv);
-        ss = fmaf(r, r, ss);
-        Y2 = fmaf(yv, yv, Y2);
-        Y1 += yv;
-        const float t = r * gx[a];
-        R0 += t;
-        R1 = fmaf(t, (float)a, R1);
-        R2 = fmaf(t, (float)(a * a), R2);
-        if constexpr (IN)
-          Rb += r;
-        else
-          Rb += ((float)a >= ulo && (float)a <= uhi) ? r : 0.0f;
-      }
-      const float dv = (cyf - (float)R + (float)b) - y;
-      const float sx1 = R1 + du0 * R0;
-      const float sx2 = R2 + 2.0f * du0 * R1 + du0 * du0 * R0;
-      SI = fmaf(gy[b], R0, SI);
-      S1 = fmaf(gy[b], sx1, S1);
-      Sy = fmaf(gy[b] * dv, R0, Sy);
-      Ss = fmaf(gy[b], fmaf(dv * dv, R0, sx2), Ss);
-      if (IN || ((float)b >= vlo && (float)b <= vhi)) Sb += Rb;
-    }
-  };
-  if (inside)
-    rows(std::true_type{});
-  else
-    rows(std::false_type{});
-  const float iso2 = 2.0f * P.inv2so2;  // 1 / sigma_obs^2
-  const float s2 = P.spsf * P.spsf;
-  d[0] = I * S1 / s2 * iso2;
-  d[1] = I * Sy / s2 * iso2;
-  d[2] = SI * iso2;
-  d[3] = I * Ss / (s2 * P.spsf) * iso2;
-  d[4] = Sb * iso2;
-  if (P.obs_model == 1) {
-    // frame likelihood ratio: + sum y^2 / (2 sigma_obs^2), whose only
-    // parameter is b (dy/db = -1 inside the frame, y = 0 outside)
-    d[4] -= Y1 * iso2;
-    return -(ss - Y2) * P.inv2so2;
-  }
-  return -ss * P.inv2so2;
+// Adds four neighbouring floats in one L2 operation.
+__device__ __forceinline__ void red_add_v4(float4* p, float x, float y, float z, float w) {
+  asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(__cvta_generic_to_global(p)), "f"(x), "f"(y), "f"(z), "f"(w)
+               : "memory");
 }
 
-template <int R>
-__global__ void __launch_bounds__(256, 3) k_adjoint(AdjointArgs a) {
+// Reverse step k: the softmax weights from the replay's log-weights, the
+// state adjoint (the likelihood's derivatives, stored by the replay, plus the
+// children's) and its transposed dynamics onto the recorded parents.  One CTA
+// per tile; the particle data is read once, coalesced.  Children of one
+// parent sit in neighbouring slots (resampling is monotone), so a segmented
+// sum over the warp's runs of equal parents leaves one vector reduction per
+// run; any other order is right too, with more of them.  Weight adjoints go
+// to the origin group per tile, gradient terms to one of GRAD_COPIES
+// accumulators, so that no address takes an atomic per warp.  Bound by the
+// 90 bytes a particle it moves and the step's normals it draws again.
+__global__ void __launch_bounds__(K1_THREADS, 4) k_adjoint(AdjointArgs a) {
+  constexpr int NW = K1_THREADS / 32;
+  constexpr unsigned FULL = 0xffffffffu;
   const int k = a.k;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  __shared__ double s_g[8][5];
-  for (int tile = blockIdx.x; tile < a.n_tiles; tile += gridDim.x) {
-    const int4 td = a.tiles[tile];
-    const TrackParams& P = a.trk[td.x];
-    const int g = td.y, Np = P.Np;
-    const long long Nt = (long long)P.G * Np;
-    const int hslot = k % a.history;
-    const float log_G = logf((float)P.G), log_Np = logf((float)Np);
-    const bool A_enters = (P.init_kind == INIT_POINT) || (P.init_kind == INIT_SHARING && g == 0);
-    float gacc[5] = {0, 0, 0, 0, 0};
-    for (int jj = threadIdx.x; jj < td.w; jj += blockDim.x) {
-      const int j = td.z + jj;
-      const long long il = (long long)g * Np + j, i = P.part_off + il;
-      const float4 s = a.pv[i];
-      const float I = a.In[i];
-      long long par = il;
-      int o = g;
-      if (k >= 1) {
-        par = a.parent[P.parent_off + (long long)hslot * Nt + il];
-        o = (int)fastdiv((uint32_t)par, P.m_Np);  // origin group (par < 2^31)
+  __shared__ float s_red[NW][8];
+  __shared__ int s_other[NW];
+  grid_dep_wait();
+  grid_dep_launch();
+  for (int m = blockIdx.x * K1_THREADS + threadIdx.x; m < a.G_total; m += gridDim.x * K1_THREADS)
+    a.dlam_clear[m] = 0.0;
+  const int4 td = a.tiles[blockIdx.x];
+  const TrackParams& P = a.trk[td.x];
+  const int g = td.y, Np = P.Np;
+  const uint32_t* __restrict__ par_t =
+      a.parent + P.parent_off + (long long)(k % a.history) * ((long long)P.G * Np);
+  const float lam = a.lam_k[P.group_off + g], dlam = (float)a.dlam_k[P.group_off + g];
+  uint32_t par[K1_PPT];
+  int o[K1_PPT], other = -1;
+  float dlw[K1_PPT], dI[K1_PPT], cI[K1_PPT];
+  float4 c[K1_PPT];
+  float v[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // gradient terms, then dL_{k-1} of g and of `other`
+#pragma unroll
+  for (int q = 0; q < K1_PPT; ++q) {
+    const int jj = threadIdx.x + q * K1_THREADS;
+    const long long il = (long long)g * Np + td.z + jj, i = P.part_off + il;
+    par[q] = 0xffffffffu;
+    o[q] = g;
+    dlw[q] = 0.0f;
+    cI[q] = 0.0f;
+    c[q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (jj < td.w) {
+      const float4 d = a.dl_pv[i];
+      const float db = a.dl_b[i], lw = a.dl_lw[i];
+      if (!a.last) {
+        c[q] = a.Cc_pv[i];
+        cI[q] = a.Cc_I[i];
       }
-      float dl[5];
-      const float l = loglik_grad<R>(a.ypad + P.ypad_off, P.pitch, P.H, P.W, s.x, s.y, I, P, dl);
-      const float lb = k >= 1 ? (float)a.lbar_prev[P.group_off + o] : -log_G;
-      const float lw = lb - log_Np + l;
-      const float lam = (float)a.lam_k[P.group_off + g];
-      const float wbar = (lw == lw && lw - lam > -87.0f) ? __expf(lw - lam) : 0.0f;
-      const float dlw = (float)a.dlam_k[P.group_off + g] * wbar;
       if (k >= 1) {
-        // dL_{k-1} of the origin group: the tile's slots originate in g or in
-        // its ring predecessor, so a warp adds two sums instead of 32 terms
-        // (slots of any third origin add theirs directly)
-        const unsigned full = __activemask();
-        const int other = __reduce_max_sync(full, o != g ? o : -1);
-        const bool third = o != g && o != other;
-        const float own = warp_sum_active(full, (o == g) ? dlw : 0.0f);
-        const float pre = warp_sum_active(full, (o != g && !third) ? dlw : 0.0f);
-        const int leader = __ffs(full) - 1;
-        if (lane == leader) {
-          if (own != 0.0f) atomicAdd(&a.D[P.group_off + g], (double)own);
-          if (other >= 0 && pre != 0.0f) atomicAdd(&a.D[P.group_off + other], (double)pre);
-        }
-        if (third && dlw != 0.0f) atomicAdd(&a.D[P.group_off + o], (double)dlw);
+        par[q] = par_t[il];
+        o[q] = (int)fastdiv(par[q], P.m_Np);  // origin group
       }
-      // adjoint of the state: the likelihood term plus the children's
-      float4 c = a.Cc_pv[i];
-      float cI = a.Cc_I[i];
-      a.Cc_pv[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      a.Cc_pv[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       a.Cc_I[i] = 0.0f;
-      c.x = fmaf(dlw, dl[0], c.x);
-      c.y = fmaf(dlw, dl[1], c.y);
-      cI = fmaf(dlw, dl[2], cI);
-      gacc[0] = fmaf(dlw, dl[3], gacc[0]);  // sigma_psf
-      gacc[2] = fmaf(dlw, dl[4], gacc[2]);  // background
-      if (k >= 1) {
+      const float wbar = (lw == lw && lw - lam > -87.0f) ? __expf(lw - lam) : 0.0f;
+      dlw[q] = dlam * wbar;
+      c[q].x = fmaf(dlw[q], d.x, c[q].x);
+      c[q].y = fmaf(dlw[q], d.y, c[q].y);
+      cI[q] = fmaf(dlw[q], d.z, cI[q]);
+      v[0] = fmaf(dlw[q], d.w, v[0]);  // sigma_psf
+      v[2] = fmaf(dlw[q], db, v[2]);   // background
+    }
+    other = max(other, o[q] != g ? o[q] : -1);
+  }
+  if (k >= 1) {
+    // dL_{k-1} of the origin groups: the tile's slots originate in g or in
+    // its ring predecessor (slots of any third origin add theirs directly)
+    other = __reduce_max_sync(FULL, other);
+#pragma unroll
+    for (int q = 0; q < K1_PPT; ++q) {
+      if (o[q] == g)
+        v[5] += dlw[q];
+      else if (o[q] == other)
+        v[6] += dlw[q];
+      else if (dlw[q] != 0.0f)
+        atomicAdd(&a.D[P.group_off + o[q]], (double)dlw[q]);
+      const int jj = threadIdx.x + q * K1_THREADS;
+      float t[5] = {c[q].x, c[q].y, c[q].x + c[q].z, c[q].y + c[q].w, cI[q]};
+      if (jj < td.w) {
+        const int j = td.z + jj;
         uint4 w0 = make_uint4(j, g, k, P.tag | (ST_PROP << 4) | 0u);
         uint4 w1 = make_uint4(j, g, k, P.tag | (ST_PROP << 4) | 1u);
         philox2(P.key0, P.key1, w0, w1);
-        float e0, e1, e2, e3, e4, e5;
+        float e0, e1, e2, e3;
         box_muller_fast(w0.x, w0.y, e0, e1);
         box_muller_fast(w0.z, w0.w, e2, e3);
-        box_muller_fast(w1.x, w1.y, e4, e5);
-        gacc[3] = fmaf(c.x, e0, fmaf(c.y, e1, gacc[3]));  // sigma_pos
-        gacc[4] = fmaf(c.z, e2, fmaf(c.w, e3, gacc[4]));  // sigma_v
-        // NCV Jacobian transposed onto the parent: x <- x, vx <- x + vx, ...
-        // Resampled children of one parent sit in neighbouring slots: lanes
-        // sharing a parent add their terms first, one lane stores the sum.
-        const long long pi = P.part_off + par;
-        float t[5] = {c.x, c.y, c.x + c.z, c.y + c.w, cI};
-        const unsigned peers = __match_any_sync(__activemask(), (unsigned long long)pi);
-        if (peers != (1u << lane)) {
+        v[3] = fmaf(c[q].x, e0, fmaf(c[q].y, e1, v[3]));  // sigma_pos
+        v[4] = fmaf(c[q].z, e2, fmaf(c[q].w, e3, v[4]));  // sigma_v
+      }
+      // NCV Jacobian transposed onto the parent (x <- x, vx <- x + vx, ...),
+      // summed over the run of lanes that share it
+      const uint32_t prev = __shfl_up_sync(FULL, par[q], 1);
+      const unsigned heads = __ballot_sync(FULL, lane == 0 || par[q] != prev);
+      const unsigned above = lane < 31 ? heads >> (lane + 1) : 0u;
+      const int left = above ? __ffs(above) - 1 : 31 - lane;  // lanes of the run after this one
 #pragma unroll
-          for (int q = 0; q < 5; ++q) t[q] = warp_sum_active(peers, t[q]);
+      for (int dd = 1; dd < 32; dd *= 2) {
+        if (!__any_sync(FULL, left >= dd)) break;
+#pragma unroll
+        for (int x = 0; x < 5; ++x) {
+          const float up = __shfl_down_sync(FULL, t[x], dd);
+          if (left >= dd) t[x] += up;
         }
-        if (lane == __ffs(peers) - 1) {
-          atomicAdd(&a.Cp_pv[pi].x, t[0]);
-          atomicAdd(&a.Cp_pv[pi].y, t[1]);
-          atomicAdd(&a.Cp_pv[pi].z, t[2]);
-          atomicAdd(&a.Cp_pv[pi].w, t[3]);
-          atomicAdd(&a.Cp_I[pi], t[4]);
-        }
-      } else if (A_enters) {
-        gacc[1] += cI;  // the initial intensity is A
+      }
+      if (((heads >> lane) & 1u) && jj < td.w) {
+        const long long pi = P.part_off + par[q];
+        red_add_v4(&a.Cp_pv[pi], t[0], t[1], t[2], t[3]);
+        atomicAdd(&a.Cp_I[pi], t[4]);
       }
     }
+  } else if ((P.init_kind == INIT_POINT) || (P.init_kind == INIT_SHARING && g == 0)) {
 #pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      const float v = warp_sum(gacc[q]);
-      if (lane == 0) s_g[warp][q] = (double)v;
+    for (int q = 0; q < K1_PPT; ++q) v[1] += cI[q];  // the initial intensity is A
+  }
+  int slot;
+  const float x = warp_reduce8(v, lane, slot);
+  if ((lane & 3) == 0) s_red[warp][slot] = x;
+  if (lane == 0) s_other[warp] = other;
+  __syncthreads();
+  if (warp == 0) {
+    if (lane < 6) {
+      double r = 0.0;
+#pragma unroll
+      for (int w = 0; w < NW; ++w) r += (double)s_red[w][lane];
+      if (r != 0.0) {
+        if (lane < 5)
+          atomicAdd(&a.grad[((long long)(blockIdx.x % GRAD_COPIES) * a.n_tracks + td.x) * GRAD_STRIDE + lane], r);
+        else
+          atomicAdd(&a.D[P.group_off + g], r);
+      }
+    } else if (k >= 1 && lane >= 8 && lane < 8 + NW) {
+      // the warps' second origins, as a rule one group: its first warp adds
+      const int w = lane - 8, ow = s_other[w];
+      double r = 0.0;
+      bool first = ow >= 0;
+      for (int u = 0; u < NW; ++u)
+        if (s_other[u] == ow) {
+          first = first && u >= w;
+          r += (double)s_red[u][6];
+        }
+      if (first && r != 0.0) atomicAdd(&a.D[P.group_off + ow], r);
     }
-    __syncthreads();
-    if (threadIdx.x < 5) {
-      double v = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += s_g[w][threadIdx.x];
-      if (v != 0.0) atomicAdd(&a.grad[td.x * 5 + threadIdx.x], v);
-    }
-    __syncthreads();
   }
 }
 
-// dL_{k-1,m} = sum of the origin-m log-weight adjoints of step k; reset D.
-__global__ void k_adjoint_groups(double* __restrict__ dlam, double* __restrict__ D, int G_total) {
-  for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < G_total; m += gridDim.x * blockDim.x) {
-    dlam[m] = D[m];
-    D[m] = 0.0;
-  }
-}
-
+// The gradient and log Z out of their accumulators.
 __global__ void k_grad_out(const double* __restrict__ g, const double* __restrict__ lz, float* __restrict__ out,
                            double* __restrict__ lz_out, int n) {
+  grid_dep_wait();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n * 5; i += gridDim.x * blockDim.x) {
-    out[i] = (float)g[i];
+    double v = 0.0;
+#pragma unroll
+    for (int c = 0; c < GRAD_COPIES; ++c) v += g[((long long)c * n + i / 5) * GRAD_STRIDE + i % 5];
+    out[i] = (float)v;
     if (lz_out && i % 5 == 0) lz_out[i / 5] = lz[i / 5];
   }
 }
 
 // ------------------------------------------------------------------ launchers
-cudaError_t launch_replay(const ReplayArgs& a, int R, int grid, cudaStream_t s) {
-  switch (R) {
-    case 1: k_replay<1><<<grid, 256, 0, s>>>(a); break;
-    case 2: k_replay<2><<<grid, 256, 0, s>>>(a); break;
-    case 3: k_replay<3><<<grid, 256, 0, s>>>(a); break;
-    case 4: k_replay<4><<<grid, 256, 0, s>>>(a); break;
-    case 5: k_replay<5><<<grid, 256, 0, s>>>(a); break;
-    case 6: k_replay<6><<<grid, 256, 0, s>>>(a); break;
-    case 7: k_replay<7><<<grid, 256, 0, s>>>(a); break;
-    default: return cudaErrorInvalidValue;
-  }
-  return cudaGetLastError();
+template <typename Arg, typename... Params>
+static cudaError_t launch_pdl(void (*kernel)(Params...), int grid, int block, bool pdl, cudaStream_t s,
+                              const Arg& arg) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, arg);
 }
 
-cudaError_t launch_replay_groups(const ReplayGroupArgs& a, int n_tracks, int max_G, cudaStream_t s) {
-  (void)max_G;
-  k_replay_groups<<<n_tracks, 256, 0, s>>>(a);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_adjoint(const AdjointArgs& a, int R, int grid, cudaStream_t s) {
+cudaError_t launch_replay(const ReplayArgs& a, int R, int n_tiles, bool pdl, cudaStream_t s) {
   switch (R) {
-    case 1: k_adjoint<1><<<grid, 256, 0, s>>>(a); break;
-    case 2: k_adjoint<2><<<grid, 256, 0, s>>>(a); break;
-    case 3: k_adjoint<3><<<grid, 256, 0, s>>>(a); break;
-    case 4: k_adjoint<4><<<grid, 256, 0, s>>>(a); break;
-    case 5: k_adjoint<5><<<grid, 256, 0, s>>>(a); break;
-    case 6: k_adjoint<6><<<grid, 256, 0, s>>>(a); break;
-    case 7: k_adjoint<7><<<grid, 256, 0, s>>>(a); break;
+    case 1: return launch_pdl(k_replay<1>, n_tiles, K1_THREADS, pdl, s, a);
+    case 2: return launch_pdl(k_replay<2>, n_tiles, K1_THREADS, pdl, s, a);
+    case 3: return launch_pdl(k_replay<3>, n_tiles, K1_THREADS, pdl, s, a);
+    case 4: return launch_pdl(k_replay<4>, n_tiles, K1_THREADS, pdl, s, a);
+    case 5: return launch_pdl(k_replay<5>, n_tiles, K1_THREADS, pdl, s, a);
+    case 6: return launch_pdl(k_replay<6>, n_tiles, K1_THREADS, pdl, s, a);
+    case 7: return launch_pdl(k_replay<7>, n_tiles, K1_THREADS, pdl, s, a);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
+}
+
+// A warp per group up to 32 groups: with few groups 256 threads suffice.
+cudaError_t launch_replay_groups(const ReplayGroupArgs& a, int n_tracks, int max_G, bool pdl, cudaStream_t s) {
+  return launch_pdl(k_replay_groups, n_tracks, max_G <= 8 ? 256 : RG_GROUP_THREADS, pdl, s, a);
+}
+
+cudaError_t launch_adjoint(const AdjointArgs& a, int n_tiles, bool pdl, cudaStream_t s) {
+  return launch_pdl(k_adjoint, n_tiles, K1_THREADS, pdl, s, a);
 }
 
 // Caller-supplied ancestry for the replay (pf_set_replay): for steps k = 1 ..
@@ -455,11 +667,6 @@ cudaError_t launch_set_replay(const TrackParams* trk, const int4* tiles, int n_t
                               cudaStream_t s) {
   if (T < 2) return cudaSuccess;
   k_set_replay<<<dim3(grid, T - 1), 256, 0, s>>>(trk, tiles, n_tiles, parents, n_total, parent, history, bad);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_adjoint_groups(double* dlam, double* D, int G_total, cudaStream_t s) {
-  k_adjoint_groups<<<(G_total + 255) / 256, 256, 0, s>>>(dlam, D, G_total);
   return cudaGetLastError();
 }
 

@@ -84,18 +84,20 @@ struct pf_handle {
   CUtensorMap* tmaps = nullptr;  // nullptr: frames read through L1 only
   // pf_backward buffers (present when every track records its ancestry)
   bool adjoint = false;
-  int adj_slots = 0, adj_ckpts = 0;
-  float4* rp_pv = nullptr;   // adj_slots x N_total (replay / segment states)
+  int adj_steps = 0;         // steps whose derivatives fit at once (the whole history, or a segment)
+  float4* rp_pv = nullptr;   // N_total x slots: the replay's states, by step parity
   float* rp_I = nullptr;
-  float4* ck_pv = nullptr;   // adj_ckpts x N_total (checkpoints)
+  float4* ck_pv = nullptr;   // N_total x checkpoints of the states
   float* ck_I = nullptr;
   float4* ca_pv[2] = {nullptr, nullptr};  // state adjoints
   float* ca_I[2] = {nullptr, nullptr};
-  double* lam_hist = nullptr;   // history x G_total
-  double* lbar_hist = nullptr;
-  double* dlam = nullptr;       // G_total
-  double* Dacc = nullptr;       // G_total
-  double* grad = nullptr;       // n_tracks x 5
+  float4* dl_pv = nullptr;      // adj_steps x N_total: the likelihood's derivatives
+  float* dl_b = nullptr;
+  float* dl_lw = nullptr;       // and the log-weights
+  float* lam = nullptr;         // history x G_total
+  float* lbar = nullptr;
+  double* dL[3] = {};           // G_total each: dL of the step, of the one before, and the next to clear
+  double* grad = nullptr;       // GRAD_COPIES x n_tracks x GRAD_STRIDE
   double* logz_rp = nullptr;    // n_tracks
   float* seed = nullptr;        // n_tracks
   int* replay_bad = nullptr;    // pf_set_replay's count of out-of-range parents
@@ -176,10 +178,10 @@ struct Layout {
   size_t trk, ts, gs, gd, tiles, frame_of, pv0, pv1, I0, I1, anc, lw, tp, ypad, hist, ghist, ring, ring_next, exo_next, keys_next,
       tile_ctr, parent, ds, rq, chunks, chunk_q, fsync,
       tmap, total;
-  size_t rp_pv, rp_I, ck_pv, ck_I, ca_pv0, ca_pv1, ca_I0, ca_I1, lam_hist, lbar_hist, dlam, Dacc, grad, logz, seed,
-      replay_bad;
+  size_t rp_pv, rp_I, ck_pv, ck_I, ca_pv0, ca_pv1, ca_I0, ca_I1, lam, lbar, dL0, dL1, dL2, logz, seed, replay_bad;
+  size_t dl_pv, dl_b, dl_lw, grad;
   bool adjoint = false;
-  int adj_slots = 0, adj_ckpts = 0;
+  int adj_steps = 0;
   long long N_total = 0, ypad_total = 0, parent_total = 0, ghist_total = 0;
   int G_total = 0, n_tiles = 0, hist_total = 0, n_chunks = 0;
   int R = 5;
@@ -249,6 +251,10 @@ std::string validate(const pf_track_config* c, int n, int history) {
   return "";
 }
 
+// Workspace that the reverse sweep may take to keep every step's derivatives:
+// 4 GiB, 1.5 % of the card (178 steps of a million particles).
+constexpr size_t ADJ_STORE_MAX = (size_t)4 << 30;
+
 // Checkpoint spacing of pf_backward for T steps: ceil(sqrt(T)).
 int adjoint_segment(int T) {
   int C = 1;
@@ -309,27 +315,38 @@ Layout plan(const pf_track_config* c, int n, int history) {
   for (int t = 0; t < n; ++t) L.adjoint = L.adjoint && c[t].record_ancestors;
   if (L.adjoint) {
     const int C = adjoint_segment(history);
-    L.adj_slots = C < 2 ? 2 : C;
-    L.adj_ckpts = (history + C - 1) / C + 1;
-    L.rp_pv = take(sizeof(float4) * (size_t)L.N_total * L.adj_slots);
-    L.rp_I = take(sizeof(float) * (size_t)L.N_total * L.adj_slots);
-    L.ck_pv = take(sizeof(float4) * (size_t)L.N_total * L.adj_ckpts);
-    L.ck_I = take(sizeof(float) * (size_t)L.N_total * L.adj_ckpts);
+    const size_t slots = C < 2 ? 2 : C, ckpts = (size_t)(history + C - 1) / C + 1;
+    L.rp_pv = take(sizeof(float4) * (size_t)L.N_total * slots);
+    L.rp_I = take(sizeof(float) * (size_t)L.N_total * slots);
+    L.ck_pv = take(sizeof(float4) * (size_t)L.N_total * ckpts);
+    L.ck_I = take(sizeof(float) * (size_t)L.N_total * ckpts);
     L.ca_pv0 = take(sizeof(float4) * (size_t)L.N_total);
     L.ca_pv1 = take(sizeof(float4) * (size_t)L.N_total);
     L.ca_I0 = take(sizeof(float) * (size_t)L.N_total);
     L.ca_I1 = take(sizeof(float) * (size_t)L.N_total);
-    L.lam_hist = take(sizeof(double) * (size_t)history * L.G_total);
-    L.lbar_hist = take(sizeof(double) * (size_t)history * L.G_total);
-    L.dlam = take(sizeof(double) * (size_t)L.G_total);
-    L.Dacc = take(sizeof(double) * (size_t)L.G_total);
-    L.grad = take(sizeof(double) * 5 * (size_t)n);
+    // (sizes that the checkpoint format has: the first two hold FP32 values)
+    L.lam = take(sizeof(double) * (size_t)history * L.G_total);
+    L.lbar = take(sizeof(double) * (size_t)history * L.G_total);
+    L.dL0 = take(sizeof(double) * (size_t)L.G_total);
+    L.dL1 = take(sizeof(double) * (size_t)L.G_total);
+    take(sizeof(double) * 5 * (size_t)n);
     L.logz = take(sizeof(double) * (size_t)n);
     L.seed = take(sizeof(float) * (size_t)n);
     L.replay_bad = take(sizeof(int));
   }
   L.saved = o;
   L.order = take(sizeof(int) * (size_t)L.G_total);
+  if (L.adjoint) {
+    // the derivatives of every step of the history where they take at most
+    // ADJ_STORE_MAX, else of one segment between checkpoints
+    const size_t per_step = (size_t)L.N_total * (sizeof(float4) + 2 * sizeof(float));
+    L.adj_steps = per_step * (size_t)history <= ADJ_STORE_MAX ? history : adjoint_segment(history);
+    L.dl_pv = take(sizeof(float4) * (size_t)L.N_total * L.adj_steps);
+    L.dl_b = take(sizeof(float) * (size_t)L.N_total * L.adj_steps);
+    L.dl_lw = take(sizeof(float) * (size_t)L.N_total * L.adj_steps);
+    L.dL2 = take(sizeof(double) * (size_t)L.G_total);
+    L.grad = take(sizeof(double) * GRAD_COPIES * GRAD_STRIDE * (size_t)n);
+  }
   L.total = o;
   return L;
 }
@@ -615,8 +632,7 @@ pf_status pf_init(const pf_track_config* cfg, int32_t n_tracks, int32_t history,
   h->tmaps = (CUtensorMap*)(w + L.tmap);
   if (L.adjoint) {
     h->adjoint = true;
-    h->adj_slots = L.adj_slots;
-    h->adj_ckpts = L.adj_ckpts;
+    h->adj_steps = L.adj_steps;
     h->rp_pv = (float4*)(w + L.rp_pv);
     h->rp_I = (float*)(w + L.rp_I);
     h->ck_pv = (float4*)(w + L.ck_pv);
@@ -625,10 +641,14 @@ pf_status pf_init(const pf_track_config* cfg, int32_t n_tracks, int32_t history,
     h->ca_pv[1] = (float4*)(w + L.ca_pv1);
     h->ca_I[0] = (float*)(w + L.ca_I0);
     h->ca_I[1] = (float*)(w + L.ca_I1);
-    h->lam_hist = (double*)(w + L.lam_hist);
-    h->lbar_hist = (double*)(w + L.lbar_hist);
-    h->dlam = (double*)(w + L.dlam);
-    h->Dacc = (double*)(w + L.Dacc);
+    h->dl_pv = (float4*)(w + L.dl_pv);
+    h->dl_b = (float*)(w + L.dl_b);
+    h->dl_lw = (float*)(w + L.dl_lw);
+    h->lam = (float*)(w + L.lam);
+    h->lbar = (float*)(w + L.lbar);
+    h->dL[0] = (double*)(w + L.dL0);
+    h->dL[1] = (double*)(w + L.dL1);
+    h->dL[2] = (double*)(w + L.dL2);
     h->grad = (double*)(w + L.grad);
     h->logz_rp = (double*)(w + L.logz);
     h->seed = (float*)(w + L.seed);
@@ -759,7 +779,7 @@ pf_status pf_init(const pf_track_config* cfg, int32_t n_tracks, int32_t history,
   std::vector<int> ident(n_tracks);  // every track reads its own padded frame until a step shares one
   for (int t = 0; t < n_tracks; ++t) ident[t] = t;
   cudaError_t e;
-  if ((e = cudaMemsetAsync(w, 0, L.total, s)) != cudaSuccess) { pf_destroy(h); return cuda_fail(nullptr, e, "cudaMemsetAsync"); }
+  if ((e = cudaMemsetAsync(w, 0, L.saved, s)) != cudaSuccess) { pf_destroy(h); return cuda_fail(nullptr, e, "cudaMemsetAsync"); }
   if ((e = cudaMemcpyAsync(h->trk, tp.data(), sizeof(TrackParams) * n_tracks, cudaMemcpyHostToDevice, s)) ||
       (e = cudaMemcpyAsync(w + L.order, order.data(), sizeof(int) * order.size(), cudaMemcpyHostToDevice, s)) ||
       (e = cudaMemcpyAsync(h->gd, gd.data(), sizeof(GroupDesc) * gd.size(), cudaMemcpyHostToDevice, s)) ||
@@ -1476,84 +1496,95 @@ pf_status pf_backward(pf_handle* h, const float* const* frames_host, int32_t T, 
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e;
   const long long N = h->N_total;
-  const int C = adjoint_segment(T);
-  const int nseg = (T + C - 1) / C;
   const int G = h->G_total;
-  auto slot_pv = [&](int i) { return h->rp_pv + (long long)i * N; };
-  auto slot_I = [&](int i) { return h->rp_I + (long long)i * N; };
-  auto ck_pv = [&](int i) { return h->ck_pv + (long long)i * N; };
-  auto ck_I = [&](int i) { return h->ck_I + (long long)i * N; };
-  if ((e = cudaMemsetAsync(h->grad, 0, sizeof(double) * 5 * h->n_tracks, s)) ||
-      (e = cudaMemsetAsync(h->logz_rp, 0, sizeof(double) * h->n_tracks, s)) ||
-      (e = cudaMemsetAsync(h->Dacc, 0, sizeof(double) * G, s)) ||
-      (e = cudaMemsetAsync(h->ca_pv[0], 0, sizeof(float4) * N, s)) ||
-      (e = cudaMemsetAsync(h->ca_pv[1], 0, sizeof(float4) * N, s)) ||
-      (e = cudaMemsetAsync(h->ca_I[0], 0, sizeof(float) * N, s)) ||
-      (e = cudaMemsetAsync(h->ca_I[1], 0, sizeof(float) * N, s)) ||
-      (e = cudaMemcpyAsync(h->seed, dlogZ_host, sizeof(float) * h->n_tracks, cudaMemcpyHostToDevice, s)))
+  // one segment of all T steps if their derivatives fit, else segments of C,
+  // replayed once for the group log-weights and checkpoints, and then each
+  // from its checkpoint
+  const bool whole = T <= h->adj_steps;
+  const int C = whole ? T : adjoint_segment(T);
+  const int nseg = (T + C - 1) / C;
+  if (h->n_tracks > 1 &&
+      (e = cudaMemcpyAsync(h->seed, dlogZ_host, sizeof(float) * h->n_tracks, cudaMemcpyHostToDevice, s)) != cudaSuccess)
     return cuda_fail(h, e, "pf_backward setup");
-  const int grid = h->k1_grid;
-  // forward replay with the recorded ancestry; checkpoints every C steps
-  InitArgs ia{h->trk, h->tiles, h->n_tiles, N, nullptr, slot_pv(0), slot_I(0)};
-  if ((e = launch_init(ia, grid, s)) != cudaSuccess) return cuda_fail(h, e, "k_init");
-  for (int k = 0; k < T; ++k) {
-    if ((e = prep_frames(h, frames_host + (long long)k * h->n_tracks, s, false)) != cudaSuccess)
+  const InitArgs ia{h->trk, h->tiles, h->n_tiles, N, nullptr, h->rp_pv, h->rp_I};
+  if ((e = launch_init(ia, h->k1_grid, s)) != cudaSuccess) return cuda_fail(h, e, "k_init");
+  // Replay of step k, its derivatives into slot `slot` (-1: not kept).  Step k
+  // reads X_{k-1} from replay buffer (k - 1) & 1; `given`: X_k comes from the
+  // checkpoint of segment k / C.
+  auto replay = [&](int k, int slot, bool given, bool groups) -> pf_status {
+    const float* const* frames = frames_host + (long long)k * h->n_tracks;
+    if (h->n_tracks > 1 && (e = prep_frames(h, frames, s, false)) != cudaSuccess)
       return cuda_fail(h, e, "k_frame_prep");
     ReplayArgs ra{};
-    ra.trk = h->trk; ra.tiles = h->tiles; ra.n_tiles = h->n_tiles; ra.parent = h->parent; ra.history = h->history;
+    ra.trk = h->trk; ra.tiles = h->tiles; ra.parent = h->parent; ra.history = h->history;
     ra.k = k;
-    ra.pv_in = k >= 1 ? slot_pv((k - 1) & 1) : nullptr;
-    ra.I_in = k >= 1 ? slot_I((k - 1) & 1) : nullptr;
-    ra.pv_out = slot_pv(k & 1);
-    ra.I_out = slot_I(k & 1);
-    ra.ck_pv = (k % C == 0) ? ck_pv(k / C) : nullptr;
-    ra.ck_I = (k % C == 0) ? ck_I(k / C) : nullptr;
-    ra.weights = 1;
+    ra.propagate = k >= 1 && !given;
+    const long long in = (long long)((k - 1) & 1) * N, out = (long long)(k & 1) * N;
+    const long long ck = (long long)(k / C) * N;
+    const bool from_ck = !given && !groups && k >= 1 && (k - 1) % C == 0;  // the segment's second step
+    ra.pv_in = from_ck ? h->ck_pv + ck : h->rp_pv + in;
+    ra.I_in = from_ck ? h->ck_I + ck : h->rp_I + in;
+    ra.pv_out = given ? h->ck_pv + ck : h->rp_pv + out;
+    ra.I_out = given ? h->ck_I + ck : h->rp_I + out;
+    if (!whole && groups && k % C == 0) {
+      ra.ck_pv = h->ck_pv + ck;
+      ra.ck_I = h->ck_I + ck;
+    }
+    if (groups && k == 0) {
+      ra.zero_pv = h->ca_pv[T & 1];
+      ra.zero_I = h->ca_I[T & 1];
+    }
+    if (slot >= 0) {
+      ra.dl_pv = h->dl_pv + (long long)slot * N;
+      ra.dl_b = h->dl_b + (long long)slot * N;
+      ra.dl_lw = h->dl_lw + (long long)slot * N;
+    }
+    ra.zraw = h->n_tracks == 1 ? frames[0] : nullptr;
     ra.ypad = h->ypad;
-    ra.lbar_prev = k >= 1 ? h->lbar_hist + (long long)(k - 1) * G : nullptr;
+    ra.lbar_prev = k >= 1 ? h->lbar + (long long)(k - 1) * G : nullptr;
     ra.tile_part = h->tile_part;
-    if ((e = launch_replay(ra, h->R, grid, s)) != cudaSuccess) return cuda_fail(h, e, "k_replay");
-    ReplayGroupArgs rg{h->trk, h->gd, h->tile_part, k, G, h->lam_hist, h->lbar_hist, h->logz_rp, h->dlam, h->seed,
-                       k == T - 1 ? 1 : 0};
-    if ((e = launch_replay_groups(rg, h->n_tracks, h->max_G, s)) != cudaSuccess)
+    if ((e = launch_replay(ra, h->R, h->n_tiles, h->pdl, s)) != cudaSuccess) return cuda_fail(h, e, "k_replay");
+    if (!groups) return PF_OK;
+    const ReplayGroupArgs rg{h->trk,  h->gd,    h->tile_part, k,
+                             G,       h->lam,   h->lbar,      h->logz_rp,
+                             h->dL[0], h->dL[1], h->grad,     h->n_tracks > 1 ? h->seed : nullptr,
+                             dlogZ_host[0], k == T - 1 ? 1 : 0};
+    if ((e = launch_replay_groups(rg, h->n_tracks, h->max_G, h->pdl, s)) != cudaSuccess)
       return cuda_fail(h, e, "k_replay_groups");
+    return PF_OK;
+  };
+  for (int k = 0; k < T; ++k) {
+    const pf_status st = replay(k, whole ? k : -1, false, true);
+    if (st != PF_OK) return st;
   }
-  // reverse sweep, segment by segment, states recomputed from checkpoints
   for (int sg = nseg - 1; sg >= 0; --sg) {
     const int k0 = sg * C, k1 = (k0 + C < T) ? k0 + C : T;
-    for (int k = k0 + 1; k < k1; ++k) {
-      ReplayArgs ra{};
-      ra.trk = h->trk; ra.tiles = h->tiles; ra.n_tiles = h->n_tiles; ra.parent = h->parent;
-      ra.history = h->history; ra.k = k;
-      ra.pv_in = (k - 1 == k0) ? ck_pv(sg) : slot_pv(k - 1 - k0);
-      ra.I_in = (k - 1 == k0) ? ck_I(sg) : slot_I(k - 1 - k0);
-      ra.pv_out = slot_pv(k - k0);
-      ra.I_out = slot_I(k - k0);
-      ra.weights = 0;
-      ra.ypad = h->ypad;
-      ra.tile_part = h->tile_part;
-      if ((e = launch_replay(ra, h->R, grid, s)) != cudaSuccess) return cuda_fail(h, e, "k_replay");
+    for (int k = k0; !whole && k < k1; ++k) {
+      const pf_status st = replay(k, k - k0, k == k0, false);
+      if (st != PF_OK) return st;
     }
     for (int k = k1 - 1; k >= k0; --k) {
-      if ((e = prep_frames(h, frames_host + (long long)k * h->n_tracks, s, false)) != cudaSuccess)
-        return cuda_fail(h, e, "k_frame_prep");
+      const long long at = (long long)(k - k0) * N;
+      const int r = T - 1 - k;  // dL rotates: step k reads buffer r, adds to r + 1 and clears r + 2
       AdjointArgs aa{};
-      aa.trk = h->trk; aa.tiles = h->tiles; aa.n_tiles = h->n_tiles; aa.parent = h->parent;
+      aa.trk = h->trk; aa.tiles = h->tiles; aa.parent = h->parent;
       aa.history = h->history; aa.k = k;
-      aa.pv = (k == k0) ? ck_pv(sg) : slot_pv(k - k0);
-      aa.In = (k == k0) ? ck_I(sg) : slot_I(k - k0);
-      aa.ypad = h->ypad;
-      aa.lbar_prev = k >= 1 ? h->lbar_hist + (long long)(k - 1) * G : nullptr;
-      aa.lam_k = h->lam_hist + (long long)k * G;
-      aa.dlam_k = h->dlam;
-      aa.D = h->Dacc;
+      aa.last = k == T - 1;
+      aa.n_tracks = h->n_tracks;
+      aa.G_total = G;
+      aa.dl_pv = h->dl_pv + at;
+      aa.dl_b = h->dl_b + at;
+      aa.dl_lw = h->dl_lw + at;
+      aa.lam_k = h->lam + (long long)k * G;
+      aa.dlam_k = h->dL[r % 3];
+      aa.D = h->dL[(r + 1) % 3];
+      aa.dlam_clear = h->dL[(r + 2) % 3];
       aa.Cc_pv = h->ca_pv[k & 1];
       aa.Cc_I = h->ca_I[k & 1];
       aa.Cp_pv = h->ca_pv[(k + 1) & 1];
       aa.Cp_I = h->ca_I[(k + 1) & 1];
       aa.grad = h->grad;
-      if ((e = launch_adjoint(aa, h->R, grid, s)) != cudaSuccess) return cuda_fail(h, e, "k_adjoint");
-      if ((e = launch_adjoint_groups(h->dlam, h->Dacc, G, s)) != cudaSuccess) return cuda_fail(h, e, "k_adjoint_groups");
+      if ((e = launch_adjoint(aa, h->n_tiles, h->pdl, s)) != cudaSuccess) return cuda_fail(h, e, "k_adjoint");
     }
   }
   if ((e = launch_grad_out(h->grad, h->logz_rp, grad_dev, logZ_dev, h->n_tracks, s)) != cudaSuccess)

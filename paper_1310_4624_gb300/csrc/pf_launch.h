@@ -172,22 +172,31 @@ struct GroupClasses {
 };
 
 // pf_backward (pf_adjoint.cu)
+// The gradient's accumulators: GRAD_COPIES of GRAD_STRIDE doubles per track
+// (five used), copy-major, so that a track's copies lie in different lines.
+constexpr int GRAD_COPIES = 16, GRAD_STRIDE = 8;
+
 struct ReplayArgs {
   const TrackParams* trk;
   const int4* tiles;
-  int n_tiles;
   const uint32_t* parent;  // recorded ancestry
   int history;
   int k;
-  const float4* pv_in;     // X_{k-1} (k >= 1)
+  int propagate;           // 1: X_k from X_{k-1}, 0: X_k is given in pv_out
+  const float4* pv_in;     // X_{k-1}
   const float* I_in;
-  float4* pv_out;          // X_k (read only at k = 0)
+  float4* pv_out;          // X_k
   float* I_out;
   float4* ck_pv;           // optional copy of X_k (checkpoint), or nullptr
   float* ck_I;
-  int weights;             // 1: log-weights and per-tile (max, sum exp)
+  float4* zero_pv;         // optional buffers to clear (the sweep's first parent adjoints)
+  float* zero_I;
+  float4* dl_pv;           // optional: dl/dx, dl/dy, dl/dI, dl/dsigma_psf,
+  float* dl_b;             // dl/db
+  float* dl_lw;            // and the log-weight, for the reverse sweep
+  const float* zraw;       // single track: the caller's frame; nullptr: the padded frames
   const float* ypad;
-  const double* lbar_prev; // lbar_{k-1} per global group (k >= 1)
+  const float* lbar_prev;  // lbar_{k-1} per global group (k >= 1)
   float* tile_part;
 };
 
@@ -197,39 +206,43 @@ struct ReplayGroupArgs {
   const float* tile_part;
   int k;
   int G_total;
-  double* lam_hist;        // [k][global group]
-  double* lbar_hist;
+  float* lam;              // L_k [k][global group]
+  float* lbar;             // lbar_k
   double* logZ;            // per track, accumulated
   double* dlam;            // per global group: the reverse sweep's seed at the last step
-  const float* seed;       // per track
+  double* dlam1;           // the sweep's next accumulator, cleared at step 0
+  double* grad;            // gradient accumulators, cleared at step 0
+  const float* seed;       // per track, or nullptr: seed0
+  float seed0;
   int last;
 };
 
 struct AdjointArgs {
   const TrackParams* trk;
   const int4* tiles;
-  int n_tiles;
   const uint32_t* parent;
   int history;
   int k;
-  const float4* pv;        // X_k
-  const float* In;
-  const float* ypad;
-  const double* lbar_prev; // lbar_{k-1} (k >= 1)
-  const double* lam_k;     // L_k
+  int last;                // 1: the last step (no state adjoint from later steps)
+  int n_tracks, G_total;
+  const float4* dl_pv;     // of step k, as the replay left them
+  const float* dl_b;
+  const float* dl_lw;
+  const float* lam_k;      // L_k
   const double* dlam_k;    // dL_k
   double* D;               // dL_{k-1} accumulator per global group
+  double* dlam_clear;      // the accumulator of the step before, cleared here
   float4* Cc_pv;           // state adjoint of X_k (read and cleared)
   float* Cc_I;
   float4* Cp_pv;           // state adjoint of X_{k-1} (accumulated)
   float* Cp_I;
-  double* grad;            // per track x 5
+  double* grad;            // gradient accumulators
 };
 
-cudaError_t launch_replay(const ReplayArgs& a, int R, int grid, cudaStream_t s);
-cudaError_t launch_replay_groups(const ReplayGroupArgs& a, int n_tracks, int max_G, cudaStream_t s);
-cudaError_t launch_adjoint(const AdjointArgs& a, int R, int grid, cudaStream_t s);
-cudaError_t launch_adjoint_groups(double* dlam, double* D, int G_total, cudaStream_t s);
+// replay and adjoint: one CTA per propagate tile
+cudaError_t launch_replay(const ReplayArgs& a, int R, int n_tiles, bool pdl, cudaStream_t s);
+cudaError_t launch_replay_groups(const ReplayGroupArgs& a, int n_tracks, int max_G, bool pdl, cudaStream_t s);
+cudaError_t launch_adjoint(const AdjointArgs& a, int n_tiles, bool pdl, cudaStream_t s);
 cudaError_t launch_grad_out(const double* g, const double* lz, float* out, double* lz_out, int n, cudaStream_t s);
 // parents (T x n_total, row k = step k) into the replay's ancestry record;
 // out-of-range indices are counted in *bad (not read or written past)
