@@ -204,10 +204,11 @@ __device__ __noinline__ float loglik_grad_frame(const PixelSource& px, int u, in
 // One CTA per tile; the box of the tile's patches is staged in shared memory
 // twice (the copy shifted by one float makes every patch row a row of aligned
 // pairs), a tile whose patches do not fit reads the frame through L1.  Bound
-// by FP32 issue.  Gradient of log Z, 16 x 65536 particles, 20 frames: 7.45 ms
-// with scalar L1 reads in two passes, 5.51 ms with this one.
+// by FP32 issue (the patch pass is ~450 instructions a particle) and the
+// latency of the gathers before it: a million particles take 56 us with four
+// CTAs an SM (64 registers, a few spilled), 59 us with three.
 template <int R>
-__global__ void __launch_bounds__(K1_THREADS, 3) k_replay(ReplayArgs a) {
+__global__ void __launch_bounds__(K1_THREADS, 4) k_replay(ReplayArgs a) {
   constexpr int D = 2 * R + 1, PAD = 2 * R + 1, NW = K1_THREADS / 32;
   __shared__ __align__(16) float s_roi[2][ROI_FLOATS + 4];
   __shared__ int s_box[NW][4];
@@ -328,7 +329,10 @@ __global__ void __launch_bounds__(K1_THREADS, 3) k_replay(ReplayArgs a) {
       l = frame_model ? loglik_grad<R, true>(rows, P.H, P.W, s[q].x, s[q].y, I[q], P, d)
                       : loglik_grad<R, false>(rows, P.H, P.W, s[q].x, s[q].y, I[q], P, d);
     } else {
-      l = loglik_grad_frame<R>(px, pu[q], pv[q], s[q], I[q], P, d);
+      float df[5];
+      l = loglik_grad_frame<R>(px, pu[q], pv[q], s[q], I[q], P, df);
+#pragma unroll
+      for (int x = 0; x < 5; ++x) d[x] = df[x];
     }
     const float lb = k >= 1 ? a.lbar_prev[P.group_off + o[q]] : -log_G;
     const float lw = lb - log_Np + l;
@@ -378,6 +382,7 @@ __global__ void __launch_bounds__(RG_GROUP_THREADS) k_replay_groups(ReplayGroupA
   const int G = P.G;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)blockDim.x >> 5;
   __shared__ double s_lam[MAX_G];
+  __shared__ float s_lamf[MAX_G], s_f[32];
   __shared__ double s_d[32];
   __shared__ double s_lc;
   // L_k,m = LSE over the group's slots, from its tiles' (max, sum exp): a
@@ -394,25 +399,35 @@ __global__ void __launch_bounds__(RG_GROUP_THREADS) k_replay_groups(ReplayGroupA
         if (ms.x > -INFINITY) S = fmaf(ms.y, expf(ms.x - M), S);
       }
     S = warp_sum(S);
-    if (lane == 0) s_lam[m] = (M > -INFINITY && S > 0.0f) ? (double)M + log((double)S) : -INFINITY;
+    if (lane == 0) {
+      const double l = (M > -INFINITY && S > 0.0f) ? (double)M + log((double)S) : -INFINITY;
+      s_lam[m] = l;
+      s_lamf[m] = (float)l;
+    }
   }
   __syncthreads();
-  double mx = -INFINITY;
-  for (int m = threadIdx.x; m < G; m += blockDim.x) mx = fmax(mx, s_lam[m]);
-  mx = warp_max_d(mx);
-  if (lane == 0) s_d[warp] = mx;
+  // log c_k = LSE over the groups: the maximum in FP32 (any value near it
+  // serves as the scale), FP64 by the warps that hold groups only -- an FP64
+  // instruction holds the SM's one pipe for 19 cycles
+  float mf = -INFINITY;
+  for (int m = threadIdx.x; m < G; m += blockDim.x) mf = fmaxf(mf, s_lamf[m]);
+  mf = warp_max(mf);
+  if (lane == 0) s_f[warp] = mf;
   __syncthreads();
-  mx = -INFINITY;
-  for (int w = 0; w < nw; ++w) mx = fmax(mx, s_d[w]);
-  __syncthreads();
-  double e = 0.0;
-  for (int m = threadIdx.x; m < G; m += blockDim.x) e += s_lam[m] > -INFINITY ? exp(s_lam[m] - mx) : 0.0;
-  e = warp_sum_d(e);
-  if (lane == 0) s_d[warp] = e;
+  const int nwa = nw < (G + 31) / 32 ? nw : (G + 31) / 32;
+  mf = -INFINITY;
+  for (int w = 0; w < nwa; ++w) mf = fmaxf(mf, s_f[w]);
+  const double mx = (double)mf;
+  if (warp < nwa) {
+    double e = 0.0;
+    for (int m = threadIdx.x; m < G; m += blockDim.x) e += s_lam[m] > -INFINITY ? exp(s_lam[m] - mx) : 0.0;
+    e = warp_sum_d(e);
+    if (lane == 0) s_d[warp] = e;
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
     double tot = 0.0;
-    for (int w = 0; w < nw; ++w) tot += s_d[w];
+    for (int w = 0; w < nwa; ++w) tot += s_d[w];
     s_lc = mx + log(tot);
     a.logZ[t] = (a.k > 0 ? a.logZ[t] : 0.0) + s_lc;
   }
@@ -481,18 +496,16 @@ __global__ void __launch_bounds__(K1_THREADS, 4) k_adjoint(AdjointArgs a) {
     cI[q] = 0.0f;
     c[q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (jj < td.w) {
-      const float4 d = a.dl_pv[i];
-      const float db = a.dl_b[i], lw = a.dl_lw[i];
+      const float4 d = __ldcs(&a.dl_pv[i]);
+      const float db = __ldcs(&a.dl_b[i]), lw = __ldcs(&a.dl_lw[i]);
       if (!a.last) {
-        c[q] = a.Cc_pv[i];
-        cI[q] = a.Cc_I[i];
+        c[q] = __ldcs(&a.Cc_pv[i]);
+        cI[q] = __ldcs(&a.Cc_I[i]);
       }
       if (k >= 1) {
         par[q] = par_t[il];
         o[q] = (int)fastdiv(par[q], P.m_Np);  // origin group
       }
-      a.Cc_pv[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      a.Cc_I[i] = 0.0f;
       const float wbar = (lw == lw && lw - lam > -87.0f) ? __expf(lw - lam) : 0.0f;
       dlw[q] = dlam * wbar;
       c[q].x = fmaf(dlw[q], d.x, c[q].x);
@@ -557,6 +570,18 @@ __global__ void __launch_bounds__(K1_THREADS, 4) k_adjoint(AdjointArgs a) {
   const float x = warp_reduce8(v, lane, slot);
   if ((lane & 3) == 0) s_red[warp][slot] = x;
   if (lane == 0) s_other[warp] = other;
+  // the adjoints read above make way for the step before last.  Cleared only
+  // now: a store into a line whose load is in flight holds up the load unit
+  // (a million particles: 137 us with the stores behind the loads, 27 us here)
+#pragma unroll
+  for (int q = 0; q < K1_PPT; ++q) {
+    const int jj = threadIdx.x + q * K1_THREADS;
+    const long long i = P.part_off + (long long)g * Np + td.z + jj;
+    if (jj < td.w) {
+      a.Cc_pv[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      a.Cc_I[i] = 0.0f;
+    }
+  }
   __syncthreads();
   if (warp == 0) {
     if (lane < 6) {
