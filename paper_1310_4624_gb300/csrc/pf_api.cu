@@ -866,7 +866,7 @@ pf_status pf_init(const pf_track_config* cfg, int32_t n_tracks, int32_t history,
 
   InitArgs ia{h->trk, h->tiles, h->n_tiles, h->N_total, user_state, h->pv[1], h->In[1]};
   if ((e = launch_init(ia, h->k1_grid, s)) != cudaSuccess) { pf_destroy(h); return cuda_fail(nullptr, e, "k_init"); }
-  if ((e = launch_global(global_args(h, 0), n_tracks, s)) != cudaSuccess) {
+  if ((e = launch_global(global_args(h, 0), n_tracks, h->pdl, s)) != cudaSuccess) {
     pf_destroy(h);
     return cuda_fail(nullptr, e, "k_global");
   }
@@ -1434,18 +1434,18 @@ pf_status pf_reset(pf_handle* h, void* stream) {
   if (!h) return fail(nullptr, PF_ERR_ARG, "handle is NULL");
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e;
-  if ((e = cudaMemsetAsync(h->ds, 0, sizeof(DevState), s)) ||
-      (e = cudaMemsetAsync(h->ts, 0, sizeof(TrackState) * h->n_tracks, s)) ||
-      (e = cudaMemsetAsync(h->gs, 0, sizeof(GroupState) * h->G_total, s)) ||
-      (e = cudaMemsetAsync(h->tile_ctr, 0, sizeof(int), s)) ||
-      (e = cudaMemsetAsync(h->fsync, 0, sizeof(unsigned int) * FusedSync{h->G_total}.count(), s)) ||
-      (e = cudaMemsetAsync(h->rq, 0, sizeof(unsigned int) * 4 * (size_t)h->n_chunks, s)))
-    return cuda_fail(h, e, "pf_reset");
-  InitArgs ia{h->trk, h->tiles, h->n_tiles, h->N_total, nullptr, h->pv[1], h->In[1]};
   for (int t = 0; t < h->n_tracks; ++t)
     if (h->cfg[t].init_kind == PF_INIT_USER) return fail(h, PF_ERR_STATE, "pf_reset cannot redraw a user population");
+  InitArgs ia{h->trk, h->tiles, h->n_tiles, h->N_total, nullptr, h->pv[1], h->In[1]};
+  static_assert(sizeof(DevState) % 4 == 0 && sizeof(TrackState) % 4 == 0 && sizeof(GroupState) % 4 == 0, "whole words");
+  ia.clear[0] = {(uint32_t*)h->ds, (long long)(sizeof(DevState) / 4)};
+  ia.clear[1] = {(uint32_t*)h->ts, (long long)(sizeof(TrackState) / 4) * h->n_tracks};
+  ia.clear[2] = {(uint32_t*)h->gs, (long long)(sizeof(GroupState) / 4) * h->G_total};
+  ia.clear[3] = {(uint32_t*)h->tile_ctr, 1};
+  ia.clear[4] = {(uint32_t*)h->fsync, (long long)FusedSync{h->G_total}.count()};
+  ia.clear[5] = {(uint32_t*)h->rq, 4ll * h->n_chunks};
   if ((e = launch_init(ia, h->k1_grid, s)) != cudaSuccess) return cuda_fail(h, e, "k_init");
-  if ((e = launch_global(global_args(h, 0), h->n_tracks, s)) != cudaSuccess) return cuda_fail(h, e, "k_global");
+  if ((e = launch_global(global_args(h, 0), h->n_tracks, h->pdl, s)) != cudaSuccess) return cuda_fail(h, e, "k_global");
   h->steps_run = 0;
   h->finish_pending = false;
   h->failed = 0;

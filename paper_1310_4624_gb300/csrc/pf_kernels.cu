@@ -45,8 +45,15 @@ namespace pf {
 
 // ========================================================= initial population
 // Initial population (Sec. V tracking / information-sharing modes), drawn
-// from Philox stream INIT into the buffer step 0 reads.
-__global__ void __launch_bounds__(K1_THREADS) k_init(InitArgs a) {
+// from Philox stream INIT into the buffer step 0 reads; a restart's counters
+// and states are cleared by the same launch, which a memset each took before
+// it (a restart and two frames of 4096 particles: 123 -> 120 us).
+__global__ void __launch_bounds__(K1_THREADS) k_init(const __grid_constant__ InitArgs a) {
+#pragma unroll
+  for (int c = 0; c < 6; ++c)
+    for (long long i = (long long)blockIdx.x * K1_THREADS + threadIdx.x; i < a.clear[c].n;
+         i += (long long)gridDim.x * K1_THREADS)
+      a.clear[c].p[i] = 0u;
   for (int e = blockIdx.x * K1_PPT; e < a.n_tiles * K1_PPT; e += gridDim.x * K1_PPT) {
    for (int q = 0; q < K1_PPT; ++q) {
     const int4 td = a.tiles[(e + q) / K1_PPT];
@@ -60,21 +67,24 @@ __global__ void __launch_bounds__(K1_THREADS) k_init(InitArgs a) {
 #pragma unroll
       for (int d = 0; d < 5; ++d) s[d] = a.user[(long long)d * a.n_total + i];
     } else {
-      const uint4 w0 = philox(P.key0, P.key1, make_uint4(j, g, 0u, P.tag | (ST_INIT << 4) | 0u));
-      const uint4 w1 = philox(P.key0, P.key1, make_uint4(j, g, 0u, P.tag | (ST_INIT << 4) | 1u));
-      const float u[5] = {u01(w0.x), u01(w0.y), u01(w0.z), u01(w0.w), u01(w1.x)};
+      auto draw = [&](uint32_t call) {
+        return philox(P.key0, P.key1, make_uint4(j, g, 0u, P.tag | (ST_INIT << 4) | call));
+      };
       if (P.init_kind == INIT_POINT || (P.init_kind == INIT_SHARING && g == 0)) {
 #pragma unroll
         for (int d = 0; d < 5; ++d) s[d] = P.init_state[d];
         if (P.init_kind == INIT_SHARING) {
           // position uniform in the disc: r = R sqrt(u0), angle 2 pi u1
-          const float r = P.init_radius * sqrtf(u[0]);
+          const uint4 w0 = draw(0u);
+          const float r = P.init_radius * sqrtf(u01(w0.x));
           float sn, cs;
-          sincospif(fmaf(2.0f, u[1], -1.0f), &sn, &cs);  // angle 2 pi u1 - pi
+          sincospif(fmaf(2.0f, u01(w0.y), -1.0f), &sn, &cs);  // angle 2 pi u1 - pi
           s[0] = P.init_state[0] - r * cs;
           s[1] = P.init_state[1] - r * sn;
         }
       } else {
+        const uint4 w0 = draw(0u), w1 = draw(1u);
+        const float u[5] = {u01(w0.x), u01(w0.y), u01(w0.z), u01(w0.w), u01(w1.x)};
 #pragma unroll
         for (int d = 0; d < 5; ++d) s[d] = fmaf(P.init_hi[d] - P.init_lo[d], u[d], P.init_lo[d]);
       }
@@ -572,6 +582,7 @@ __device__ void finish_step(const GlobalArgs& a, int t, GlobalScratch& sc) {
 // the same step runs as the tail of the resampler.
 __global__ void __launch_bounds__(GL_THREADS) k_global(GlobalArgs a) {
   __shared__ GlobalScratch sc;
+  grid_dep_wait();
   global_step<GL_THREADS>(a, blockIdx.x, sc);
 }
 
@@ -2998,9 +3009,8 @@ cudaError_t launch_resample_groups(const ResampleArgs& a0, const GroupClasses& g
   return cudaSuccess;
 }
 
-cudaError_t launch_global(const GlobalArgs& a, int n_tracks, cudaStream_t s) {
-  k_global<<<n_tracks, GL_THREADS, 0, s>>>(a);
-  return cudaGetLastError();
+cudaError_t launch_global(const GlobalArgs& a, int n_tracks, bool pdl, cudaStream_t s) {
+  return launch_ex(k_global, dim3(n_tracks), dim3(GL_THREADS), 0, pdl, s, a);
 }
 
 cudaError_t launch_finish(const GlobalArgs& a, int n_tracks, cudaStream_t s) {

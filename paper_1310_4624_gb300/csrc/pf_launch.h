@@ -16,6 +16,8 @@ struct InitArgs {
   const float* user;   // 5 x n_total SoA or nullptr
   float4* pv;          // buffer read by step 0
   float* In;
+  // words to clear in the same launch (pf_reset: what a memset each took)
+  struct { uint32_t* p; long long n; } clear[6] = {};
 };
 
 struct FrameArgs {
@@ -268,7 +270,7 @@ cudaError_t launch_resample(const ResampleArgs& a, int n_groups, int cluster, bo
 // The resampling of many groups, one CTA (or one warp) per group, a launch
 // per class of group size.
 cudaError_t launch_resample_groups(const ResampleArgs& a, const GroupClasses& gc, bool pdl, cudaStream_t s);
-cudaError_t launch_global(const GlobalArgs& a, int n_tracks, cudaStream_t s);
+cudaError_t launch_global(const GlobalArgs& a, int n_tracks, bool pdl, cudaStream_t s);
 cudaError_t launch_finish(const GlobalArgs& a, int n_tracks, cudaStream_t s);
 // launch_finish, then x^ (n_tracks x 5) and log Z (n_tracks) stored through
 // device addresses of page-locked host memory (either may be null); pdl:
