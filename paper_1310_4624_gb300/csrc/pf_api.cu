@@ -498,14 +498,16 @@ K1Args k1_args(const pf_handle* h) {
 }
 
 // A single-track step reads the caller's frame directly (no frame
-// preparation kernel) when a TMA descriptor can describe it: the driver
+// preparation kernel): by TMA when a descriptor can describe it (the driver
 // entry point is available, the frame starts on 16 bytes, its rows are a
-// multiple of 16 bytes and it holds at least one staging box.  Sets the
-// descriptor in `a` and returns true, else leaves `a` unchanged.
+// multiple of 16 bytes and it holds at least one staging box), else by plain
+// loads.  Returns false, and leaves `a` unchanged, for several tracks.
 bool raw_frame_map(const pf_handle* h, const float* frame, K1Args* a) {
-  if (h->n_tracks != 1 || !h->encode || !frame) return false;
+  if (h->n_tracks != 1 || !frame) return false;
   const pf_track_config& c = h->cfg[0];
-  if (((uintptr_t)frame & 15) != 0 || (c.W % 4) != 0 || c.W < ROI_W || c.H < ROI_BOX_H) return false;
+  a->raw_frame = RAW_FRAME_LOADS;
+  a->zraw = frame;
+  if (!h->encode || ((uintptr_t)frame & 15) != 0 || (c.W % 4) != 0 || c.W < ROI_W || c.H < ROI_BOX_H) return true;
   cuuint64_t dims[2] = {(cuuint64_t)c.W, (cuuint64_t)c.H};
   cuuint64_t strides[1] = {(cuuint64_t)c.W * sizeof(float)};
   cuuint32_t box[2] = {(cuuint32_t)ROI_W, (cuuint32_t)ROI_BOX_H};
@@ -514,9 +516,8 @@ bool raw_frame_map(const pf_handle* h, const float* frame, K1Args* a) {
   const CUresult r = ((PFN_cuTensorMapEncodeTiled_v12000)h->encode)(
       &m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, (void*)frame, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
       CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) return false;
-  a->raw_frame = 1;
-  a->zraw = frame;
+  if (r != CUDA_SUCCESS) return true;
+  a->raw_frame = RAW_FRAME_TMA;
   a->zmap = m;
   return true;
 }
@@ -913,7 +914,7 @@ pf_status pf_step(pf_handle* h, const float* const* frames, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e;
   K1Args k1 = k1_args(h);
-  if (h->variants || !raw_frame_map(h, frames[0], &k1)) {
+  if (!raw_frame_map(h, frames[0], &k1)) {
     if ((e = mark(h, PF_KERNEL_FRAME_PREP, s)) != cudaSuccess) return cuda_fail(h, e, "profile event");
     if ((e = prep_frames(h, frames, s)) != cudaSuccess) return cuda_fail(h, e, "k_frame_prep");
     if ((e = mark(h, PF_KERNEL_FRAME_PREP, s)) != cudaSuccess) return cuda_fail(h, e, "profile event");

@@ -913,8 +913,12 @@ static_assert(ROI_SMEM <= FUSED_SMEM && sizeof(GlobalScratch) <= FUSED_SMEM, "fu
 
 // Propagate + weight: tiles of K1_TILE = K1_PPT x K1_THREADS slots of one
 // group, K1_PPT particles per thread.  Each tile stages the bounding box of
-// its particles' patches (at most ROI_W x ROI_ROWS floats) in shared memory
-// by TMA; tiles whose patches do not fit read the frame through L1.
+// its particles' patches (at most ROI_W x ROI_ROWS floats) in shared memory,
+// by TMA, or by plain loads from a frame that no TMA descriptor can describe
+// (rows off the 16-byte grid: padding it first took a launch a step, 7 us of
+// 32 on 33 x 3001 particles, 6 of 37 on 95 x 1269 with method variants, whose
+// instance spills a few registers for it); tiles whose patches do not fit read the frame
+// through L1.
 // Leading blocks draw the next step's rings and exchange offsets and finish
 // the previous step.
 // SINGLE: one track, whose parameters come from the kernel's constant
@@ -1148,14 +1152,36 @@ __global__ void __launch_bounds__(K1_THREADS, K1_MIN_BLOCKS) k_propagate_weight(
       vmin = min(vmin, s_box[w][2]);
       vmax = max(vmax, s_box[w][3]);
     }
-    // raw frame: the box's left edge on a 4-float boundary of the frame
-    // (a TMA requirement), in padded coordinates
-    const bool raw = SINGLE && a.raw_frame;
-    const int u0 = raw ? (((umin - PAD) & ~3) + PAD) : (umin & ~3);
+    // raw frame by TMA: the box's left edge on a 4-float boundary of the
+    // frame (a TMA requirement), in padded coordinates
+    const bool raw = (SINGLE || VARIANTS) && a.raw_frame;
+    const bool plain = raw && a.raw_frame == RAW_FRAME_LOADS;  // (any box: no copy engine, no alignment)
+    const int u0 = plain ? umin : raw ? (((umin - PAD) & ~3) + PAD) : (umin & ~3);
     const int nbox = (vmax + D - vmin + ROI_BOX_H - 1) / ROI_BOX_H;
     const bool staged = (raw || a.tmaps != nullptr) && (umax + D - u0) <= ROI_W && nbox <= ROI_MAX_BOXES;
 
-    if (staged) {
+    if (staged && plain) {
+      // y = z - b inside the frame, 0 outside, and the shifted copy: eight
+      // threads a row, 32 rows a pass
+      const int cols = umax + D - u0, nrows = vmax + D - vmin, c0 = threadIdx.x & 7;
+      float* roi = &s_roi[0][0];
+      float* roiB = &s_roi[1][0];
+      for (int r = threadIdx.x >> 3; r < nrows; r += K1_THREADS / 8) {
+        const int yy = vmin - PAD + r;
+        const bool rin = (unsigned)yy < (unsigned)P.H;
+        const float* __restrict__ zr = a.zraw + (long long)yy * P.W;
+#pragma unroll
+        for (int i = 0; i < ROI_W / 8; ++i) {
+          const int c = c0 + 8 * i, xx = u0 - PAD + c;
+          if (c < cols) {
+            const float y = rin && (unsigned)xx < (unsigned)P.W ? __fsub_rn(__ldg(zr + xx), P.bg) : 0.0f;
+            roi[r * ROI_W + c] = y;
+            if (r * ROI_W + c > 0) roiB[r * ROI_W + c - 1] = y;
+          }
+        }
+      }
+      __syncthreads();
+    } else if (staged) {
       if (threadIdx.x == 0 && !a.test_withhold_copy) {
         fence_proxy_async();  // earlier generic reads of s_roi before the async-proxy writes
         mbar_expect_tx(&s_bar, (uint32_t)(nbox * ROI_W * ROI_BOX_H * sizeof(float)));
@@ -2928,7 +2954,7 @@ cudaError_t fused_occupancy(int R, int* blocks_per_sm) {
 
 // Instances: one track, several tracks, and tracks that use a method
 // variant (groups that carry their particles' own weights under Alg. 1's
-// resampling test, or keyed send sets; any track count, frames prepared).
+// resampling test, or keyed send sets; any track count).
 template <int R>
 static cudaError_t launch_propagate_r(const K1Args& a, dim3 g, bool pdl, cudaStream_t s) {
   if (a.variants) return launch_propagate_rs<R, false, true>(a, g, pdl, s);

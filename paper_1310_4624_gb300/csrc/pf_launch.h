@@ -8,6 +8,8 @@
 
 namespace pf {
 
+constexpr int RAW_FRAME_TMA = 1, RAW_FRAME_LOADS = 2;  // K1Args::raw_frame
+
 struct InitArgs {
   const TrackParams* trk;
   const int4* tiles;   // (track, group, first slot, count) per tile
@@ -80,8 +82,9 @@ struct K1Args {
   int n_tracks;
   TrackParams p0;            // n_tracks == 1: a copy of trk[0]
   // n_tracks == 1 and raw_frame: the step reads the caller's frame (W x H
-  // float32, row pitch W) directly, through zmap (TMA, zero fill outside)
-  // or zraw, instead of the padded frame y = z - b.
+  // float32, row pitch W) directly, staged through zmap (RAW_FRAME_TMA, zero
+  // fill outside) or by loads from zraw (RAW_FRAME_LOADS), instead of the
+  // padded frame y = z - b.
   int raw_frame;
   const float* zraw;
   int test_withhold_copy;    // failure-detection test: issue no staging copy, so the bounded wait runs out
