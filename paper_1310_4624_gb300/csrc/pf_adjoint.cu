@@ -207,8 +207,9 @@ __device__ __noinline__ float loglik_grad_frame(const PixelSource& px, int u, in
 // by FP32 issue (the patch pass is ~450 instructions a particle) and the
 // latency of the gathers before it: a million particles take 56 us with four
 // CTAs an SM (64 registers, a few spilled), 59 us with three.
-template <int R>
-__global__ void __launch_bounds__(K1_THREADS, 4) k_replay(ReplayArgs a) {
+// SINGLE: one track, its parameters and round keys in the constant bank.
+template <int R, bool SINGLE>
+__global__ void __launch_bounds__(K1_THREADS, 4) k_replay(const __grid_constant__ ReplayArgs a) {
   constexpr int D = 2 * R + 1, PAD = 2 * R + 1, NW = K1_THREADS / 32;
   __shared__ __align__(16) float s_roi[2][ROI_FLOATS + 4];
   __shared__ int s_box[NW][4];
@@ -218,7 +219,7 @@ __global__ void __launch_bounds__(K1_THREADS, 4) k_replay(ReplayArgs a) {
   grid_dep_wait();
   grid_dep_launch();
   const int4 td = a.tiles[tile];
-  const TrackParams& P = a.trk[td.x];
+  const TrackParams& P = SINGLE ? a.p0 : a.trk[td.x];
   const int g = td.y, Np = P.Np;
   const long long Nt = (long long)P.G * Np;
   const uint32_t* __restrict__ par_t = a.parent + P.parent_off + (long long)(k % a.history) * Nt;
@@ -242,7 +243,10 @@ __global__ void __launch_bounds__(K1_THREADS, 4) k_replay(ReplayArgs a) {
       I[q] = a.I_in[P.part_off + par];
       uint4 w0 = make_uint4(j, g, k, P.tag | (ST_PROP << 4) | 0u);
       uint4 w1 = make_uint4(j, g, k, P.tag | (ST_PROP << 4) | 1u);
-      philox2(P.key0, P.key1, w0, w1);
+      if constexpr (SINGLE)
+        philox2_rk(P.rk, w0, w1);
+      else
+        philox2(P.key0, P.key1, w0, w1);
       float e0, e1, e2, e3, e4, e5;
       box_muller_fast(w0.x, w0.y, e0, e1);
       box_muller_fast(w0.z, w0.w, e2, e3);
@@ -464,7 +468,8 @@ __device__ __forceinline__ void red_add_v4(float4* p, float x, float y, float z,
 // to the origin group per tile, gradient terms to one of GRAD_COPIES
 // accumulators, so that no address takes an atomic per warp.  Bound by the
 // 90 bytes a particle it moves and the step's normals it draws again.
-__global__ void __launch_bounds__(K1_THREADS, 4) k_adjoint(AdjointArgs a) {
+template <bool SINGLE>
+__global__ void __launch_bounds__(K1_THREADS, 4) k_adjoint(const __grid_constant__ AdjointArgs a) {
   constexpr int NW = K1_THREADS / 32;
   constexpr unsigned FULL = 0xffffffffu;
   const int k = a.k;
@@ -476,7 +481,7 @@ __global__ void __launch_bounds__(K1_THREADS, 4) k_adjoint(AdjointArgs a) {
   for (int m = blockIdx.x * K1_THREADS + threadIdx.x; m < a.G_total; m += gridDim.x * K1_THREADS)
     a.dlam_clear[m] = 0.0;
   const int4 td = a.tiles[blockIdx.x];
-  const TrackParams& P = a.trk[td.x];
+  const TrackParams& P = SINGLE ? a.p0 : a.trk[td.x];
   const int g = td.y, Np = P.Np;
   const uint32_t* __restrict__ par_t =
       a.parent + P.parent_off + (long long)(k % a.history) * ((long long)P.G * Np);
@@ -534,7 +539,10 @@ __global__ void __launch_bounds__(K1_THREADS, 4) k_adjoint(AdjointArgs a) {
         const int j = td.z + jj;
         uint4 w0 = make_uint4(j, g, k, P.tag | (ST_PROP << 4) | 0u);
         uint4 w1 = make_uint4(j, g, k, P.tag | (ST_PROP << 4) | 1u);
-        philox2(P.key0, P.key1, w0, w1);
+        if constexpr (SINGLE)
+          philox2_rk(P.rk, w0, w1);
+        else
+          philox2(P.key0, P.key1, w0, w1);
         float e0, e1, e2, e3;
         box_muller_fast(w0.x, w0.y, e0, e1);
         box_muller_fast(w0.z, w0.w, e2, e3);
@@ -638,15 +646,21 @@ static cudaError_t launch_pdl(void (*kernel)(Params...), int grid, int block, bo
   return cudaLaunchKernelEx(&cfg, kernel, arg);
 }
 
+template <int R>
+static cudaError_t launch_replay_r(const ReplayArgs& a, int n_tiles, bool pdl, cudaStream_t s) {
+  if (a.n_tracks == 1) return launch_pdl(k_replay<R, true>, n_tiles, K1_THREADS, pdl, s, a);
+  return launch_pdl(k_replay<R, false>, n_tiles, K1_THREADS, pdl, s, a);
+}
+
 cudaError_t launch_replay(const ReplayArgs& a, int R, int n_tiles, bool pdl, cudaStream_t s) {
   switch (R) {
-    case 1: return launch_pdl(k_replay<1>, n_tiles, K1_THREADS, pdl, s, a);
-    case 2: return launch_pdl(k_replay<2>, n_tiles, K1_THREADS, pdl, s, a);
-    case 3: return launch_pdl(k_replay<3>, n_tiles, K1_THREADS, pdl, s, a);
-    case 4: return launch_pdl(k_replay<4>, n_tiles, K1_THREADS, pdl, s, a);
-    case 5: return launch_pdl(k_replay<5>, n_tiles, K1_THREADS, pdl, s, a);
-    case 6: return launch_pdl(k_replay<6>, n_tiles, K1_THREADS, pdl, s, a);
-    case 7: return launch_pdl(k_replay<7>, n_tiles, K1_THREADS, pdl, s, a);
+    case 1: return launch_replay_r<1>(a, n_tiles, pdl, s);
+    case 2: return launch_replay_r<2>(a, n_tiles, pdl, s);
+    case 3: return launch_replay_r<3>(a, n_tiles, pdl, s);
+    case 4: return launch_replay_r<4>(a, n_tiles, pdl, s);
+    case 5: return launch_replay_r<5>(a, n_tiles, pdl, s);
+    case 6: return launch_replay_r<6>(a, n_tiles, pdl, s);
+    case 7: return launch_replay_r<7>(a, n_tiles, pdl, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -657,7 +671,8 @@ cudaError_t launch_replay_groups(const ReplayGroupArgs& a, int n_tracks, int max
 }
 
 cudaError_t launch_adjoint(const AdjointArgs& a, int n_tiles, bool pdl, cudaStream_t s) {
-  return launch_pdl(k_adjoint, n_tiles, K1_THREADS, pdl, s, a);
+  if (a.n_tracks == 1) return launch_pdl(k_adjoint<true>, n_tiles, K1_THREADS, pdl, s, a);
+  return launch_pdl(k_adjoint<false>, n_tiles, K1_THREADS, pdl, s, a);
 }
 
 // Caller-supplied ancestry for the replay (pf_set_replay): for steps k = 1 ..

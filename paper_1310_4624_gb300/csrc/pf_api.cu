@@ -1544,6 +1544,8 @@ pf_status pf_backward(pf_handle* h, const float* const* frames_host, int32_t T, 
     ra.ypad = h->ypad;
     ra.lbar_prev = k >= 1 ? h->lbar + (long long)(k - 1) * G : nullptr;
     ra.tile_part = h->tile_part;
+    ra.n_tracks = h->n_tracks;
+    ra.p0 = h->tp[0];
     if ((e = launch_replay(ra, h->R, h->n_tiles, h->pdl, s)) != cudaSuccess) return cuda_fail(h, e, "k_replay");
     if (!groups) return PF_OK;
     const ReplayGroupArgs rg{h->trk,  h->gd,    h->tile_part, k,
@@ -1585,6 +1587,7 @@ pf_status pf_backward(pf_handle* h, const float* const* frames_host, int32_t T, 
       aa.Cp_pv = h->ca_pv[(k + 1) & 1];
       aa.Cp_I = h->ca_I[(k + 1) & 1];
       aa.grad = h->grad;
+      aa.p0 = h->tp[0];
       if ((e = launch_adjoint(aa, h->n_tiles, h->pdl, s)) != cudaSuccess) return cuda_fail(h, e, "k_adjoint");
     }
   }

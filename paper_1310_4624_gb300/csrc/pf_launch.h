@@ -203,6 +203,8 @@ struct ReplayArgs {
   const float* ypad;
   const float* lbar_prev;  // lbar_{k-1} per global group (k >= 1)
   float* tile_part;
+  int n_tracks;
+  TrackParams p0;          // n_tracks == 1: a copy of trk[0]
 };
 
 struct ReplayGroupArgs {
@@ -242,6 +244,7 @@ struct AdjointArgs {
   float4* Cp_pv;           // state adjoint of X_{k-1} (accumulated)
   float* Cp_I;
   double* grad;            // gradient accumulators
+  TrackParams p0;          // n_tracks == 1: a copy of trk[0]
 };
 
 // replay and adjoint: one CTA per propagate tile
