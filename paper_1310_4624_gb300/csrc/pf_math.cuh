@@ -35,22 +35,9 @@ __device__ __forceinline__ float warp_sum(float v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-// Sum over the lanes of `mask` (every lane of the mask calls it; the
-// result reaches all of them).
-__device__ __forceinline__ float warp_sum_active(unsigned mask, float v) {
-  if (mask == 0xffffffffu) return warp_sum(v);
-  float s = 0.0f;
-  for (unsigned m = mask; m; m &= m - 1) s += __shfl_sync(mask, v, __ffs(m) - 1);
-  return s;
-}
 __device__ __forceinline__ double warp_sum_d(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-__device__ __forceinline__ double warp_max_d(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
 __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
@@ -69,28 +56,6 @@ __device__ __forceinline__ float block_max(float v, float* sh) {
   float r = sh[0];
 #pragma unroll
   for (int w = 1; w < NT / 32; ++w) r = fmaxf(r, sh[w]);
-  __syncthreads();
-  return r;
-}
-template <int NT>
-__device__ __forceinline__ double block_sum_d(double v, double* sh) {
-  v = warp_sum_d(v);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double r = 0.0;
-#pragma unroll
-  for (int w = 0; w < NT / 32; ++w) r += sh[w];
-  __syncthreads();
-  return r;
-}
-template <int NT>
-__device__ __forceinline__ double block_max_d(double v, double* sh) {
-  v = warp_max_d(v);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double r = sh[0];
-#pragma unroll
-  for (int w = 1; w < NT / 32; ++w) r = fmax(r, sh[w]);
   __syncthreads();
   return r;
 }
