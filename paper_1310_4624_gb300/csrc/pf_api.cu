@@ -358,8 +358,14 @@ int num_sms() {
   return sms > 0 ? sms : 1;
 }
 
-int resample_cluster(int Np, int pad) {
-  int c = (Np + pad + RS_SUB - 1) / RS_SUB;
+// CTAs per group: one per sub-chunk, at most 8; 16 (a non-portable cluster)
+// for groups that not even 16 CTAs hold in their registers, while 8 each would
+// leave SMs idle: 320 -> 189 us for one group of 2^20, 128 -> 92 us for four of
+// 2^18.  Groups that fit gain nothing (8 x 100000: 72 and 73 us; 16 x 65536: 61
+// and 64 us).
+int resample_cluster(int G, int Np, int pad) {
+  const int c = (Np + pad + RS_SUB - 1) / RS_SUB;
+  if (c > 32 && 8ll * G < num_sms()) return resample_max_cluster();
   return c < 1 ? 1 : (c > 8 ? 8 : c);
 }
 
@@ -552,7 +558,7 @@ QuantCoeffs resample_coeffs() { return make_qc(); }
 int resample_pad(const float* logw, const uint32_t* anc, int G, int Np) {
   return ((((uintptr_t)logw | (uintptr_t)anc) & 15) || (G > 1 && (Np & 3))) ? 3 : 0;
 }
-int resample_cluster_size(int Np, int pad) { return resample_cluster(Np, pad); }
+int resample_cluster_size(int G, int Np, int pad) { return resample_cluster(G, Np, pad); }
 void set_handleless_error(const char* msg) { g_err = msg; }
 }  // namespace pf
 
@@ -849,7 +855,7 @@ pf_status pf_init(const pf_track_config* cfg, int32_t n_tracks, int32_t history,
     for (int t = 0; t < n_tracks; ++t) maxNp = cfg[t].Np > maxNp ? cfg[t].Np : maxNp;
     h->rs_threads = maxNp <= RS_THREADS_SMALL * RS_ITEMS ? RS_THREADS_SMALL : RS_THREADS;
     if (n_tracks == 1) {
-      h->rs_cluster = resample_cluster(cfg[0].Np, h->rs_pad);
+      h->rs_cluster = resample_cluster(cfg[0].G, cfg[0].Np, h->rs_pad);
       if (h->rs_threads == RS_THREADS_SMALL && maxNp + h->rs_pad > RS_THREADS_SMALL * RS_ITEMS) h->rs_cluster = 2;
     } else {
       const int sub = h->rs_threads * RS_ITEMS;
@@ -1142,7 +1148,7 @@ pf_status pf_autotune(pf_handle* h, const float* const* frames, int32_t* k1_grid
       best_t = 0;
     }
     for (int nt : {RS_THREADS, RS_THREADS_SMALL})
-      for (int c = 1; c <= 8 && e == cudaSuccess; c *= 2) {
+      for (int c = 1; c <= std::max(8, h->rs_cluster) && e == cudaSuccess; c *= 2) {
         const ResampleArgs ra = resample_args(h, 0);
         float ms = 0.0f;
         for (int rep = 0; rep < 2; ++rep)
@@ -1376,7 +1382,7 @@ pf_status pf_resample(const float* logw, const uint32_t* u, int32_t G, int32_t N
   ra.max_np = Np;
   ra.lean = 1;
   ra.pad = resample_pad(logw, anc, G, Np);
-  if ((e = launch_resample(ra, G, resample_cluster(Np, ra.pad), false, s)) != cudaSuccess)
+  if ((e = launch_resample(ra, G, resample_cluster(G, Np, ra.pad), false, s)) != cudaSuccess)
     return cuda_fail(nullptr, e, "k_resample");
   return PF_OK;
 }

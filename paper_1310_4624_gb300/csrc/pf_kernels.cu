@@ -2976,17 +2976,56 @@ cudaError_t launch_propagate(const K1Args& a, int R, int grid, bool pdl, cudaStr
   }
 }
 
+template <int NTR, int ITEMS, bool LEAN>
+constexpr size_t resample_smem() {
+  return LEAN ? RS_MARK_OFF + NTR * ITEMS * sizeof(uint32_t)
+              : pad8(NTR * RS_ITEMS) * sizeof(unsigned long long) + pad8(2 * NTR * RS_ITEMS) * sizeof(uint32_t);
+}
+
+// The instance's shared memory and, for the general one, clusters beyond the
+// portable 8.
+template <int NTR, int ITEMS, bool LEAN, bool EXTRA>
+static cudaError_t resample_attributes() {
+  static std::once_flag once;
+  static cudaError_t err = cudaSuccess;
+  std::call_once(once, [] {
+    err = cudaFuncSetAttribute(k_resample<NTR, ITEMS, LEAN, EXTRA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)resample_smem<NTR, ITEMS, LEAN>());
+    if (err == cudaSuccess && !LEAN)
+      err = cudaFuncSetAttribute(k_resample<NTR, ITEMS, LEAN, EXTRA>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  });
+  return err;
+}
+
+int resample_max_cluster() {
+  static std::once_flag once;
+  static int most = 8;
+  std::call_once(once, [] {
+    if (resample_attributes<RS_THREADS, RS_ITEMS, false, true>() != cudaSuccess) return;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(16);
+    cfg.blockDim = dim3(RS_THREADS);
+    cfg.dynamicSmemBytes = resample_smem<RS_THREADS, RS_ITEMS, false>();
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 16;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_resample<RS_THREADS, RS_ITEMS, false, true>, &cfg) != cudaSuccess)
+      cudaGetLastError();
+    else if (n >= 4)
+      most = 16;
+  });
+  return most;
+}
+
 template <int NTR, int ITEMS, bool LEAN, bool EXTRA>
 static cudaError_t launch_resample_t(const ResampleArgs& a, int n_groups, int cluster, bool pdl, cudaStream_t s) {
-  constexpr size_t smem = LEAN ? RS_MARK_OFF + NTR * ITEMS * sizeof(uint32_t)
-                              : pad8(NTR * RS_ITEMS) * sizeof(unsigned long long) +
-                                    pad8(2 * NTR * RS_ITEMS) * sizeof(uint32_t);
+  constexpr size_t smem = resample_smem<NTR, ITEMS, LEAN>();
   static_assert(sizeof(GlobalScratch) <= smem, "the global step's scratch lives in the resampler's shared memory");
-  static std::once_flag once;
-  static cudaError_t attr_err = cudaSuccess;
-  std::call_once(once, [] {
-    attr_err = cudaFuncSetAttribute(k_resample<NTR, ITEMS, LEAN, EXTRA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  });
+  const cudaError_t attr_err = resample_attributes<NTR, ITEMS, LEAN, EXTRA>();
   if (attr_err != cudaSuccess) return attr_err;
   const int clusters = n_groups + (a.fuse_global == 2 ? 1 : 0);  // the global step's extra cluster
   return launch_ex(k_resample<NTR, ITEMS, LEAN, EXTRA>, dim3((unsigned)(clusters * cluster)), dim3(NTR), cluster, pdl, s, a, smem);

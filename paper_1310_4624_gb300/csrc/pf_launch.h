@@ -273,6 +273,9 @@ cudaError_t fused_occupancy(int R, int* blocks_per_sm);
 // threads: RS_THREADS, or RS_THREADS_SMALL (eight CTAs per SM, for batches of small groups)
 cudaError_t launch_resample(const ResampleArgs& a, int n_groups, int cluster, bool pdl, cudaStream_t s,
                             int threads = RS_THREADS);
+// Largest cluster that the general 512-thread resampler can be launched with:
+// 16 if the device has room for several, else the portable 8.
+int resample_max_cluster();
 // The resampling of many groups, one CTA (or one warp) per group, a launch
 // per class of group size.
 cudaError_t launch_resample_groups(const ResampleArgs& a, const GroupClasses& gc, bool pdl, cudaStream_t s);
@@ -289,7 +292,7 @@ const void* propagate_kernel(int R);
 
 // Host helpers shared by the C-ABI entry points (defined in pf_api.cu).
 QuantCoeffs resample_coeffs();             // weight-code coefficients
-int resample_cluster_size(int Np, int pad);  // resampler cluster size for one group of Np
+int resample_cluster_size(int G, int Np, int pad);  // resampler cluster size for one group of Np
 // ResampleArgs::pad for G groups of Np in a caller's arrays
 int resample_pad(const float* logw, const uint32_t* anc, int G, int Np);
 void set_handleless_error(const char* msg);  // text for pf_last_error(NULL)

@@ -155,7 +155,7 @@ extern "C" pf_status pf_resample_noalloc(const float* logw, const uint32_t* u, i
   ra.max_np = Np;
   ra.lean = 1;
   ra.pad = resample_pad(logw, anc, G, Np);
-  if ((e = launch_resample(ra, G, resample_cluster_size(Np, ra.pad), false, s)) != cudaSuccess)
+  if ((e = launch_resample(ra, G, resample_cluster_size(G, Np, ra.pad), false, s)) != cudaSuccess)
     return fail(PF_ERR_CUDA, std::string("k_resample: ") + cudaGetErrorString(e));
   return PF_OK;
 }
