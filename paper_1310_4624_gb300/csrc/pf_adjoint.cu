@@ -26,6 +26,7 @@
 #include <climits>
 #include <cmath>
 #include <cstdint>
+#include <type_traits>
 
 #include "pf_device.cuh"
 #include "pf_launch.h"
@@ -50,149 +51,108 @@ struct PixelSource {
   }
 };
 
-// Two neighbouring pixels of a patch row: from the staged box (8-byte aligned
-// pairs) or from the frame.
+// A patch's pixels: from the staged box or from the frame.
 struct StagedRows {
   const float* base;
-  __device__ __forceinline__ float2 pair(int b, int p) const {
-    return *reinterpret_cast<const float2*>(base + b * ROI_W + 2 * p);
-  }
   __device__ __forceinline__ float one(int b, int a) const { return base[b * ROI_W + a]; }
 };
 struct FrameRows {
   const PixelSource& px;
   int u, v;
-  __device__ __forceinline__ float2 pair(int b, int p) const {
-    return make_float2(px.at(u + 2 * p, v + b), px.at(u + 2 * p + 1, v + b));
-  }
   __device__ __forceinline__ float one(int b, int a) const { return px.at(u + a, v + b); }
 };
 
-// Log-likelihood (Sec. V model) and its partial derivatives: d[0..4] = dl/dx,
-// dl/dy, dl/dI, dl/dsigma_psf, dl/db.  One pass over the patch, columns 2p and
-// 2p + 1 as one packed FP32 pair.  With r = y - I gx gy per pixel, what the
-// derivatives need of the columns is A_a = sum_b gy_b r_ab (sum r gx gy (u-x)^n
-// = sum_a gx_a (u_a-x)^n A_a, taken once after the rows) and of the rows
-// R_b = sum_a gx_a r_ab, so a pair costs five packed operations (r, r^2, A, R,
-// sum r) where sums by row of r gx, r gx a and r gx a^2 cost eight a pixel.
-// Pixels outside the frame count as background, so only inside pixels depend
-// on b: a patch over the border (rare) sums those in a pass of its own.
-template <int R, bool FRAME, class Rows>
-__device__ __forceinline__ float loglik_grad(const Rows& rows, int H, int W, float x, float y, float I,
+// Log-likelihood (Sec. V model) and its partial derivatives for the
+// adjoint: d[0..4] = dl/dx, dl/dy, dl/dI, dl/dsigma_psf, dl/db.  One pass
+// over the patch with separable row sums: per row v with r = y - I gx gy,
+// R0 = sum r gx, R1 = sum r gx a, R2 = sum r gx a^2 (a the column offset), so
+// that sum r gx (u - x) = R1 + du0 R0 and sum r gx (u - x)^2 = R2 + 2 du0 R1
+// + du0^2 R0 with du0 = cx - R - x.  Pixels outside the frame count as
+// background, so only inside pixels depend on b.
+// The replay's group log-weights come from patch_sum's order of the same
+// pixels; both orders are part of the result's rounding and are kept.
+template <int R, class Rows>
+__device__ __forceinline__ float loglik_grad(const Rows& px, int H, int W, float x, float y, float I,
                                              const TrackParams& P, float (&d)[5]) {
   constexpr int D = 2 * R + 1;
   const float cxf = floorf(x + 0.5f), cyf = floorf(y + 0.5f);
-  const float cc = P.c_psf, kappa = P.kappa;
   float gx[D];
-  gauss_row<R>(cxf, x, cc, kappa, gx);
-  float2 A[R];
-#pragma unroll
-  for (int p = 0; p < R; ++p) A[p] = make_float2(0.0f, 0.0f);
-  float Al = 0.0f;  // column 2R
-  float2 ss = make_float2(0.0f, 0.0f), Sb = ss, Y2 = ss, Y1 = ss;
-  float Sy = 0.0f, Sy2 = 0.0f;
-  const float dy = cyf - y;
-  auto row = [&](int b, float gy) {
-    const float nI = -(I * gy);
-    const float2 nI2 = make_float2(nI, nI), gy2 = make_float2(gy, gy);
-    float2 R0 = make_float2(0.0f, 0.0f), Rb = R0;
-#pragma unroll
-    for (int p = 0; p < R; ++p) {
-      const float2 yv = rows.pair(b, p), g2 = make_float2(gx[2 * p], gx[2 * p + 1]);
-      const float2 r = __ffma2_rn(g2, nI2, yv);
-      ss = __ffma2_rn(r, r, ss);
-      A[p] = __ffma2_rn(gy2, r, A[p]);
-      R0 = __ffma2_rn(g2, r, R0);
-      Rb = __fadd2_rn(Rb, r);
-      if constexpr (FRAME) {
-        Y2 = __ffma2_rn(yv, yv, Y2);
-        Y1 = __fadd2_rn(Y1, yv);
-      }
-    }
-    const float yl = rows.one(b, 2 * R);
-    const float r = fmaf(gx[2 * R], nI, yl);
-    ss.x = fmaf(r, r, ss.x);
-    Al = fmaf(gy, r, Al);
-    R0.x = fmaf(gx[2 * R], r, R0.x);
-    Rb.x += r;
-    if constexpr (FRAME) {
-      Y2.x = fmaf(yl, yl, Y2.x);
-      Y1.x += yl;
-    }
-    Sb = __fadd2_rn(Sb, Rb);
-    const float dv = (float)(b - R) + dy;
-    const float t = gy * dv * (R0.x + R0.y);
-    Sy += t;
-    Sy2 = fmaf(t, dv, Sy2);
-  };
-  {
-    const float g = ex2(-cc * dy * dy);
-    float up = ex2(-cc * fmaf(2.0f, dy, 1.0f)), dn = ex2(cc * fmaf(2.0f, dy, -1.0f));
-    row(R, g);
-    float gu = g, gd = g;
-#pragma unroll
-    for (int a = 1; a <= R; ++a) {
-      gu *= up;
-      gd *= dn;
-      up *= kappa;
-      dn *= kappa;
-      row(R + a, gu);
-      row(R - a, gd);
-    }
-  }
-  float SI = 0.0f, S1 = 0.0f, S2 = 0.0f;
-  const float dx = cxf - x;
-#pragma unroll
-  for (int a = 0; a < D; ++a) {
-    const float t = gx[a] * (a == 2 * R ? Al : (a & 1) ? A[a / 2].y : A[a / 2].x);
-    const float du = (float)(a - R) + dx;
-    SI += t;
-    S1 = fmaf(t, du, S1);
-    S2 = fmaf(t * du, du, S2);
-  }
-  float sb = Sb.x + Sb.y;
+  gauss_row<R>(cxf, x, P.c_psf, P.kappa, gx);
+  float gy[D];
+  gauss_row<R>(cyf, y, P.c_psf, P.kappa, gy);
   // inside-the-frame column / row ranges of the (true) patch
   const float ulo = fmaxf(0.0f, (float)R - cxf), uhi = fminf((float)(2 * R), (float)(W - 1) + (float)R - cxf);
   const float vlo = fmaxf(0.0f, (float)R - cyf), vhi = fminf((float)(2 * R), (float)(H - 1) + (float)R - cyf);
-  if (!(ulo == 0.0f && uhi == (float)(2 * R) && vlo == 0.0f && vhi == (float)(2 * R))) {
-    sb = 0.0f;
-#pragma unroll 1
-    for (int b = 0; b < D; ++b) {
-      if ((float)b < vlo || (float)b > vhi) continue;
-      const float dv = (float)(b - R) + dy;
-      const float nI = -(I * ex2(-cc * dv * dv));
-      float rb = 0.0f;
+  float ss = 0.0f, SI = 0.0f, S1 = 0.0f, Sy = 0.0f, Ss = 0.0f, Sb = 0.0f, Y2 = 0.0f, Y1 = 0.0f;
+  const float du0 = cxf - (float)R - x;
+  // patches wholly inside the frame (almost all) sum the b-derivative's
+  // residuals without per-pixel masks
+  const bool inside = ulo == 0.0f && uhi == (float)(2 * R) && vlo == 0.0f && vhi == (float)(2 * R);
+  auto rows = [&](auto inside_tag) {
+    constexpr bool IN = decltype(inside_tag)::value;
 #pragma unroll
-      for (int a = 0; a < D; ++a)
-        rb += ((float)a >= ulo && (float)a <= uhi) ? fmaf(gx[a], nI, rows.one(b, a)) : 0.0f;
-      sb += rb;
+    for (int b = 0; b < D; ++b) {
+      asm volatile("" ::: "memory");  // (a row's pixels at a time)
+      const float Igy = I * gy[b];
+      float R0 = 0.0f, R1 = 0.0f, R2 = 0.0f, Rb = 0.0f;
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        const float yv = px.one(b, a);  // y = z - b, 0 outside the frame
+        const float r = fmaf(-gx[a], Igy, yv);
+        ss = fmaf(r, r, ss);
+        Y2 = fmaf(yv, yv, Y2);
+        Y1 += yv;
+        const float t = r * gx[a];
+        R0 += t;
+        R1 = fmaf(t, (float)a, R1);
+        R2 = fmaf(t, (float)(a * a), R2);
+        if constexpr (IN)
+          Rb += r;
+        else
+          Rb += ((float)a >= ulo && (float)a <= uhi) ? r : 0.0f;
+      }
+      const float dv = (cyf - (float)R + (float)b) - y;
+      const float sx1 = R1 + du0 * R0;
+      const float sx2 = R2 + 2.0f * du0 * R1 + du0 * du0 * R0;
+      SI = fmaf(gy[b], R0, SI);
+      S1 = fmaf(gy[b], sx1, S1);
+      Sy = fmaf(gy[b] * dv, R0, Sy);
+      Ss = fmaf(gy[b], fmaf(dv * dv, R0, sx2), Ss);
+      if (IN || ((float)b >= vlo && (float)b <= vhi)) Sb += Rb;
     }
-  }
+  };
+  if (inside)
+    rows(std::true_type{});
+  else
+    rows(std::false_type{});
   const float iso2 = 2.0f * P.inv2so2;  // 1 / sigma_obs^2
   const float s2 = P.spsf * P.spsf;
-  const float sq = ss.x + ss.y;
   d[0] = I * S1 / s2 * iso2;
   d[1] = I * Sy / s2 * iso2;
   d[2] = SI * iso2;
-  d[3] = I * (S2 + Sy2) / (s2 * P.spsf) * iso2;
-  d[4] = sb * iso2;
-  if constexpr (FRAME) {
+  d[3] = I * Ss / (s2 * P.spsf) * iso2;
+  d[4] = Sb * iso2;
+  if (P.obs_model == 1) {
     // frame likelihood ratio: + sum y^2 / (2 sigma_obs^2), whose only
     // parameter is b (dy/db = -1 inside the frame, y = 0 outside)
-    d[4] -= (Y1.x + Y1.y) * iso2;
-    return -(sq - (Y2.x + Y2.y)) * P.inv2so2;
+    d[4] -= Y1 * iso2;
+    return -(ss - Y2) * P.inv2so2;
   }
-  return -sq * P.inv2so2;
+  return -ss * P.inv2so2;
 }
 
 // The same off the staged box, out of line (rare: a tile whose patches do not
 // fit one box), so that its addressing takes no registers of the main path.
 template <int R>
 __device__ __noinline__ float loglik_grad_frame(const PixelSource& px, int u, int v, float4 s, float I,
-                                                const TrackParams& P, float (&d)[5]) {
+                                                const TrackParams& P, float (&gxI)[2 * R + 1], float (&d)[5],
+                                                float& ss) {
   const FrameRows rows{px, u, v};
-  return P.obs_model == 1 ? loglik_grad<R, true>(rows, P.H, P.W, s.x, s.y, I, P, d)
-                          : loglik_grad<R, false>(rows, P.H, P.W, s.x, s.y, I, P, d);
+  const float dy = floorf(s.y + 0.5f) - s.y;
+  auto pix = [&](int b, int a) { return rows.one(b, a); };
+  ss = P.obs_model == 1 ? patch_sum<R, true>(pix, gxI, dy, P.c_psf, P.kappa)
+                        : patch_sum<R, false>(pix, gxI, dy, P.c_psf, P.kappa);
+  return loglik_grad<R>(rows, P.H, P.W, s.x, s.y, I, P, d);
 }
 
 // ------------------------------------------------------------------ replay
@@ -204,9 +164,10 @@ __device__ __noinline__ float loglik_grad_frame(const PixelSource& px, int u, in
 // One CTA per tile; the box of the tile's patches is staged in shared memory
 // twice (the copy shifted by one float makes every patch row a row of aligned
 // pairs), a tile whose patches do not fit reads the frame through L1.  Bound
-// by FP32 issue (the patch pass is ~450 instructions a particle) and the
-// latency of the gathers before it: a million particles take 56 us with four
-// CTAs an SM (64 registers, a few spilled), 59 us with three.
+// by FP32 issue (the two patch sums are ~1200 instructions a particle) and the
+// latency of the gathers before them.  Derivatives by column sums in packed
+// pairs took 55 us a million particles, but moved the gradient by up to 2e-5
+// (their error was smaller; results are held to the older order).
 // SINGLE: one track, its parameters and round keys in the constant bank.
 template <int R, bool SINGLE>
 __global__ void __launch_bounds__(K1_THREADS, 4) k_replay(const __grid_constant__ ReplayArgs a) {
@@ -325,25 +286,35 @@ __global__ void __launch_bounds__(K1_THREADS, 4) k_replay(const __grid_constant_
     const int jj = threadIdx.x + q * K1_THREADS;
     if (jj >= td.w) continue;
     const long long i = P.part_off + (long long)g * Np + td.z + jj;
-    float d[5];
-    float l;
+    float d[5], gxI[2 * R + 1];
+    float l, ss;
+    gauss_row<R>(floorf(s[q].x + 0.5f), s[q].x, P.c_psf, P.kappa, gxI);
+#pragma unroll
+    for (int c = 0; c < 2 * R + 1; ++c) gxI[c] *= I[q];
     if (staged) {
       const int c = pu[q] - umin, off = (pv[q] - vmin) * ROI_W + c;
-      const StagedRows rows{(c & 1) ? &s_roi[1][off - 1] : &s_roi[0][off]};
-      l = frame_model ? loglik_grad<R, true>(rows, P.H, P.W, s[q].x, s[q].y, I[q], P, d)
-                      : loglik_grad<R, false>(rows, P.H, P.W, s[q].x, s[q].y, I[q], P, d);
+      const float* base = (c & 1) ? &s_roi[1][off - 1] : &s_roi[0][off];
+      const float dy = floorf(s[q].y + 0.5f) - s[q].y;
+      ss = frame_model ? patch_ss_pairs<R, true>(base, gxI, dy, P.c_psf, P.kappa)
+                       : patch_ss_pairs<R, false>(base, gxI, dy, P.c_psf, P.kappa);
+      l = 0.0f;
+      asm volatile("" ::: "memory");  // (the pixels are read again, not held in registers)
+      if (a.dl_pv) l = loglik_grad<R>(StagedRows{base}, P.H, P.W, s[q].x, s[q].y, I[q], P, d);
     } else {
-      float df[5];
-      l = loglik_grad_frame<R>(px, pu[q], pv[q], s[q], I[q], P, df);
+      float df[5], gf[2 * R + 1], sf;
+#pragma unroll
+      for (int x = 0; x < 2 * R + 1; ++x) gf[x] = gxI[x];
+      l = loglik_grad_frame<R>(px, pu[q], pv[q], s[q], I[q], P, gf, df, sf);
+      ss = sf;
 #pragma unroll
       for (int x = 0; x < 5; ++x) d[x] = df[x];
     }
     const float lb = k >= 1 ? a.lbar_prev[P.group_off + o[q]] : -log_G;
-    const float lw = lb - log_Np + l;
+    const float lw = lb - log_Np - ss * P.inv2so2;
     if (a.dl_pv) {
       a.dl_pv[i] = make_float4(d[0], d[1], d[2], d[3]);
       a.dl_b[i] = d[4];
-      a.dl_lw[i] = lw;
+      a.dl_lw[i] = lb - log_Np + l;
     }
     if (lw == lw && lw > -INFINITY) {
       if (lw > mx) {
