@@ -167,7 +167,8 @@ __device__ __noinline__ float loglik_grad_frame(const PixelSource& px, int u, in
 // by FP32 issue (the two patch sums are ~1200 instructions a particle) and the
 // latency of the gathers before them.  Derivatives by column sums in packed
 // pairs took 55 us a million particles, but moved the gradient by up to 2e-5
-// (their error was smaller; results are held to the older order).
+// (their error was smaller; results are held to the older order: gradient of
+// 16 x 65536 particles over 20 frames 7.7 -> 4.2 ms, 3.5 with the packed sums).
 // SINGLE: one track, its parameters and round keys in the constant bank.
 template <int R, bool SINGLE>
 __global__ void __launch_bounds__(K1_THREADS, 4) k_replay(const __grid_constant__ ReplayArgs a) {
