@@ -2616,6 +2616,9 @@ __global__ void __launch_bounds__(TEAM* TEAMS, 1024 / (TEAM * TEAMS))
     auto item0 = [&](int sub) { return sub * CAP - a0 + tid * ITEMS; };  // the thread's first item
 #pragma unroll
     for (int r = 0; r < ITEMS; r += 4) reinterpret_cast<uint4*>(s_mark)[(ITEMS / 4) * tid + r / 4] = make_uint4(0u, 0u, 0u, 0u);
+    // other lanes set these marks: one warp has no other barrier before that
+    // (shuffles order no memory), larger teams have the ones of their sums
+    if constexpr (TEAM == 32) __syncwarp();
 
     float v[ITEMS];
     unsigned long long qv[ITEMS];
