@@ -33,8 +33,9 @@ struct pf_handle {
   int k1_grid = 1, rs_cluster = 1;
   int rs_threads = RS_THREADS;  // resampler CTA: RS_THREADS, or RS_THREADS_SMALL for small groups
   int rs_pad = 0;               // 0: every group starts on a 16-byte boundary, else 3 (ResampleArgs::pad)
-  // several tracks: the groups by class of size, resampled by one CTA each
-  // (PFARNA_RS_THREADS unset; pf_autotune may prefer the cluster kernel)
+  // several tracks: the groups by class of size, the large ones on clusters
+  // while they are few, the others by one CTA each (PFARNA_RS_THREADS unset;
+  // pf_autotune may prefer the cluster kernel for all)
   bool rs_by_class = false;
   int rs_sum_nt = RS_THREADS;   // GlobalArgs::sum_nt of those launches
   GroupClasses classes{};
@@ -758,6 +759,8 @@ pf_status pf_init(const pf_track_config* cfg, int32_t n_tracks, int32_t history,
     while (n < L.G_total && (c == 3 || gd[order[n]].Np + h->rs_pad > RG_THREADS[c] * RS_ITEMS)) ++n;
     h->classes.begin[c] = n;
   }
+  int n_big = 0;  // groups of more than one sub-chunk of the largest class
+  while (n_big < L.G_total && gd[order[n_big]].Np + h->rs_pad > RG_THREADS[0] * RS_ITEMS) ++n_big;
 
   // One TMA descriptor per track over its padded frame (boxes of ROI_W x
   // ROI_BOX_H floats).  If the driver cannot encode them, the propagate
@@ -848,26 +851,38 @@ pf_status pf_init(const pf_track_config* cfg, int32_t n_tracks, int32_t history,
     if (cfg[t].resample_rule == PF_RESAMPLE_ESS || cfg[t].send_rule == PF_SEND_KEYED) h->variants = true;
   }
   {
-    // resampler shape: small CTAs (eight per SM) when every group fits one
-    // of their sub-chunks; clusters sized to the largest group, as long as
-    // the launch stays within about two waves of two CTAs per SM
+    // Resampler shape.  One track: a cluster per group.  Several tracks:
+    // groups of one sub-chunk of a one-CTA class take those classes (a step
+    // of 8 groups of 64 to 2048 particles: 24 to 33 us by them, 27 to 33 by a
+    // CTA of the cluster kernel; of 2048 groups of 2048: 196 and 250).  Larger
+    // groups take them only where there are more than two per SM, enough to
+    // fill the chip with one CTA each; fewer of them run on clusters, whose
+    // CTAs share a group.  Measured, the step by one CTA each and by clusters:
+    // 2 groups of 2^20 2195 and 476 us, 8 of 65536 145 and 44, 64 of 16384 80
+    // and 59, 256 of 8192 113 and 108, 512 of 8192 187 and 201, 1024 of 4096
+    // 190 and 200.
     int maxNp = 1;
     for (int t = 0; t < n_tracks; ++t) maxNp = cfg[t].Np > maxNp ? cfg[t].Np : maxNp;
     h->rs_threads = maxNp <= RS_THREADS_SMALL * RS_ITEMS ? RS_THREADS_SMALL : RS_THREADS;
+    const char* rt = std::getenv("PFARNA_RS_THREADS");  // "128" / "512": the cluster kernel with CTAs of this size
     if (n_tracks == 1) {
       h->rs_cluster = resample_cluster(cfg[0].G, cfg[0].Np, h->rs_pad);
       if (h->rs_threads == RS_THREADS_SMALL && maxNp + h->rs_pad > RS_THREADS_SMALL * RS_ITEMS) h->rs_cluster = 2;
     } else {
-      const int sub = h->rs_threads * RS_ITEMS;
+      if (n_big > 2 * h->sms) n_big = 0;
+      h->rs_by_class = !rt && n_big < L.G_total;
+      // clusters sized to the largest group, as long as their launch stays
+      // within about two waves of two CTAs per SM
+      const int sub = h->rs_threads * RS_ITEMS, n = h->rs_by_class && n_big > 0 ? n_big : L.G_total;
       int c = (maxNp + sub - 1) / sub;
       c = c < 1 ? 1 : (c > 8 ? 8 : c);
-      while (c > 1 && (long long)h->G_total * c > 4LL * h->sms) c >>= 1;
+      while (c > 1 && (long long)n * c > 4LL * h->sms) c >>= 1;
       h->rs_cluster = c;
+      h->classes.begin[0] = h->rs_by_class ? n_big : 0;
+      h->classes.cluster = c;
     }
-    const char* rt = std::getenv("PFARNA_RS_THREADS");  // "128" / "512": force the resampler's CTA size
     if (rt && std::atoi(rt) == RS_THREADS_SMALL) h->rs_threads = RS_THREADS_SMALL;
     if (rt && std::atoi(rt) == RS_THREADS) h->rs_threads = RS_THREADS;
-    h->rs_by_class = n_tracks > 1 && !rt;
     h->rs_sum_nt = h->rs_threads;
   }
 

@@ -2121,8 +2121,7 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? (ITEMS > RS_ITEMS ? 1 : 2) :
   cg::cluster_group cl = cg::this_cluster();
   const int C = (int)cl.num_blocks();
   const int rank = (int)cl.block_rank();
-  const int grp = blockIdx.x / C;
-  if (a.fuse_global == 2 && grp >= a.n_groups) {
+  if (a.fuse_global == 2 && (int)blockIdx.x >= a.n_groups * C) {
     // the extra cluster of a one-track step: its first CTA runs the
     // track's global step once every group has reported; nothing waits on
     // it within the launch
@@ -2132,6 +2131,7 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? (ITEMS > RS_ITEMS ? 1 : 2) :
     grid_dep_launch();
     return;
   }
+  const int grp = a.list ? a.list[blockIdx.x / C] : blockIdx.x / C;
   const GroupDesc d = a.gd[grp];
   const int Np = d.Np;
   // LEAN: items and outputs are split in units of the 16-byte boundaries of
@@ -2205,6 +2205,7 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? (ITEMS > RS_ITEMS ? 1 : 2) :
   if (!a.u_arr)
     u = philox(Pt->key0, Pt->key1, make_uint4((uint32_t)d.g, 0u, (uint32_t)kk, Pt->tag | (ST_RESAMPLE << 4))).x;
   grid_dep_wait();
+  if (a.list) grid_dep_launch();  // the step's other classes of groups run beside this launch
   if (a.u_arr) u = a.u_arr[grp];
   if (a.tile_ctr && blockIdx.x == 0 && threadIdx.x == 0) *a.tile_ctr = 0;  // for the next propagate launch
   // A propagate launch that timed out or met an out-of-range ancestor left
@@ -3062,6 +3063,16 @@ static cudaError_t launch_groups_t(const ResampleArgs& a, bool pdl, cudaStream_t
 cudaError_t launch_resample_groups(const ResampleArgs& a0, const GroupClasses& gc, bool pdl, cudaStream_t s) {
   ResampleArgs a = a0;
   bool first = true;
+  if (gc.begin[0] > 0) {
+    a.n_groups = gc.begin[0];
+    a.list = gc.list;
+    if (a.glob.sum_nt == RS_THREADS) a.glob.sum_nt = 0;  // (that CTA's own order)
+    const cudaError_t e = launch_resample(a, a.n_groups, gc.cluster, pdl, s, RS_THREADS);
+    if (e != cudaSuccess) return e;
+    a.glob.sum_nt = a0.glob.sum_nt;
+    a.tile_ctr = nullptr;
+    first = false;
+  }
   for (int c = 0; c < 3; ++c) {
     a.n_groups = gc.begin[c + 1] - gc.begin[c];
     if (a.n_groups == 0) continue;

@@ -163,17 +163,19 @@ struct ResampleArgs {
   int pad;                     // 0: every group starts on 16 bytes of the log-weights and the ancestors, else 3
   int* tile_ctr;               // propagate kernel's tile counter to reset, or nullptr
   GlobalArgs glob;             // (fuse_global) arguments of that step, finalize = 1
-  // one-CTA resampler (launch_resample_groups): the groups of this launch
+  // launch_resample_groups: the groups of this launch
   const int* list;             // global group indices, or nullptr (0 .. n_groups - 1)
   int wait_last;               // 1: a launch behind another class of the same step, which waits for that one
                                // at its end instead of its start
 };
 
 // The groups of a batch by class of size (RG_THREADS): list[begin[c] ..
-// begin[c + 1]) are those of class c, the largest first.
+// begin[c + 1]) are those of class c, the largest first; the begin[0] groups
+// before them run on clusters of `cluster` CTAs.
 struct GroupClasses {
   const int* list;             // device
   int begin[4];
+  int cluster;
 };
 
 // pf_backward (pf_adjoint.cu)
@@ -276,8 +278,8 @@ cudaError_t launch_resample(const ResampleArgs& a, int n_groups, int cluster, bo
 // Largest cluster that the general 512-thread resampler can be launched with:
 // 16 if the device has room for several, else the portable 8.
 int resample_max_cluster();
-// The resampling of many groups, one CTA (or one warp) per group, a launch
-// per class of group size.
+// The resampling of many groups: a few large ones on clusters, the others by
+// one CTA (or one warp) each, a launch per class of group size.
 cudaError_t launch_resample_groups(const ResampleArgs& a, const GroupClasses& gc, bool pdl, cudaStream_t s);
 cudaError_t launch_global(const GlobalArgs& a, int n_tracks, bool pdl, cudaStream_t s);
 cudaError_t launch_finish(const GlobalArgs& a, int n_tracks, cudaStream_t s);
