@@ -7,6 +7,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -1649,12 +1650,18 @@ pf_status pf_profile_read(pf_handle* h, int32_t n, int64_t* launches, double* to
   return PF_OK;
 }
 
-// Checkpoint: a header, then the workspace except the TMA descriptors.
+// Checkpoint: a header, then the workspace except the TMA descriptors.  The
+// header carries every launch shape that decides an order of summation.  The
+// first form of the header ended at rs_threads; it is still read: a filter
+// saved so resampled with the cluster kernel of that size.
 struct CheckpointHeader {
   unsigned long long magic, sig, ws_total;
   int32_t abi, steps_run, finish_pending, k1_grid, rs_cluster, rs_threads;
+  int32_t rs_by_class, rs_big, rs_big_cluster, rs_sum_nt;  // pf_handle: rs_by_class, classes.begin[0] and .cluster
 };
-static const unsigned long long kCheckpointMagic = 0x6b70635f666e7270ull;  // "prnf_cpk"
+static const unsigned long long kCheckpointMagic1 = 0x6b70635f666e7270ull;  // "prnf_cpk"
+static const unsigned long long kCheckpointMagic = 0x326b70635f666e72ull;   // "rnf_cpk2"
+constexpr size_t kCheckpointHeader1 = offsetof(CheckpointHeader, rs_by_class);
 
 pf_status pf_checkpoint_bytes(const pf_handle* h, size_t* bytes) {
   if (!h || !bytes) return fail(nullptr, PF_ERR_ARG, "NULL argument");
@@ -1669,7 +1676,8 @@ pf_status pf_save(pf_handle* h, void* host, size_t bytes, void* stream) {
   if (bytes < need) return fail(h, PF_ERR_ARG, "checkpoint buffer too small");
   cudaStream_t s = (cudaStream_t)stream;
   CheckpointHeader hd{kCheckpointMagic, h->cfg_sig, h->ws_total, PF_ABI_VERSION, h->steps_run,
-                      h->finish_pending ? 1 : 0, h->k1_grid, h->rs_cluster, h->rs_threads};
+                      h->finish_pending ? 1 : 0, h->k1_grid, h->rs_cluster, h->rs_threads,
+                      h->rs_by_class ? 1 : 0, h->classes.begin[0], h->classes.cluster, h->rs_sum_nt};
   std::memcpy(host, &hd, sizeof hd);
   char* dst = (char*)host + sizeof hd;
   cudaError_t e;
@@ -1683,16 +1691,23 @@ pf_status pf_save(pf_handle* h, void* host, size_t bytes, void* stream) {
 
 pf_status pf_load(pf_handle* h, const void* host, size_t bytes, void* stream) {
   if (!h || !host) return fail(h, PF_ERR_ARG, "NULL argument");
-  size_t need = 0;
-  pf_checkpoint_bytes(h, &need);
   CheckpointHeader hd{};
-  if (bytes < sizeof hd) return fail(h, PF_ERR_ARG, "not a checkpoint");
-  std::memcpy(&hd, host, sizeof hd);
-  if (hd.magic != kCheckpointMagic || hd.abi != PF_ABI_VERSION) return fail(h, PF_ERR_ARG, "not a checkpoint");
-  if (hd.sig != h->cfg_sig || hd.ws_total != h->ws_total || bytes < need)
+  if (bytes < kCheckpointHeader1) return fail(h, PF_ERR_ARG, "not a checkpoint");
+  std::memcpy(&hd, host, kCheckpointHeader1);
+  const size_t head = hd.magic == kCheckpointMagic ? sizeof hd : kCheckpointHeader1;
+  if ((hd.magic != kCheckpointMagic && hd.magic != kCheckpointMagic1) || hd.abi != PF_ABI_VERSION || bytes < head)
+    return fail(h, PF_ERR_ARG, "not a checkpoint");
+  std::memcpy(&hd, host, head);
+  if (hd.sig != h->cfg_sig || hd.ws_total != h->ws_total || bytes < head + h->ws_total - h->tmap_bytes)
     return fail(h, PF_ERR_ARG, "checkpoint of a filter with other configurations");
+  const bool shapes_ok =
+      hd.magic == kCheckpointMagic1 ||
+      ((!hd.rs_by_class || h->n_tracks > 1) && hd.rs_big >= 0 && hd.rs_big <= h->classes.begin[1] &&
+       (hd.rs_big == 0 || (hd.rs_big_cluster >= 1 && hd.rs_big_cluster <= 8)) &&
+       (hd.rs_sum_nt == RS_THREADS || hd.rs_sum_nt == RS_THREADS_SMALL));
+  if (!shapes_ok) return fail(h, PF_ERR_ARG, "checkpoint with launch shapes out of range");
   cudaStream_t s = (cudaStream_t)stream;
-  const char* src = (const char*)host + sizeof hd;
+  const char* src = (const char*)host + head;
   cudaError_t e;
   if ((e = cudaMemcpyAsync(h->ws, src, h->tmap_off, cudaMemcpyHostToDevice, s)) ||
       (e = cudaMemcpyAsync(h->ws + h->tmap_off + h->tmap_bytes, src + h->tmap_off,
@@ -1704,6 +1719,13 @@ pf_status pf_load(pf_handle* h, const void* host, size_t bytes, void* stream) {
   h->k1_grid = hd.k1_grid;
   h->rs_cluster = hd.rs_cluster;
   h->rs_threads = hd.rs_threads == RS_THREADS_SMALL ? RS_THREADS_SMALL : RS_THREADS;
+  h->rs_by_class = hd.rs_by_class != 0;
+  h->rs_sum_nt = h->rs_threads;
+  if (hd.magic == kCheckpointMagic) {
+    h->rs_sum_nt = hd.rs_sum_nt;
+    h->classes.begin[0] = hd.rs_big;
+    h->classes.cluster = hd.rs_big_cluster;
+  }
   h->failed = 0;
   h->last_stream = s;
   if (h->graph) {  // a captured step may hold other launch shapes
