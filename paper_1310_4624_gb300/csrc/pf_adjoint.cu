@@ -56,10 +56,27 @@ struct StagedRows {
   const float* base;
   __device__ __forceinline__ float one(int b, int a) const { return base[b * ROI_W + a]; }
 };
+// From the frame, with one bit per row and per column of the patch that lies
+// inside it: the test of a pixel is one bit at a constant place, and its load
+// is predicated, whether the patch crosses an edge or not (a few lanes of
+// nearly every warp of scattered patches do).
 struct FrameRows {
-  const PixelSource& px;
-  int u, v;
-  __device__ __forceinline__ float one(int b, int a) const { return px.at(u + a, v + b); }
+  const float* base;  // the patch's first pixel (outside the frame if the patch crosses an edge)
+  int w;
+  uint32_t rows, cols;
+  float bg;
+  __device__ __forceinline__ FrameRows(const PixelSource& px, int u, int v, int D)
+      : base(px.z + (long long)(v - px.sub) * px.w + (u - px.sub)), w(px.w), rows(bits(v - px.sub, D, px.h)),
+        cols(bits(u - px.sub, D, px.w)), bg(px.bg) {}
+  // bit i: 0 <= first + i < n, for i < D
+  static __device__ __forceinline__ uint32_t bits(int first, int D, int n) {
+    const int lo = min(max(-first, 0), D), hi = min(max(n - first, 0), D);
+    return ((1u << hi) - 1u) & ~((1u << lo) - 1u);
+  }
+  __device__ __forceinline__ float one(int b, int a) const {
+    const uint32_t m = ((rows >> b) & 1u) ? cols : 0u;
+    return ((m >> a) & 1u) ? __fsub_rn(__ldg(base + (long long)b * w + a), bg) : 0.0f;
+  }
 };
 
 // Log-likelihood (Sec. V model) and its partial derivatives for the
@@ -71,15 +88,16 @@ struct FrameRows {
 // background, so only inside pixels depend on b.
 // The replay's group log-weights come from patch_sum's order of the same
 // pixels; both orders are part of the result's rounding and are kept.
-template <int R, class Rows>
-__device__ __forceinline__ float loglik_grad(const Rows& px, int H, int W, float x, float y, float I,
+// ROLLED: a loop over the rows (gy from memory, every patch masked), for
+// patches read from the frame, whose loads would otherwise be hoisted into
+// more registers than there are; the sums and their order are the same.
+template <int R, bool ROLLED, class Rows, class Gy>
+__device__ __forceinline__ float loglik_grad(const Rows& px, const Gy& gy, int H, int W, float x, float y, float I,
                                              const TrackParams& P, float (&d)[5]) {
   constexpr int D = 2 * R + 1;
   const float cxf = floorf(x + 0.5f), cyf = floorf(y + 0.5f);
   float gx[D];
   gauss_row<R>(cxf, x, P.c_psf, P.kappa, gx);
-  float gy[D];
-  gauss_row<R>(cyf, y, P.c_psf, P.kappa, gy);
   // inside-the-frame column / row ranges of the (true) patch
   const float ulo = fmaxf(0.0f, (float)R - cxf), uhi = fminf((float)(2 * R), (float)(W - 1) + (float)R - cxf);
   const float vlo = fmaxf(0.0f, (float)R - cyf), vhi = fminf((float)(2 * R), (float)(H - 1) + (float)R - cyf);
@@ -90,10 +108,11 @@ __device__ __forceinline__ float loglik_grad(const Rows& px, int H, int W, float
   const bool inside = ulo == 0.0f && uhi == (float)(2 * R) && vlo == 0.0f && vhi == (float)(2 * R);
   auto rows = [&](auto inside_tag) {
     constexpr bool IN = decltype(inside_tag)::value;
-#pragma unroll
+#pragma unroll(ROLLED ? 1 : D)
     for (int b = 0; b < D; ++b) {
       asm volatile("" ::: "memory");  // (a row's pixels at a time)
-      const float Igy = I * gy[b];
+      const float gyb = gy(b);
+      const float Igy = I * gyb;
       float R0 = 0.0f, R1 = 0.0f, R2 = 0.0f, Rb = 0.0f;
 #pragma unroll
       for (int a = 0; a < D; ++a) {
@@ -114,14 +133,14 @@ __device__ __forceinline__ float loglik_grad(const Rows& px, int H, int W, float
       const float dv = (cyf - (float)R + (float)b) - y;
       const float sx1 = R1 + du0 * R0;
       const float sx2 = R2 + 2.0f * du0 * R1 + du0 * du0 * R0;
-      SI = fmaf(gy[b], R0, SI);
-      S1 = fmaf(gy[b], sx1, S1);
-      Sy = fmaf(gy[b] * dv, R0, Sy);
-      Ss = fmaf(gy[b], fmaf(dv * dv, R0, sx2), Ss);
+      SI = fmaf(gyb, R0, SI);
+      S1 = fmaf(gyb, sx1, S1);
+      Sy = fmaf(gyb * dv, R0, Sy);
+      Ss = fmaf(gyb, fmaf(dv * dv, R0, sx2), Ss);
       if (IN || ((float)b >= vlo && (float)b <= vhi)) Sb += Rb;
     }
   };
-  if (inside)
+  if (!ROLLED && inside)
     rows(std::true_type{});
   else
     rows(std::false_type{});
@@ -141,21 +160,90 @@ __device__ __forceinline__ float loglik_grad(const Rows& px, int H, int W, float
   return -ss * P.inv2so2;
 }
 
-// The same off the staged box, out of line (rare: a tile whose patches do not
-// fit one box), so that its addressing takes no registers of the main path.
-template <int R>
-__device__ __noinline__ float loglik_grad_frame(const PixelSource& px, int u, int v, float4 s, float I,
-                                                const TrackParams& P, float (&gxI)[2 * R + 1], float (&d)[5],
-                                                float& ss) {
-  const FrameRows rows{px, u, v};
-  const float dy = floorf(s.y + 0.5f) - s.y;
-  auto pix = [&](int b, int a) { return rows.one(b, a); };
-  ss = P.obs_model == 1 ? patch_sum<R, true>(pix, gxI, dy, P.c_psf, P.kappa)
-                        : patch_sum<R, false>(pix, gxI, dy, P.c_psf, P.kappa);
-  return loglik_grad<R>(rows, P.H, P.W, s.x, s.y, I, P, d);
+// ------------------------------------------------------------------ replay
+// A particle's log-weight into the thread's running (max, sum exp), and what
+// the reverse sweep takes of it (log-weight `lwg`, derivatives d).
+__device__ __forceinline__ void weigh(float lw, float& mx, float& sm) {
+  if (lw == lw && lw > -INFINITY) {
+    if (lw > mx) {
+      sm = sm * __expf(mx - lw) + 1.0f;
+      mx = lw;
+    } else {
+      sm += __expf(lw - mx);
+    }
+  }
+}
+__device__ __forceinline__ void keep_derivatives(const ReplayArgs& a, long long i, const float (&d)[5], float lwg) {
+  a.dl_pv[i] = make_float4(d[0], d[1], d[2], d[3]);
+  a.dl_b[i] = d[4];
+  a.dl_lw[i] = lwg;
 }
 
-// ------------------------------------------------------------------ replay
+// The pixels that patches are taken from, of a single track's frame or of
+// the track's padded frame.
+template <int R>
+__device__ __forceinline__ PixelSource pixel_source(const ReplayArgs& a, const TrackParams& P) {
+  constexpr int PAD = 2 * R + 1;
+  return a.zraw ? PixelSource{a.zraw, P.W, P.H, PAD, P.bg}
+                : PixelSource{a.ypad + P.ypad_off, P.pitch, P.H + 2 * PAD, 0, 0.0f};
+}
+
+// A patch's corner in padded-frame coordinates (centre clamped so that a
+// patch wholly off the frame reads background).
+template <int R>
+__device__ __forceinline__ int patch_corner(float x, int n) {
+  return (int)fminf(fmaxf(floorf(x + 0.5f), -(float)(R + 1)), (float)(n + R)) - R + (2 * R + 1);
+}
+
+// The weights of a tile whose patches do not fit one staging box (a spread
+// population): the patches are read from the frame.  Out of line, and from
+// the states the tile has just stored, so that nothing of it takes registers
+// of the staged path; gy of the rolled row loop lies in s_gy (one float per
+// thread and row, of the staging buffer that such a tile does not use).  Bound
+// by L1: a lane's pixel is a line of its own, in both passes over a patch.
+// The gradient over two frames of 64 x 16384 spread particles: 1939 us with
+// the patch's rows and arrays spilled under the staged path's registers, 1052
+// from prepared frames without bounds checks, 739 here.
+template <int R>
+__device__ __noinline__ float2 replay_off_box(const ReplayArgs& a, const TrackParams& P, int4 td, float* s_gy) {
+  constexpr int D = 2 * R + 1;
+  const int g = td.y, Np = P.Np, k = a.k;
+  const float log_G = logf((float)P.G), log_Np = logf((float)Np);
+  const PixelSource px = pixel_source<R>(a, P);
+  const uint32_t* __restrict__ par_t =
+      a.parent + P.parent_off + (long long)(k % a.history) * ((long long)P.G * Np);
+  float mx = -INFINITY, sm = 0.0f;
+  for (int jj = threadIdx.x; jj < td.w; jj += K1_THREADS) {
+    const long long il = (long long)g * Np + td.z + jj, i = P.part_off + il;
+    const float4 s = a.pv_out[i];
+    const float I = a.I_out[i];
+    const float lb = k >= 1 ? a.lbar_prev[P.group_off + (int)fastdiv(par_t[il], P.m_Np)] : -log_G;
+    const FrameRows rows(px, patch_corner<R>(s.x, P.W), patch_corner<R>(s.y, P.H), D);
+    float ss;
+    {
+      float gxI[D];
+      gauss_row<R>(floorf(s.x + 0.5f), s.x, P.c_psf, P.kappa, gxI);
+#pragma unroll
+      for (int c = 0; c < D; ++c) gxI[c] *= I;
+      const float dy = floorf(s.y + 0.5f) - s.y;
+      auto pix = [&](int b, int c) { return rows.one(b, c); };
+      ss = P.obs_model == 1 ? patch_sum<R, true>(pix, gxI, dy, P.c_psf, P.kappa)
+                            : patch_sum<R, false>(pix, gxI, dy, P.c_psf, P.kappa);
+    }
+    weigh(lb - log_Np - ss * P.inv2so2, mx, sm);
+    if (a.dl_pv) {
+      float gy[D], d[5];
+      gauss_row<R>(floorf(s.y + 0.5f), s.y, P.c_psf, P.kappa, gy);
+#pragma unroll
+      for (int b = 0; b < D; ++b) s_gy[b * K1_THREADS + threadIdx.x] = gy[b];
+      const float l = loglik_grad<R, true>(rows, [&](int b) { return s_gy[b * K1_THREADS + threadIdx.x]; }, P.H, P.W,
+                                           s.x, s.y, I, P, d);
+      keep_derivatives(a, i, d, lb - log_Np + l);
+    }
+  }
+  return make_float2(mx, sm);
+}
+
 // Replay of step k for every slot: the state (propagate: NCV from the
 // recorded parent and the step's normals; else as given in pv_out), the
 // log-weights' (max, sum exp) per tile for the group log-weights and, where
@@ -172,7 +260,7 @@ __device__ __noinline__ float loglik_grad_frame(const PixelSource& px, int u, in
 // SINGLE: one track, its parameters and round keys in the constant bank.
 template <int R, bool SINGLE>
 __global__ void __launch_bounds__(K1_THREADS, 4) k_replay(const __grid_constant__ ReplayArgs a) {
-  constexpr int D = 2 * R + 1, PAD = 2 * R + 1, NW = K1_THREADS / 32;
+  constexpr int D = 2 * R + 1, NW = K1_THREADS / 32;
   __shared__ __align__(16) float s_roi[2][ROI_FLOATS + 4];
   __shared__ int s_box[NW][4];
   __shared__ float s_m[NW], s_s[NW];
@@ -232,8 +320,8 @@ __global__ void __launch_bounds__(K1_THREADS, 4) k_replay(const __grid_constant_
       a.zero_pv[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       a.zero_I[i] = 0.0f;
     }
-    pu[q] = (int)fminf(fmaxf(floorf(s[q].x + 0.5f), -(float)(R + 1)), (float)(P.W + R)) - R + PAD;
-    pv[q] = (int)fminf(fmaxf(floorf(s[q].y + 0.5f), -(float)(R + 1)), (float)(P.H + R)) - R + PAD;
+    pu[q] = patch_corner<R>(s[q].x, P.W);
+    pv[q] = patch_corner<R>(s[q].y, P.H);
     umin = min(umin, pu[q]);
     umax = max(umax, pu[q]);
     vmin = min(vmin, pv[q]);
@@ -241,8 +329,7 @@ __global__ void __launch_bounds__(K1_THREADS, 4) k_replay(const __grid_constant_
   }
 
   // the box of the tile's patches, staged as y values
-  const PixelSource px = a.zraw ? PixelSource{a.zraw, P.W, P.H, PAD, P.bg}
-                                : PixelSource{a.ypad + P.ypad_off, P.pitch, P.H + 2 * PAD, 0, 0.0f};
+  const PixelSource px = pixel_source<R>(a, P);
   umin = __reduce_min_sync(0xffffffffu, umin);
   umax = __reduce_max_sync(0xffffffffu, umax);
   vmin = __reduce_min_sync(0xffffffffu, vmin);
@@ -279,52 +366,42 @@ __global__ void __launch_bounds__(K1_THREADS, 4) k_replay(const __grid_constant_
     __syncthreads();
   }
 
-  const float log_G = logf((float)P.G), log_Np = logf((float)Np);
-  const bool frame_model = P.obs_model == 1;
   float mx = -INFINITY, sm = 0.0f;
+  if (staged) {
+    const float log_G = logf((float)P.G), log_Np = logf((float)Np);
+    const bool frame_model = P.obs_model == 1;
 #pragma unroll
-  for (int q = 0; q < K1_PPT; ++q) {
-    const int jj = threadIdx.x + q * K1_THREADS;
-    if (jj >= td.w) continue;
-    const long long i = P.part_off + (long long)g * Np + td.z + jj;
-    float d[5], gxI[2 * R + 1];
-    float l, ss;
-    gauss_row<R>(floorf(s[q].x + 0.5f), s[q].x, P.c_psf, P.kappa, gxI);
-#pragma unroll
-    for (int c = 0; c < 2 * R + 1; ++c) gxI[c] *= I[q];
-    if (staged) {
+    for (int q = 0; q < K1_PPT; ++q) {
+      const int jj = threadIdx.x + q * K1_THREADS;
+      if (jj >= td.w) continue;
+      const long long i = P.part_off + (long long)g * Np + td.z + jj;
       const int c = pu[q] - umin, off = (pv[q] - vmin) * ROI_W + c;
       const float* base = (c & 1) ? &s_roi[1][off - 1] : &s_roi[0][off];
-      const float dy = floorf(s[q].y + 0.5f) - s[q].y;
-      ss = frame_model ? patch_ss_pairs<R, true>(base, gxI, dy, P.c_psf, P.kappa)
-                       : patch_ss_pairs<R, false>(base, gxI, dy, P.c_psf, P.kappa);
-      l = 0.0f;
-      asm volatile("" ::: "memory");  // (the pixels are read again, not held in registers)
-      if (a.dl_pv) l = loglik_grad<R>(StagedRows{base}, P.H, P.W, s[q].x, s[q].y, I[q], P, d);
-    } else {
-      float df[5], gf[2 * R + 1], sf;
+      float ss;
+      {
+        float gxI[D];
+        gauss_row<R>(floorf(s[q].x + 0.5f), s[q].x, P.c_psf, P.kappa, gxI);
 #pragma unroll
-      for (int x = 0; x < 2 * R + 1; ++x) gf[x] = gxI[x];
-      l = loglik_grad_frame<R>(px, pu[q], pv[q], s[q], I[q], P, gf, df, sf);
-      ss = sf;
-#pragma unroll
-      for (int x = 0; x < 5; ++x) d[x] = df[x];
-    }
-    const float lb = k >= 1 ? a.lbar_prev[P.group_off + o[q]] : -log_G;
-    const float lw = lb - log_Np - ss * P.inv2so2;
-    if (a.dl_pv) {
-      a.dl_pv[i] = make_float4(d[0], d[1], d[2], d[3]);
-      a.dl_b[i] = d[4];
-      a.dl_lw[i] = lb - log_Np + l;
-    }
-    if (lw == lw && lw > -INFINITY) {
-      if (lw > mx) {
-        sm = sm * __expf(mx - lw) + 1.0f;
-        mx = lw;
-      } else {
-        sm += __expf(lw - mx);
+        for (int x = 0; x < D; ++x) gxI[x] *= I[q];
+        const float dy = floorf(s[q].y + 0.5f) - s[q].y;
+        ss = frame_model ? patch_ss_pairs<R, true>(base, gxI, dy, P.c_psf, P.kappa)
+                         : patch_ss_pairs<R, false>(base, gxI, dy, P.c_psf, P.kappa);
       }
+      const float lb = k >= 1 ? a.lbar_prev[P.group_off + o[q]] : -log_G;
+      asm volatile("" ::: "memory");  // (the pixels are read again, not held in registers)
+      if (a.dl_pv) {
+        float gy[D], d[5];
+        gauss_row<R>(floorf(s[q].y + 0.5f), s[q].y, P.c_psf, P.kappa, gy);
+        const float l = loglik_grad<R, false>(StagedRows{base}, [&](int b) { return gy[b]; }, P.H, P.W, s[q].x, s[q].y,
+                                              I[q], P, d);
+        keep_derivatives(a, i, d, lb - log_Np + l);
+      }
+      weigh(lb - log_Np - ss * P.inv2so2, mx, sm);
     }
+  } else {
+    const float2 ms = replay_off_box<R>(a, P, td, &s_roi[0][0]);
+    mx = ms.x;
+    sm = ms.y;
   }
   // block (max, sum exp) of the tile
   const float m2 = warp_max(mx);
