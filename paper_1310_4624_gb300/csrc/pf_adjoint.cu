@@ -537,9 +537,15 @@ __global__ void __launch_bounds__(K1_THREADS, 4) k_adjoint(const __grid_constant
   const float lam = a.lam_k[P.group_off + g], dlam = (float)a.dlam_k[P.group_off + g];
   uint32_t par[K1_PPT];
   int o[K1_PPT], other = -1;
-  float dlw[K1_PPT], dI[K1_PPT], cI[K1_PPT];
+  float dlw[K1_PPT], cI[K1_PPT];
   float4 c[K1_PPT];
-  float v[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // gradient terms, then dL_{k-1} of g and of `other`
+  // sums over the warp: the gradient terms (0 .. 4), and for dL_{k-1} the
+  // weight adjoints that came from g (OWN) and from `other` (PRE), one FP32
+  // sum per 32 particles and FP64 from there on; the term of A (1) has a value
+  // at step 0 only, which has no dL before it
+  static_assert(K1_PPT == 2, "one sum per particle of a thread");
+  constexpr int OWN[K1_PPT] = {5, 7}, PRE[K1_PPT] = {6, 1};
+  float v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
 #pragma unroll
   for (int q = 0; q < K1_PPT; ++q) {
     const int jj = threadIdx.x + q * K1_THREADS;
@@ -577,9 +583,9 @@ __global__ void __launch_bounds__(K1_THREADS, 4) k_adjoint(const __grid_constant
 #pragma unroll
     for (int q = 0; q < K1_PPT; ++q) {
       if (o[q] == g)
-        v[5] += dlw[q];
+        v[OWN[q]] = dlw[q];
       else if (o[q] == other)
-        v[6] += dlw[q];
+        v[PRE[q]] = dlw[q];
       else if (dlw[q] != 0.0f)
         atomicAdd(&a.D[P.group_off + o[q]], (double)dlw[q]);
       const int jj = threadIdx.x + q * K1_THREADS;
@@ -643,8 +649,13 @@ __global__ void __launch_bounds__(K1_THREADS, 4) k_adjoint(const __grid_constant
   if (warp == 0) {
     if (lane < 6) {
       double r = 0.0;
+      if (lane != PRE[1] || k == 0) {
 #pragma unroll
-      for (int w = 0; w < NW; ++w) r += (double)s_red[w][lane];
+        for (int w = 0; w < NW; ++w) r += (double)s_red[w][lane];
+        if (lane == OWN[0])
+#pragma unroll
+          for (int w = 0; w < NW; ++w) r += (double)s_red[w][OWN[1]];
+      }
       if (r != 0.0) {
         if (lane < 5)
           atomicAdd(&a.grad[((long long)(blockIdx.x % GRAD_COPIES) * a.n_tracks + td.x) * GRAD_STRIDE + lane], r);
@@ -659,7 +670,7 @@ __global__ void __launch_bounds__(K1_THREADS, 4) k_adjoint(const __grid_constant
       for (int u = 0; u < NW; ++u)
         if (s_other[u] == ow) {
           first = first && u >= w;
-          r += (double)s_red[u][6];
+          r += (double)s_red[u][PRE[0]] + (double)s_red[u][PRE[1]];
         }
       if (first && r != 0.0) atomicAdd(&a.D[P.group_off + ow], r);
     }
