@@ -339,10 +339,11 @@ Layout plan(const pf_track_config* c, int n, int history) {
   L.saved = o;
   L.order = take(sizeof(int) * (size_t)L.G_total);
   if (L.adjoint) {
-    // the derivatives of every step of the history where they take at most
-    // ADJ_STORE_MAX, else of one segment between checkpoints
+    // the derivatives of as many steps of the history as ADJ_STORE_MAX holds,
+    // and of one segment between checkpoints at least
     const size_t per_step = (size_t)L.N_total * (sizeof(float4) + 2 * sizeof(float));
-    L.adj_steps = per_step * (size_t)history <= ADJ_STORE_MAX ? history : adjoint_segment(history);
+    const size_t fit = ADJ_STORE_MAX / per_step;
+    L.adj_steps = fit < (size_t)history ? std::max((int)fit, adjoint_segment(history)) : history;
     L.dl_pv = take(sizeof(float4) * (size_t)L.N_total * L.adj_steps);
     L.dl_b = take(sizeof(float) * (size_t)L.N_total * L.adj_steps);
     L.dl_lw = take(sizeof(float) * (size_t)L.N_total * L.adj_steps);
