@@ -646,33 +646,35 @@ __global__ void __launch_bounds__(K1_THREADS, 4) k_adjoint(const __grid_constant
     }
   }
   __syncthreads();
+  // FP64 from here, where an instruction holds the SM's one pipe for 19
+  // cycles: a warp's lanes share the sums, four to a slot, and a second warp
+  // takes the other origins (one lane summing all eight warps, twice for the
+  // second sums, took 7 us more for a million particles)
+  static_assert(NW == 8, "two warps' sums per lane");
   if (warp == 0) {
-    if (lane < 6) {
-      double r = 0.0;
-      if (lane != PRE[1] || k == 0) {
+    const int at = lane & 7, w = lane >> 3;
+    double r = (double)s_red[w][at] + (double)s_red[w + 4][at];
+    r += __shfl_xor_sync(FULL, r, 8);
+    r += __shfl_xor_sync(FULL, r, 16);
+    const double second = __shfl_down_sync(FULL, r, OWN[1] - OWN[0]);
+    if (lane == OWN[0]) r += second;
+    if (lane < OWN[0] && r != 0.0 && (lane != PRE[1] || k == 0))
+      atomicAdd(&a.grad[((long long)(blockIdx.x % GRAD_COPIES) * a.n_tracks + td.x) * GRAD_STRIDE + lane], r);
+    else if (lane == OWN[0] && r != 0.0)
+      atomicAdd(&a.D[P.group_off + g], r);
+  } else if (warp == 1 && k >= 1) {
+    // the warps' second origins, as a rule one group
+    const int ow = lane < NW ? s_other[lane] : -1, m = __reduce_max_sync(FULL, ow);
+    if (m < 0) return;
+    double r = 0.0;
+    if (ow >= 0) r = (double)s_red[lane][PRE[0]] + (double)s_red[lane][PRE[1]];
+    if (__all_sync(FULL, ow < 0 || ow == m)) {
 #pragma unroll
-        for (int w = 0; w < NW; ++w) r += (double)s_red[w][lane];
-        if (lane == OWN[0])
-#pragma unroll
-          for (int w = 0; w < NW; ++w) r += (double)s_red[w][OWN[1]];
-      }
-      if (r != 0.0) {
-        if (lane < 5)
-          atomicAdd(&a.grad[((long long)(blockIdx.x % GRAD_COPIES) * a.n_tracks + td.x) * GRAD_STRIDE + lane], r);
-        else
-          atomicAdd(&a.D[P.group_off + g], r);
-      }
-    } else if (k >= 1 && lane >= 8 && lane < 8 + NW) {
-      // the warps' second origins, as a rule one group: its first warp adds
-      const int w = lane - 8, ow = s_other[w];
-      double r = 0.0;
-      bool first = ow >= 0;
-      for (int u = 0; u < NW; ++u)
-        if (s_other[u] == ow) {
-          first = first && u >= w;
-          r += (double)s_red[u][PRE[0]] + (double)s_red[u][PRE[1]];
-        }
-      if (first && r != 0.0) atomicAdd(&a.D[P.group_off + ow], r);
+      for (int d = 1; d < NW; d *= 2) r += __shfl_xor_sync(FULL, r, d);
+      if (lane != 0) r = 0.0;
+      if (r != 0.0) atomicAdd(&a.D[P.group_off + m], r);
+    } else if (r != 0.0) {
+      atomicAdd(&a.D[P.group_off + ow], r);
     }
   }
 }
