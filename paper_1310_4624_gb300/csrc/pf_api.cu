@@ -38,7 +38,7 @@ struct pf_handle {
   // while they are few, the others by one CTA each (PFARNA_RS_THREADS unset;
   // pf_autotune may prefer the cluster kernel for all)
   bool rs_by_class = false;
-  int rs_sum_nt = RS_THREADS;   // GlobalArgs::sum_nt of those launches
+  int rs_sum_nt = RS_THREADS;   // several tracks: GlobalArgs::sum_nt, whichever kernel resamples
   GroupClasses classes{};
   int steps_run = 0;
   int failed = 0;
@@ -871,17 +871,20 @@ pf_status pf_init(const pf_track_config* cfg, int32_t n_tracks, int32_t history,
       h->rs_cluster = resample_cluster(cfg[0].G, cfg[0].Np, h->rs_pad);
       if (h->rs_threads == RS_THREADS_SMALL && maxNp + h->rs_pad > RS_THREADS_SMALL * RS_ITEMS) h->rs_cluster = 2;
     } else {
-      if (n_big > 2 * h->sms) n_big = 0;
-      h->rs_by_class = !rt && n_big < L.G_total;
       // clusters sized to the largest group, as long as their launch stays
       // within about two waves of two CTAs per SM
-      const int sub = h->rs_threads * RS_ITEMS, n = h->rs_by_class && n_big > 0 ? n_big : L.G_total;
-      int c = (maxNp + sub - 1) / sub;
-      c = c < 1 ? 1 : (c > 8 ? 8 : c);
-      while (c > 1 && (long long)n * c > 4LL * h->sms) c >>= 1;
-      h->rs_cluster = c;
-      h->classes.begin[0] = h->rs_by_class ? n_big : 0;
-      h->classes.cluster = c;
+      const int sub = h->rs_threads * RS_ITEMS;
+      auto cluster_for = [&](int n) {
+        int c = (maxNp + sub - 1) / sub;
+        c = c < 1 ? 1 : (c > 8 ? 8 : c);
+        while (c > 1 && (long long)n * c > 4LL * h->sms) c >>= 1;
+        return c;
+      };
+      if (n_big > 2 * h->sms) n_big = 0;
+      h->rs_by_class = !rt && n_big < L.G_total;
+      h->rs_cluster = cluster_for(L.G_total);
+      h->classes.begin[0] = n_big < L.G_total ? n_big : 0;
+      h->classes.cluster = cluster_for(n_big);
     }
     if (rt && std::atoi(rt) == RS_THREADS_SMALL) h->rs_threads = RS_THREADS_SMALL;
     if (rt && std::atoi(rt) == RS_THREADS) h->rs_threads = RS_THREADS;
@@ -900,12 +903,13 @@ pf_status pf_init(const pf_track_config* cfg, int32_t n_tracks, int32_t history,
 
 // The step's resampling (fuse = 1: with the tracks' global steps).
 static cudaError_t launch_step_resample(const pf_handle* h, int fuse, bool pdl, cudaStream_t s) {
+  ResampleArgs ra = resample_args(h, fuse);
   if (h->rs_by_class) {
-    ResampleArgs ra = resample_args(h, fuse);
     ra.glob.sum_nt = h->rs_sum_nt;
     return launch_resample_groups(ra, h->classes, pdl, s);
   }
-  return launch_resample(resample_args(h, fuse), h->G_total, h->rs_cluster, pdl, s, h->rs_threads);
+  if (h->n_tracks > 1 && h->rs_threads != h->rs_sum_nt) ra.glob.sum_nt = h->rs_sum_nt;
+  return launch_resample(ra, h->G_total, h->rs_cluster, pdl, s, h->rs_threads);
 }
 
 // The kernels of one step after frame preparation: the fused step, or
@@ -1084,10 +1088,12 @@ pf_status pf_graph_step(pf_handle* h, const float* const* table_dev, int32_t T_t
   return PF_OK;
 }
 
-// Autotuner results by problem shape (tracks, particles, groups, largest
-// group, SMs): propagate grid and resampler cluster size.
+// Autotuner results by problem shape: the device, its SMs, the patch radius,
+// and of every track the groups, their size and the method variants (which
+// decide the kernels' instances and the groups' alignment).  The propagate
+// grid, and the resampler's cluster and CTA size (0: by class of size).
 static std::mutex g_tune_mutex;
-static std::map<std::tuple<int, long long, int, int, int>, std::tuple<int, int, int>> g_tune_cache;
+static std::map<std::vector<int>, std::tuple<int, int, int>> g_tune_cache;
 
 pf_status pf_autotune(pf_handle* h, const float* const* frames, int32_t* k1_grid_out, int32_t* cluster_out,
                       void* stream) {
@@ -1098,10 +1104,12 @@ pf_status pf_autotune(pf_handle* h, const float* const* frames, int32_t* k1_grid
   for (int t = 0; t < h->n_tracks; ++t)
     if (!frames[t]) return fail(h, PF_ERR_ARG, "NULL frame pointer");
   cudaStream_t s = (cudaStream_t)stream;
-  int maxNp = 1;
-  for (int t = 0; t < h->n_tracks; ++t) maxNp = h->cfg[t].Np > maxNp ? h->cfg[t].Np : maxNp;
-  const auto key = std::make_tuple(h->n_tracks, h->N_total, h->G_total, maxNp, h->sms);
   cudaError_t e;
+  int device = 0;
+  if ((e = cudaGetDevice(&device)) != cudaSuccess) return cuda_fail(h, e, "cudaGetDevice");
+  std::vector<int> key{device, h->sms, h->R};
+  for (const pf_track_config& c : h->cfg)
+    key.insert(key.end(), {(int)c.G, (int)c.Np, (int)c.resample_rule, (int)c.send_rule});
   if ((e = prep_frames(h, frames, s)) != cudaSuccess) return cuda_fail(h, e, "k_frame_prep");
   bool cached = false;
   {

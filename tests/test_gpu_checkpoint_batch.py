@@ -118,3 +118,22 @@ def test_damaged_shapes_are_refused(dev):
     a.load(ck)
     _steps(a, frames, 1, 2)
     a.close()
+
+
+@pytest.mark.parametrize("threads", [128, 512])
+def test_weight_sum_does_not_depend_on_the_kernel(dev, threads):
+    """The same filter continued by the one-CTA classes and by the cluster
+    kernel (as the autotuner may choose it, at either CTA size): the carried
+    weights' sum keeps its order."""
+    make, frames = _make(dev, SIZES["many_groups"])
+    a = make()
+    _steps(a, frames, 0, 3)
+    ck = a.save()
+    ref = _steps(a, frames, 3, 8)
+    tuned = bytearray(ck)
+    tuned[40:52] = struct.pack("<iii", 1, threads, 0)  # cluster, CTA size, not by class
+    b = make()
+    b.load(tuned)
+    _same(_steps(b, frames, 3, 8), ref)
+    a.close()
+    b.close()
