@@ -2557,7 +2557,6 @@ __global__ void __launch_bounds__(TEAM* TEAMS, 1024 / (TEAM * TEAMS))
   __shared__ __align__(16) unsigned char s_buf[MARKS > sizeof(GlobalScratch) ? MARKS : sizeof(GlobalScratch)];
   __shared__ unsigned long long s_w[2][NW];
   __shared__ uint32_t s_m[NW];
-  __shared__ float s_f[NW];
   __shared__ float s_stat[NW][8];
   __shared__ uint32_t s_u;
   __shared__ int s_last[TEAMS];
@@ -2604,14 +2603,14 @@ __global__ void __launch_bounds__(TEAM* TEAMS, 1024 / (TEAM * TEAMS))
       (*reinterpret_cast<volatile const unsigned int*>(&a.ds->err) & (ERR_TIMEOUT | ERR_INDEX)) != 0u;
   int last_track = -1;
   if (gi < a.n_groups && !failed) {
-    const int grp = a.list ? a.list[gi] : gi;
+    const int grp = a.list[gi];
     const GroupDesc d = a.gd[grp];
     const int Np = d.Np;
-    const TrackParams* __restrict__ Pt = a.glob.trk ? a.glob.trk + d.track : nullptr;
-    const int kk = a.u_arr ? 0 : __ldcg(&a.glob.ts[d.track].k);
+    const TrackParams* __restrict__ Pt = a.glob.trk + d.track;
+    const int kk = __ldcg(&a.glob.ts[d.track].k);
     const float* __restrict__ lw = ((a.lw1 && (kk & 1)) ? a.lw1 : a.lw) + d.base;
     uint32_t* __restrict__ anc = a.anc + (kk & 1) * a.anc_stride + d.base;
-    const bool ess_rule = Pt && Pt->resample_rule == 1;
+    const bool ess_rule = Pt->resample_rule == 1;
     const int a0 = off16(lw), b0 = off16(anc);
     const int n_sub = (Np + a0 + CAP - 1) / CAP;
     auto item0 = [&](int sub) { return sub * CAP - a0 + tid * ITEMS; };  // the thread's first item
@@ -2626,31 +2625,13 @@ __global__ void __launch_bounds__(TEAM* TEAMS, 1024 / (TEAM * TEAMS))
     load_items<ITEMS>(lw, item0(0), 0, Np, v);
     uint32_t u = 0;
     if (warp == 0) {
-      u = a.u_arr ? a.u_arr[grp]
-                  : philox(Pt->key0, Pt->key1, make_uint4((uint32_t)d.g, 0u, (uint32_t)kk, Pt->tag | (ST_RESAMPLE << 4))).x;
+      u = philox(Pt->key0, Pt->key1, make_uint4((uint32_t)d.g, 0u, (uint32_t)kk, Pt->tag | (ST_RESAMPLE << 4))).x;
       if (TEAM > 32 && tid == 0) s_u = u;
     }
-    float M = -INFINITY;
-    if (a.tile_part != nullptr) {
-      const uint32_t mk = __ldcg(&a.gs[grp].mkey[kk & 1]);
-      M = mk == 0u ? -INFINITY : key_float((int)(mk ^ 0x80000000u));
-      if (tid == 0) a.gs[grp].mkey[(kk + 1) & 1] = 0u;  // for the next step's tiles
-    } else {
-      float m = -INFINITY;
-      for (int sub = 0; sub < n_sub; ++sub) {
-        if (sub > 0) load_items<ITEMS>(lw, item0(sub), 0, Np, v);
-#pragma unroll
-        for (int r = 0; r < ITEMS; ++r) m = fmaxf(m, v[r]);
-      }
-      M = warp_max(m);
-      if constexpr (TEAM > 32) {
-        if (lane == 0) s_f[warp] = M;
-        sync();
-#pragma unroll
-        for (int w = 0; w < NW; ++w) M = fmaxf(M, s_f[w]);
-      }
-      if (n_sub > 1) load_items<ITEMS>(lw, item0(0), 0, Np, v);
-    }
+    // the largest tile maximum, raised by the propagate tiles
+    const uint32_t mk = __ldcg(&a.gs[grp].mkey[kk & 1]);
+    const float M = mk == 0u ? -INFINITY : key_float((int)(mk ^ 0x80000000u));
+    if (tid == 0) a.gs[grp].mkey[(kk + 1) & 1] = 0u;  // for the next step's tiles
 
     // codes and the group's total; under Alg. 1's test also the sums of
     // c = q >> 20 and c^2
@@ -2680,7 +2661,7 @@ __global__ void __launch_bounds__(TEAM* TEAMS, 1024 / (TEAM * TEAMS))
       resample = Q == 0 || ess_below(E1, E2, (uint32_t)Np, Pt->ess_t);
     }
 
-    if (a.tile_part != nullptr) {
+    {
       // group estimate and ESS from the propagate tiles' partial sums, each
       // tile's sums rescaled from its own maximum to the group maximum
       GroupState& G = a.gs[grp];
@@ -2726,13 +2707,10 @@ __global__ void __launch_bounds__(TEAM* TEAMS, 1024 / (TEAM * TEAMS))
       }
     }
 
-    const unsigned long long obase = a.local_idx ? 0ull : (unsigned long long)d.g * (unsigned long long)Np;
+    const unsigned long long obase = (unsigned long long)d.g * (unsigned long long)Np;
     if (Q == 0 || !resample) {
       // no finite weight, or Alg. 1's test keeps the particles: identity
-      for (int i = tid; i < Np; i += TEAM) {
-        anc[i] = (uint32_t)(obase + i);
-        if (a.q_out) a.q_out[d.base + i] = 0ull;
-      }
+      for (int i = tid; i < Np; i += TEAM) anc[i] = (uint32_t)(obase + i);
     } else {
       FastCount fc;
       fc.init(Q, (uint32_t)Np, u);
@@ -2751,10 +2729,6 @@ __global__ void __launch_bounds__(TEAM* TEAMS, 1024 / (TEAM * TEAMS))
           scan(tsum, excl, tot);
         }
         const int i0 = item0(sub);
-        if (a.q_out)
-#pragma unroll
-          for (int r = 0; r < ITEMS; ++r)
-            if (i0 + r >= 0 && i0 + r < Np) a.q_out[d.base + i0 + r] = qv[r];
         const int jh = sub + 1 < n_sub ? count_fast(fc, carry + tot, Q, (uint32_t)Np, u) : Np;
         // windows of CAP outputs from a 16-byte boundary of the ancestors
         for (int w0 = ((jl + b0) & ~3) - b0; w0 < jh; w0 += CAP) {

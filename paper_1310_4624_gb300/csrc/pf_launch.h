@@ -164,7 +164,7 @@ struct ResampleArgs {
   int* tile_ctr;               // propagate kernel's tile counter to reset, or nullptr
   GlobalArgs glob;             // (fuse_global) arguments of that step, finalize = 1
   // launch_resample_groups: the groups of this launch
-  const int* list;             // global group indices, or nullptr (0 .. n_groups - 1)
+  const int* list;             // global group indices; k_resample: nullptr stands for 0 .. n_groups - 1
   int wait_last;               // 1: a launch behind another class of the same step, which waits for that one
                                // at its end instead of its start
 };
