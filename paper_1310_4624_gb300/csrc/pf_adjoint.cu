@@ -51,32 +51,10 @@ struct PixelSource {
   }
 };
 
-// A patch's pixels: from the staged box or from the frame.
+// A patch's pixels from the staged box (from the frame: FramePatch).
 struct StagedRows {
   const float* base;
-  __device__ __forceinline__ float one(int b, int a) const { return base[b * ROI_W + a]; }
-};
-// From the frame, with one bit per row and per column of the patch that lies
-// inside it: the test of a pixel is one bit at a constant place, and its load
-// is predicated, whether the patch crosses an edge or not (a few lanes of
-// nearly every warp of scattered patches do).
-struct FrameRows {
-  const float* base;  // the patch's first pixel (outside the frame if the patch crosses an edge)
-  int w;
-  uint32_t rows, cols;
-  float bg;
-  __device__ __forceinline__ FrameRows(const PixelSource& px, int u, int v, int D)
-      : base(px.z + (long long)(v - px.sub) * px.w + (u - px.sub)), w(px.w), rows(bits(v - px.sub, D, px.h)),
-        cols(bits(u - px.sub, D, px.w)), bg(px.bg) {}
-  // bit i: 0 <= first + i < n, for i < D
-  static __device__ __forceinline__ uint32_t bits(int first, int D, int n) {
-    const int lo = min(max(-first, 0), D), hi = min(max(n - first, 0), D);
-    return ((1u << hi) - 1u) & ~((1u << lo) - 1u);
-  }
-  __device__ __forceinline__ float one(int b, int a) const {
-    const uint32_t m = ((rows >> b) & 1u) ? cols : 0u;
-    return ((m >> a) & 1u) ? __fsub_rn(__ldg(base + (long long)b * w + a), bg) : 0.0f;
-  }
+  __device__ __forceinline__ float operator()(int b, int a) const { return base[b * ROI_W + a]; }
 };
 
 // Log-likelihood (Sec. V model) and its partial derivatives for the
@@ -116,7 +94,7 @@ __device__ __forceinline__ float loglik_grad(const Rows& px, const Gy& gy, int H
       float R0 = 0.0f, R1 = 0.0f, R2 = 0.0f, Rb = 0.0f;
 #pragma unroll
       for (int a = 0; a < D; ++a) {
-        const float yv = px.one(b, a);  // y = z - b, 0 outside the frame
+        const float yv = px(b, a);  // y = z - b, 0 outside the frame
         const float r = fmaf(-gx[a], Igy, yv);
         ss = fmaf(r, r, ss);
         Y2 = fmaf(yv, yv, Y2);
@@ -218,7 +196,8 @@ __device__ __noinline__ float2 replay_off_box(const ReplayArgs& a, const TrackPa
     const float4 s = a.pv_out[i];
     const float I = a.I_out[i];
     const float lb = k >= 1 ? a.lbar_prev[P.group_off + (int)fastdiv(par_t[il], P.m_Np)] : -log_G;
-    const FrameRows rows(px, patch_corner<R>(s.x, P.W), patch_corner<R>(s.y, P.H), D);
+    const FramePatch rows(px.z, px.w, px.h, px.bg, patch_corner<R>(s.x, P.W) - px.sub,
+                          patch_corner<R>(s.y, P.H) - px.sub, D);
     float ss;
     {
       float gxI[D];
@@ -226,9 +205,8 @@ __device__ __noinline__ float2 replay_off_box(const ReplayArgs& a, const TrackPa
 #pragma unroll
       for (int c = 0; c < D; ++c) gxI[c] *= I;
       const float dy = floorf(s.y + 0.5f) - s.y;
-      auto pix = [&](int b, int c) { return rows.one(b, c); };
-      ss = P.obs_model == 1 ? patch_sum<R, true>(pix, gxI, dy, P.c_psf, P.kappa)
-                            : patch_sum<R, false>(pix, gxI, dy, P.c_psf, P.kappa);
+      ss = P.obs_model == 1 ? patch_sum<R, true>(rows, gxI, dy, P.c_psf, P.kappa)
+                            : patch_sum<R, false>(rows, gxI, dy, P.c_psf, P.kappa);
     }
     weigh(lb - log_Np - ss * P.inv2so2, mx, sm);
     if (a.dl_pv) {

@@ -506,17 +506,31 @@ K1Args k1_args(const pf_handle* h) {
   return a;
 }
 
+// Steps after a start that spreads the population, over which its tiles do not
+// fit staging boxes (a sharing start gathers within about five frames).
+constexpr int SPREAD_STEPS = 8;
+
 // A single-track step reads the caller's frame directly (no frame
 // preparation kernel): by TMA when a descriptor can describe it (the driver
 // entry point is available, the frame starts on 16 bytes, its rows are a
 // multiple of 16 bytes and it holds at least one staging box), else by plain
-// loads.  Returns false, and leaves `a` unchanged, for several tracks.
+// loads.  Returns false, and leaves `a` unchanged, for several tracks, for a
+// fused step with method variants, whose instance serves any track count, and
+// while a population that starts spread has not had time to gather, where
+// method variants or plain loads would pay for bounds checks on every pixel
+// (step of 64 x 16384 spread particles from the caller's frame and prepared:
+// with variants 144 and 102 us; odd frame, radius 7, 165 and 147, radius 5, 104
+// and 98.  Gathered, the launch of the preparation is what counts: 54 and 64,
+// 61 and 67, 50 and 56).
 bool raw_frame_map(const pf_handle* h, const float* frame, K1Args* a) {
-  if (h->n_tracks != 1 || !frame) return false;
+  if (h->n_tracks != 1 || !frame || (h->fused && h->variants)) return false;
   const pf_track_config& c = h->cfg[0];
+  const bool tma =
+      h->encode && ((uintptr_t)frame & 15) == 0 && (c.W % 4) == 0 && c.W >= ROI_W && c.H >= ROI_BOX_H;
+  if (c.init_kind != PF_INIT_POINT && h->steps_run < SPREAD_STEPS && (h->variants || !tma)) return false;
   a->raw_frame = RAW_FRAME_LOADS;
   a->zraw = frame;
-  if (!h->encode || ((uintptr_t)frame & 15) != 0 || (c.W % 4) != 0 || c.W < ROI_W || c.H < ROI_BOX_H) return true;
+  if (!tma) return true;
   cuuint64_t dims[2] = {(cuuint64_t)c.W, (cuuint64_t)c.H};
   cuuint64_t strides[1] = {(cuuint64_t)c.W * sizeof(float)};
   cuuint32_t box[2] = {(cuuint32_t)ROI_W, (cuuint32_t)ROI_BOX_H};

@@ -911,14 +911,41 @@ constexpr size_t FUSED_SMEM = sizeof(unsigned long long) * pad8(RS_CHUNK) + size
 constexpr size_t ROI_SMEM = sizeof(float) * 2 * (ROI_FLOATS + 4);
 static_assert(ROI_SMEM <= FUSED_SMEM && sizeof(GlobalScratch) <= FUSED_SMEM, "fused step shared memory");
 
+// From this radius on, tiles off the staging box read the caller's frame out
+// of line: the patch's row then takes so many registers that its loads run one
+// by one (step of 64 x 16384 spread particles at radius 7, 223 us in line and
+// 165 out of line).  Below, in line is faster (radius 5: 105 and 113, and the
+// staged path keeps its registers, 50.2 and 50.9 us; radius 3: 67 and 71).
+constexpr int RAW_OUT_OF_LINE_R = 6;
+
+// The log-weights of a tile of n slots whose patches do not fit the staging
+// box, from the caller's frame: lw holds the particles' weight offsets and
+// gets the log-likelihoods added.  Out of line, from the states that the tile
+// has just stored, so that nothing of it takes registers of the staged path.
+template <int R>
+__device__ __noinline__ void weigh_off_box(const float* __restrict__ z, const TrackParams& P, int n, const float4* pv,
+                                           const float* In, float* lw) {
+  for (int jj = threadIdx.x; jj < n; jj += K1_THREADS) {
+    const float4 s = pv[jj];
+    const float cx = floorf(s.x + 0.5f), cy = floorf(s.y + 0.5f);
+    // (the centre clamped so that a patch wholly off the frame reads background)
+    const FramePatch pix(z, P.W, P.H, P.bg, (int)fminf(fmaxf(cx, -(float)(R + 1)), (float)(P.W + R)) - R,
+                         (int)fminf(fmaxf(cy, -(float)(R + 1)), (float)(P.H + R)) - R, 2 * R + 1);
+    float gxI[2 * R + 1];
+    gauss_row_scaled<R>(cx, s.x, P.c_psf, P.kappa, In[jj], gxI);
+    const float ss = P.obs_model == 1 ? patch_sum<R, true>(pix, gxI, cy - s.y, P.c_psf, P.kappa)
+                                      : patch_sum<R, false>(pix, gxI, cy - s.y, P.c_psf, P.kappa);
+    lw[jj] = fmaf(-ss, P.inv2so2, lw[jj]);
+  }
+}
+
 // Propagate + weight: tiles of K1_TILE = K1_PPT x K1_THREADS slots of one
 // group, K1_PPT particles per thread.  Each tile stages the bounding box of
 // its particles' patches (at most ROI_W x ROI_ROWS floats) in shared memory,
 // by TMA, or by plain loads from a frame that no TMA descriptor can describe
 // (rows off the 16-byte grid: padding it first took a launch a step, 7 us of
-// 32 on 33 x 3001 particles, 6 of 37 on 95 x 1269 with method variants, whose
-// instance spills a few registers for it); tiles whose patches do not fit read the frame
-// through L1.
+// 32 on 33 x 3001 particles, 6 of 37 on 95 x 1269 with method variants); tiles
+// whose patches do not fit read the frame through L1.
 // Leading blocks draw the next step's rings and exchange offsets and finish
 // the previous step.
 // SINGLE: one track, whose parameters come from the kernel's constant
@@ -1154,7 +1181,7 @@ __global__ void __launch_bounds__(K1_THREADS, K1_MIN_BLOCKS) k_propagate_weight(
     }
     // raw frame by TMA: the box's left edge on a 4-float boundary of the
     // frame (a TMA requirement), in padded coordinates
-    const bool raw = (SINGLE || VARIANTS) && a.raw_frame;
+    const bool raw = SINGLE && a.raw_frame;
     const bool plain = raw && a.raw_frame == RAW_FRAME_LOADS;  // (any box: no copy engine, no alignment)
     const int u0 = plain ? umin : raw ? (((umin - PAD) & ~3) + PAD) : (umin & ~3);
     const int nbox = (vmax + D - vmin + ROI_BOX_H - 1) / ROI_BOX_H;
@@ -1237,52 +1264,75 @@ __global__ void __launch_bounds__(K1_THREADS, K1_MIN_BLOCKS) k_propagate_weight(
 
     // Alg. 1 step U with the renormalised carried weight (Alg. 3 step 4)
     float lw[K1_PPT];
+    if (SINGLE && R >= RAW_OUT_OF_LINE_R && raw && !staged) {
 #pragma unroll
-    for (int q = 0; q < K1_PPT; ++q) {
-      const int jj = threadIdx.x + q * K1_THREADS;
-      lw[q] = -INFINITY;
-      if (jj < td.w) {
-        float gxI[D];  // I gx(u), u = cx - R .. cx + R
-        gauss_row_scaled<R>(floorf(s[q].x + 0.5f), s[q].x, P.c_psf, P.kappa, I[q], gxI);
-        const float dy = floorf(s[q].y + 0.5f) - s[q].y;
-        float ss;
-        const bool frame_model = P.obs_model == 1;
-        if (staged) {
-          const int c = pu[q] - u0, o = (pv[q] - vmin) * ROI_W;
-#ifdef PF_DEBUG
-          // first and last floats the pairwise row loads touch
-          if (o + c - (c & 1) < 0 || o + c - (c & 1) + 2 * R * ROI_W + 2 * R + 1 >= ROI_FLOATS + 4) {
-            set_error(a.ds, ERR_DEBUG, 103u, (uint32_t)(o + c), (uint32_t)(ROI_FLOATS + 4));
-            ss = 0.0f;
-          } else
-#endif
-          {
-            const float* base = (c & 1) ? &s_roi[1][o + c - 1] : &s_roi[0][o + c];
-            ss = frame_model ? patch_ss_pairs<R, true>(base, gxI, dy, P.c_psf, P.kappa)
-                             : patch_ss_pairs<R, false>(base, gxI, dy, P.c_psf, P.kappa);
-          }
-        } else if (raw) {
-          ss = frame_model
-                   ? patch_ss_raw<R, true>(a.zraw, P.W, P.H, P.bg, pu[q] - PAD, pv[q] - PAD, gxI, dy, P.c_psf, P.kappa)
-                   : patch_ss_raw<R, false>(a.zraw, P.W, P.H, P.bg, pu[q] - PAD, pv[q] - PAD, gxI, dy, P.c_psf,
-                                            P.kappa);
-        } else {
-#ifdef PF_DEBUG
-          // the patch inside the padded frame (H + 2 PAD rows of P.pitch floats)
-          if (pu[q] < 0 || pu[q] + 2 * R >= P.pitch || pv[q] < 0 || pv[q] + 2 * R >= P.H + 2 * PAD) {
-            set_error(a.ds, ERR_DEBUG, 104u, (uint32_t)pu[q], (uint32_t)pv[q]);
-            ss = 0.0f;
-          } else
-#endif
-          {
-            const float* base = a.ypad + ypad_off + (long long)pv[q] * P.pitch + pu[q];
-            ss = frame_model ? patch_ss<R, true, false>(base, P.pitch, gxI, dy, P.c_psf, P.kappa)
-                             : patch_ss<R, false, false>(base, P.pitch, gxI, dy, P.c_psf, P.kappa);
-          }
+      for (int q = 0; q < K1_PPT; ++q) {
+        const int jj = threadIdx.x + q * K1_THREADS;
+        const bool carried = VARIANTS && ((cmask >> (from_pred[q] ? 1 : 0)) & 1);  // (its offset is there already)
+        if (jj < td.w && !carried) lw_t[g * Np + td.z + jj] = from_pred[q] ? off_s : off_g;
+      }
+      const int i0 = g * Np + td.z;
+      weigh_off_box<R>(a.zraw, P, td.w, pvc_t + i0, Ic_t + i0, lw_t + i0);
+#pragma unroll
+      for (int q = 0; q < K1_PPT; ++q) {
+        const int jj = threadIdx.x + q * K1_THREADS;
+        lw[q] = -INFINITY;
+        s[q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        I[q] = 0.0f;
+        if (jj < td.w) {
+          s[q] = pvc_t[i0 + jj];
+          I[q] = Ic_t[i0 + jj];
+          lw[q] = lw_t[i0 + jj];
         }
-        const bool carried = VARIANTS && ((cmask >> (from_pred[q] ? 1 : 0)) & 1);
-        lw[q] = fmaf(-ss, P.inv2so2, carried ? lw_t[g * Np + td.z + jj] : (from_pred[q] ? off_s : off_g));
-        lw_t[g * Np + td.z + jj] = lw[q];
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < K1_PPT; ++q) {
+        const int jj = threadIdx.x + q * K1_THREADS;
+        lw[q] = -INFINITY;
+        if (jj < td.w) {
+          float gxI[D];  // I gx(u), u = cx - R .. cx + R
+          gauss_row_scaled<R>(floorf(s[q].x + 0.5f), s[q].x, P.c_psf, P.kappa, I[q], gxI);
+          const float dy = floorf(s[q].y + 0.5f) - s[q].y;
+          float ss;
+          const bool frame_model = P.obs_model == 1;
+          if (staged) {
+            const int c = pu[q] - u0, o = (pv[q] - vmin) * ROI_W;
+#ifdef PF_DEBUG
+            // first and last floats the pairwise row loads touch
+            if (o + c - (c & 1) < 0 || o + c - (c & 1) + 2 * R * ROI_W + 2 * R + 1 >= ROI_FLOATS + 4) {
+              set_error(a.ds, ERR_DEBUG, 103u, (uint32_t)(o + c), (uint32_t)(ROI_FLOATS + 4));
+              ss = 0.0f;
+            } else
+#endif
+            {
+              const float* base = (c & 1) ? &s_roi[1][o + c - 1] : &s_roi[0][o + c];
+              ss = frame_model ? patch_ss_pairs<R, true>(base, gxI, dy, P.c_psf, P.kappa)
+                               : patch_ss_pairs<R, false>(base, gxI, dy, P.c_psf, P.kappa);
+            }
+          } else if (R < RAW_OUT_OF_LINE_R && raw) {
+            ss = frame_model ? patch_ss_raw<R, true>(a.zraw, P.W, P.H, P.bg, pu[q] - PAD, pv[q] - PAD, gxI, dy, P.c_psf,
+                                                     P.kappa)
+                             : patch_ss_raw<R, false>(a.zraw, P.W, P.H, P.bg, pu[q] - PAD, pv[q] - PAD, gxI, dy,
+                                                      P.c_psf, P.kappa);
+          } else {
+#ifdef PF_DEBUG
+            // the patch inside the padded frame (H + 2 PAD rows of P.pitch floats)
+            if (pu[q] < 0 || pu[q] + 2 * R >= P.pitch || pv[q] < 0 || pv[q] + 2 * R >= P.H + 2 * PAD) {
+              set_error(a.ds, ERR_DEBUG, 104u, (uint32_t)pu[q], (uint32_t)pv[q]);
+              ss = 0.0f;
+            } else
+#endif
+            {
+              const float* base = a.ypad + ypad_off + (long long)pv[q] * P.pitch + pu[q];
+              ss = frame_model ? patch_ss<R, true, false>(base, P.pitch, gxI, dy, P.c_psf, P.kappa)
+                               : patch_ss<R, false, false>(base, P.pitch, gxI, dy, P.c_psf, P.kappa);
+            }
+          }
+          const bool carried = VARIANTS && ((cmask >> (from_pred[q] ? 1 : 0)) & 1);
+          lw[q] = fmaf(-ss, P.inv2so2, carried ? lw_t[g * Np + td.z + jj] : (from_pred[q] ? off_s : off_g));
+          lw_t[g * Np + td.z + jj] = lw[q];
+        }
       }
     }
 
@@ -2930,13 +2980,15 @@ cudaError_t fused_occupancy(int R, int* blocks_per_sm) {
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, K1_THREADS, FUSED_SMEM);
 }
 
-// Instances: one track, several tracks, and tracks that use a method
-// variant (groups that carry their particles' own weights under Alg. 1's
-// resampling test, or keyed send sets; any track count).
+// Instances: one track or several, with and without the method variants
+// (groups that carry their particles' own weights under Alg. 1's resampling
+// test, or keyed send sets).  Only the one-track instances read the caller's
+// frame, so the others spill nothing for it.
 template <int R>
 static cudaError_t launch_propagate_r(const K1Args& a, dim3 g, bool pdl, cudaStream_t s) {
+  if (a.n_tracks == 1)
+    return a.variants ? launch_propagate_rs<R, true, true>(a, g, pdl, s) : launch_propagate_rs<R, true, false>(a, g, pdl, s);
   if (a.variants) return launch_propagate_rs<R, false, true>(a, g, pdl, s);
-  if (a.n_tracks == 1) return launch_propagate_rs<R, true, false>(a, g, pdl, s);
   return launch_propagate_rs<R, false, false>(a, g, pdl, s);
 }
 

@@ -89,7 +89,7 @@ struct K1Args {
   const float* zraw;
   int test_withhold_copy;    // failure-detection test: issue no staging copy, so the bounded wait runs out
   int variants;              // 1: some track resamples by Alg. 1's test (groups may carry weights) or
-                             // uses keyed send sets: launches the variants instance (frames prepared)
+                             // uses keyed send sets: launches a variants instance
   uint4* keys_next;          // two buffers (by step parity) of G_total: keyed send-permutation keys of step k+1
   const int* frame_of;       // per track: the track whose padded frame to read this step, or nullptr (its own)
   // fused step (one persistent launch per step): the resampling chunks,

@@ -251,6 +251,31 @@ __device__ __forceinline__ float patch_ss_raw(const float* __restrict__ z, int W
       gxI, dy, c, kappa);
 }
 
+// Bit i: pixel first + i of one axis lies in the frame (0 <= first + i < n), for i < D.
+__device__ __forceinline__ uint32_t inside_bits(int first, int D, int n) {
+  const int lo = min(max(-first, 0), D), hi = min(max(n - first, 0), D);
+  return ((1u << hi) - 1u) & ~((1u << lo) - 1u);
+}
+
+// A patch of the caller's frame z (w x h, pitch w) with its corner at
+// (x0, y0), instead of the padded frame: pixel values z - bg inside the frame,
+// 0 outside.  One bit per row and per column says what lies inside: the test
+// of a pixel is a bit at a constant place and its load is predicated, whether
+// the patch crosses an edge or not (a few lanes of nearly every warp of
+// scattered patches do), with one address per row.
+struct FramePatch {
+  const float* base;  // pixel (x0, y0), outside the frame if the patch crosses an edge
+  int w;
+  uint32_t rows, cols;
+  float bg;
+  __device__ __forceinline__ FramePatch(const float* z, int w_, int h, float bg_, int x0, int y0, int D)
+      : base(z + (long long)y0 * w_ + x0), w(w_), rows(inside_bits(y0, D, h)), cols(inside_bits(x0, D, w_)), bg(bg_) {}
+  __device__ __forceinline__ float operator()(int b, int a) const {
+    const uint32_t m = ((rows >> b) & 1u) ? cols : 0u;
+    return ((m >> a) & 1u) ? __fsub_rn(__ldg(base + (long long)b * w + a), bg) : 0.0f;
+  }
+};
+
 // Natural log of a uniform u = ((w >> 9) + 1/2) 2^-23: MUFU log2 where its
 // absolute error (2^-22 on [1/2, 2]) is small against |ln u|, and the series
 // -(t + t^2/2 + t^3/3), t = 1 - u, for the top 2^-10 of the interval.
