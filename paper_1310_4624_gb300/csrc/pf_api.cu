@@ -1737,6 +1737,19 @@ pf_status pf_load(pf_handle* h, const void* host, size_t bytes, void* stream) {
                            h->ws_total - h->tmap_off - h->tmap_bytes, cudaMemcpyHostToDevice, s)) ||
       (e = cudaStreamSynchronize(s)))
     return cuda_fail(h, e, "pf_load");
+  // the saved parameters (pf_set_theta), of which single-track launches take
+  // the host's copy
+  if ((e = cudaMemcpy(h->tp.data(), h->trk, sizeof(TrackParams) * h->tp.size(), cudaMemcpyDeviceToHost)) != cudaSuccess)
+    return cuda_fail(h, e, "pf_load");
+  for (int t = 0; t < h->n_tracks; ++t) {
+    pf_track_config& c = h->cfg[t];
+    const TrackParams& P = h->tp[t];
+    c.sigma_psf = P.spsf;
+    c.init_state[4] = P.init_state[4];
+    c.background = P.bg;
+    c.sigma_pos = P.spos;
+    c.sigma_v = P.sv;
+  }
   h->steps_run = hd.steps_run;
   h->finish_pending = hd.finish_pending != 0;
   h->k1_grid = hd.k1_grid;
