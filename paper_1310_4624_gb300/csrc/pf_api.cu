@@ -1473,6 +1473,10 @@ pf_status pf_set_theta(pf_handle* h, int32_t track, const float* theta) {
   P.sv = sv;
   cudaError_t e = cudaMemcpy(h->trk + track, &P, sizeof(TrackParams), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return cuda_fail(h, e, "uploading track parameters");
+  if (h->graph) {  // a captured single-track step holds the old parameters
+    cudaGraphExecDestroy(h->graph);
+    h->graph = nullptr;
+  }
   return PF_OK;
 }
 
