@@ -365,11 +365,17 @@ int num_sms() {
 // for groups that not even 16 CTAs hold in their registers, while 8 each would
 // leave SMs idle: 320 -> 189 us for one group of 2^20, 128 -> 92 us for four of
 // 2^18.  Groups that fit gain nothing (8 x 100000: 72 and 73 us; 16 x 65536: 61
-// and 64 us).
-int resample_cluster(int G, int Np, int pad) {
-  const int c = (Np + pad + RS_SUB - 1) / RS_SUB;
+// and 64 us).  off: elements that groups may start off a 16-byte boundary by;
+// where room for them alone takes one more CTA per group and those CTAs would
+// not run at once (two per SM), the groups go without: launch_resample drops
+// the vectors (the step of 256 x 4095 particles, 512 CTAs: 61 us with them, 53
+// without; of 128 x 8191, 384 CTAs: 59 and 53; of 128 x 4095, 256 CTAs: 36 and
+// 39).
+int resample_cluster(int G, int Np, int off) {
+  auto clamp = [](int c) { return c < 1 ? 1 : (c > 8 ? 8 : c); };
+  const int c = (Np + off + RS_SUB - 1) / RS_SUB, c0 = (Np + RS_SUB - 1) / RS_SUB;
   if (c > 32 && 8ll * G < num_sms()) return resample_max_cluster();
-  return c < 1 ? 1 : (c > 8 ? 8 : c);
+  return clamp(c) > clamp(c0) && (long long)G * clamp(c) > 2ll * num_sms() ? clamp(c0) : clamp(c);
 }
 
 pf_status check_device(pf_handle* h) {
@@ -883,7 +889,6 @@ pf_status pf_init(const pf_track_config* cfg, int32_t n_tracks, int32_t history,
     const char* rt = std::getenv("PFARNA_RS_THREADS");  // "128" / "512": the cluster kernel with CTAs of this size
     if (n_tracks == 1) {
       h->rs_cluster = resample_cluster(cfg[0].G, cfg[0].Np, h->rs_pad);
-      if (h->rs_threads == RS_THREADS_SMALL && maxNp + h->rs_pad > RS_THREADS_SMALL * RS_ITEMS) h->rs_cluster = 2;
     } else {
       // clusters sized to the largest group, as long as their launch stays
       // within about two waves of two CTAs per SM

@@ -2114,16 +2114,17 @@ __device__ __forceinline__ int count_fast(const FastCount& fc, unsigned long lon
   return c;
 }
 
-// ITEMS log-weights of a group at its items i0 .. i0 + ITEMS - 1 (a multiple
-// of four items from a 16-byte boundary), -inf outside [lo, hi): whole float4
-// inside the range, single loads at its ends.  Through L2: one 32-byte sector
-// per thread and no line to keep.
+// ITEMS log-weights of a group at its items i0 .. i0 + ITEMS - 1, -inf outside
+// [lo, hi): whole float4 inside the range (vec: i0 is a multiple of four items
+// from a 16-byte boundary), single loads at its ends.  Through L2: one 32-byte
+// sector per thread and no line to keep.
 template <int ITEMS>
-__device__ __forceinline__ void load_items(const float* __restrict__ lw, int i0, int lo, int hi, float (&v)[ITEMS]) {
+__device__ __forceinline__ void load_items(const float* __restrict__ lw, int i0, int lo, int hi, float (&v)[ITEMS],
+                                           bool vec = true) {
 #pragma unroll
   for (int r = 0; r < ITEMS; r += 4) {
     const int i = i0 + r;
-    if (i >= lo && i + 4 <= hi) {
+    if (vec && i >= lo && i + 4 <= hi) {
       const float4 x = __ldcg(reinterpret_cast<const float4*>(lw + i));
       v[r] = x.x; v[r + 1] = x.y; v[r + 2] = x.z; v[r + 3] = x.w;
     } else {
@@ -2133,15 +2134,15 @@ __device__ __forceinline__ void load_items(const float* __restrict__ lw, int i0,
   }
 }
 
-// Ancestors of ITEMS consecutive outputs j0 .. (a multiple of four outputs
-// from a 16-byte boundary), those in [lo, hi) stored.
+// Ancestors of ITEMS consecutive outputs j0 .. (vec: a multiple of four
+// outputs from a 16-byte boundary), those in [lo, hi) stored.
 template <int ITEMS>
 __device__ __forceinline__ void store_items(uint32_t* __restrict__ anc, int j0, int lo, int hi,
-                                            const uint32_t (&o)[ITEMS]) {
+                                            const uint32_t (&o)[ITEMS], bool vec = true) {
 #pragma unroll
   for (int r = 0; r < ITEMS; r += 4) {
     const int j = j0 + r;
-    if (j >= lo && j + 4 <= hi) {
+    if (vec && j >= lo && j + 4 <= hi) {
       *reinterpret_cast<uint4*>(anc + j) = make_uint4(o[r], o[r + 1], o[r + 2], o[r + 3]);
     } else {
 #pragma unroll
@@ -2187,7 +2188,8 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? (ITEMS > RS_ITEMS ? 1 : 2) :
   // LEAN: items and outputs are split in units of the 16-byte boundaries of
   // their arrays: a0 (b0) elements of the first item's (output's) float4 lie
   // before the group, so that every load and store of a group at any offset
-  // is a whole vector except at the group's two ends
+  // is a whole vector except at the group's two ends (pad = 0: in units of the
+  // group's own start, by single loads and stores where that is off the grid)
   const int chunk = LEAN ? rs_chunk_lean(Np, C, a.pad) : ((Np + C - 1) / C + 7) & ~7;
   // In a filter step: the track's step index (read before the cluster
   // barrier that precedes every ticket below, since the track's global step,
@@ -2196,12 +2198,12 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? (ITEMS > RS_ITEMS ? 1 : 2) :
   const TrackParams* __restrict__ Pt = a.glob.trk ? a.glob.trk + d.track : nullptr;
   const int kk = a.u_arr ? 0 : a.glob.ts[d.track].k;
   const float* __restrict__ lw = ((a.lw1 && (kk & 1)) ? a.lw1 : a.lw) + d.base;
-  const int a0 = LEAN ? off16(lw) : 0;
+  const int a0 = LEAN && a.pad ? off16(lw) : 0;
   const int lo = LEAN ? max(rank * chunk - a0, 0) : min(rank * chunk, Np);
   const int hi = LEAN ? min((rank + 1) * chunk - a0, Np) : min(lo + chunk, Np);
   const bool single = LEAN || (hi - lo) <= SUB;  // the whole chunk stays in registers
   const bool ess_rule = EXTRA && Pt && Pt->resample_rule == 1;
-  const bool vec = off16(lw) == 0;
+  const bool vec = off16(lw) == a0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
   __shared__ float s_pub_max;
@@ -2226,7 +2228,7 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? (ITEMS > RS_ITEMS ? 1 : 2) :
   float v[ITEMS];
   auto load_sub = [&](int sub) {
     if constexpr (LEAN) {
-      load_items<ITEMS>(lw, rank * chunk - a0 + (int)threadIdx.x * ITEMS, lo, hi, v);
+      load_items<ITEMS>(lw, rank * chunk - a0 + (int)threadIdx.x * ITEMS, lo, hi, v, vec);
     } else {
       const int i0 = sub + (int)threadIdx.x * ITEMS;
       if (vec && i0 + ITEMS <= hi) {
@@ -2456,7 +2458,7 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? (ITEMS > RS_ITEMS ? 1 : 2) :
 #pragma unroll
         for (int r = 0; r < ITEMS; ++r)
           if (i0 + r >= lo && i0 + r < hi) a.q_out[d.base + i0 + r] = qv[r];
-      const int b0 = off16(anc);  // outputs in units of the ancestors' 16-byte boundaries
+      const int b0 = a.pad ? off16(anc) : 0;  // outputs in units of the ancestors' 16-byte boundaries
       int c = count_fast(fc, S, Q, (uint32_t)Np, u) + b0;
 #pragma unroll
       for (int r = 0; r < ITEMS; ++r) {
@@ -2547,7 +2549,8 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? (ITEMS > RS_ITEMS ? 1 : 2) :
     if (Q != 0 && resample) {
       // running maximum over this CTA's positions (the first one that holds
       // an output of the group always holds a mark)
-      const int j0 = rank * chunk - off16(anc) + (int)threadIdx.x * ITEMS;  // the thread's first output
+      const int b0 = a.pad ? off16(anc) : 0;
+      const int j0 = rank * chunk - b0 + (int)threadIdx.x * ITEMS;  // the thread's first output
       uint32_t m[ITEMS];
 #pragma unroll
       for (int r = 0; r < ITEMS; r += 4) {
@@ -2569,12 +2572,12 @@ __global__ void __launch_bounds__(NTR, NTR >= 512 ? (ITEMS > RS_ITEMS ? 1 : 2) :
 #pragma unroll
       for (int w = 0; w < NTR / 32; ++w)
         if (w < warp) pre = max(pre, (uint32_t)s_w[w]);
-      const int jhi = min((rank + 1) * chunk - off16(anc), Np);
+      const int jhi = min((rank + 1) * chunk - b0, Np);
       if (j0 >= 0 && j0 < jhi && max(pre, m[0]) == 0u) set_error(a.ds, ERR_INVARIANT, 12u, (uint32_t)grp, (uint32_t)j0);
       uint32_t o[ITEMS];
 #pragma unroll
       for (int r = 0; r < ITEMS; ++r) o[r] = (uint32_t)(obase + max(max(m[r], pre), 1u) - 1u);
-      store_items<ITEMS>(anc, j0, 0, jhi, o);
+      store_items<ITEMS>(anc, j0, 0, jhi, o, off16(anc) == b0);
     }
   }
 
@@ -3061,9 +3064,16 @@ static cudaError_t launch_resample_t(const ResampleArgs& a, int n_groups, int cl
   return launch_ex(k_resample<NTR, ITEMS, LEAN, EXTRA>, dim3((unsigned)(clusters * cluster)), dim3(NTR), cluster, pdl, s, a, smem);
 }
 
-cudaError_t launch_resample(const ResampleArgs& a, int n_groups, int cluster, bool pdl, cudaStream_t s, int threads) {
+cudaError_t launch_resample(const ResampleArgs& a0, int n_groups, int cluster, bool pdl, cudaStream_t s, int threads) {
   // the lean instances while every CTA's chunk fits their registers: 8 items
-  // per thread, 16 for the largest groups (65536 particles on a cluster of 8)
+  // per thread, 16 for the largest groups (65536 particles on a cluster of 8).
+  // Room for groups off the 16-byte grid is given up where it alone would
+  // take the larger instance (the step of 64 groups of 32767: 132 us with it,
+  // 104 by single loads and stores; of 4 groups of 65535: 45 and 31).
+  ResampleArgs a = a0;
+  for (int items = RS_ITEMS; items <= 2 * RS_ITEMS; items *= 2)
+    if (rs_chunk_lean(a.max_np, cluster, 0) <= threads * items && rs_chunk_lean(a.max_np, cluster, a.pad) > threads * items)
+      a.pad = 0;
   const long long chunk = rs_chunk_lean(a.max_np, cluster, a.pad);
   const bool small = threads == RS_THREADS_SMALL, extra = !a.lean || a.q_out;
   if (chunk <= (long long)threads * RS_ITEMS) {

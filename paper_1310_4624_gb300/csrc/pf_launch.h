@@ -161,6 +161,7 @@ struct ResampleArgs {
   int lean;                    // 1: no group under Alg. 1's test
   int max_np;                  // the largest group of the launch (for that test)
   int pad;                     // 0: every group starts on 16 bytes of the log-weights and the ancestors, else 3
+                               // (to the kernel: 0 also where groups off the grid go without vectors)
   int* tile_ctr;               // propagate kernel's tile counter to reset, or nullptr
   GlobalArgs glob;             // (fuse_global) arguments of that step, finalize = 1
   // launch_resample_groups: the groups of this launch
@@ -295,7 +296,7 @@ const void* propagate_kernel(int R);
 // Host helpers shared by the C-ABI entry points (defined in pf_api.cu).
 QuantCoeffs resample_coeffs();             // weight-code coefficients
 int resample_cluster_size(int G, int Np, int pad);  // resampler cluster size for one group of Np
-// ResampleArgs::pad for G groups of Np in a caller's arrays
+// ResampleArgs::pad for G groups of Np in a caller's arrays (the cluster kernel at RS_THREADS)
 int resample_pad(const float* logw, const uint32_t* anc, int G, int Np);
 void set_handleless_error(const char* msg);  // text for pf_last_error(NULL)
 // The no-allocation resampler's error word on the current device (defined
