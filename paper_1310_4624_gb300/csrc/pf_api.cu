@@ -931,6 +931,19 @@ static cudaError_t launch_step_resample(const pf_handle* h, int fuse, bool pdl, 
   return launch_resample(ra, h->G_total, h->rs_cluster, pdl, s, h->rs_threads);
 }
 
+// The propagate kernel's split of shared memory and cache, in percent, or -1
+// for the driver's choice.  The general resampler's CTAs take 74 KB each; next
+// to the choice for the propagate kernel's 21 KB that makes every SM drain
+// between the two launches of a one-track step, so that neither starts beside
+// the other.  (Step under Alg. 1's test, from a point: 3 x 65537 particles 51
+// us, 42 with the same split; 32 x 65536, 128 and 114.  After a preparation
+// launch the smaller cache costs more than the overlap gives: 196 and 204 us
+// of 32 x 65536 spread.)
+static int k1_carveout(const pf_handle* h, const K1Args& k1) {
+  if (!k1.raw_frame || resample_is_lean(resample_args(h, 1), h->rs_cluster, h->rs_threads)) return -1;
+  return 75;
+}
+
 // The kernels of one step after frame preparation: the fused step, or
 // propagate + weight, then resample with the global step as its tail.
 // marks: record profiling events (not while a graph is being captured).
@@ -943,7 +956,7 @@ static cudaError_t launch_step_kernels(pf_handle* h, cudaStream_t s, bool marks,
     return marks ? mark(h, PF_KERNEL_FUSED_STEP, s) : cudaSuccess;
   }
   if (marks && (e = mark(h, PF_KERNEL_PROPAGATE_WEIGHT, s)) != cudaSuccess) return e;
-  if ((e = launch_propagate(k1, h->R, h->k1_grid + h->n_ring_blocks, h->pdl, s)) != cudaSuccess) return e;
+  if ((e = launch_propagate(k1, h->R, h->k1_grid + h->n_ring_blocks, h->pdl, s, k1_carveout(h, k1))) != cudaSuccess) return e;
   if (marks && (e = mark(h, PF_KERNEL_PROPAGATE_WEIGHT, s)) != cudaSuccess) return e;
   if (marks && (e = mark(h, PF_KERNEL_RESAMPLE, s)) != cudaSuccess) return e;
   if ((e = launch_step_resample(h, 1, h->pdl, s)) != cudaSuccess) return e;

@@ -2890,14 +2890,19 @@ cudaError_t launch_init(const InitArgs& a, int grid, cudaStream_t s) {
 // stream serialization (see launch_* in pf_launch.h).
 template <typename... Params, typename Arg>
 static cudaError_t launch_ex(void (*kernel)(Params...), dim3 grid, dim3 block, int cluster, bool pdl,
-                             cudaStream_t s, const Arg& arg, size_t smem = 0) {
+                             cudaStream_t s, const Arg& arg, size_t smem = 0, int carveout = -1) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[2];
+  cudaLaunchAttribute attr[3];
   int n = 0;
+  if (carveout >= 0) {  // shared memory's part of an SM's shared memory and cache, percent
+    attr[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[n].val.sharedMemCarveout = (unsigned)carveout;
+    ++n;
+  }
   if (cluster > 0) {
     attr[n].id = cudaLaunchAttributeClusterDimension;
     attr[n].val.clusterDim.x = (unsigned)cluster;
@@ -2943,8 +2948,8 @@ const void* propagate_kernel(int R) {
 }
 
 template <int R, bool SINGLE, bool VARIANTS>
-static cudaError_t launch_propagate_rs(const K1Args& a, dim3 g, bool pdl, cudaStream_t s) {
-  return launch_ex(k_propagate_weight<R, SINGLE, VARIANTS, false>, g, dim3(K1_THREADS), 0, pdl, s, a);
+static cudaError_t launch_propagate_rs(const K1Args& a, dim3 g, bool pdl, cudaStream_t s, int carveout) {
+  return launch_ex(k_propagate_weight<R, SINGLE, VARIANTS, false>, g, dim3(K1_THREADS), 0, pdl, s, a, 0, carveout);
 }
 
 template <int R, bool SINGLE, bool VARIANTS>
@@ -2995,23 +3000,24 @@ cudaError_t fused_occupancy(int R, int* blocks_per_sm) {
 // test, or keyed send sets).  Only the one-track instances read the caller's
 // frame, so the others spill nothing for it.
 template <int R>
-static cudaError_t launch_propagate_r(const K1Args& a, dim3 g, bool pdl, cudaStream_t s) {
+static cudaError_t launch_propagate_r(const K1Args& a, dim3 g, bool pdl, cudaStream_t s, int carveout) {
   if (a.n_tracks == 1)
-    return a.variants ? launch_propagate_rs<R, true, true>(a, g, pdl, s) : launch_propagate_rs<R, true, false>(a, g, pdl, s);
-  if (a.variants) return launch_propagate_rs<R, false, true>(a, g, pdl, s);
-  return launch_propagate_rs<R, false, false>(a, g, pdl, s);
+    return a.variants ? launch_propagate_rs<R, true, true>(a, g, pdl, s, carveout)
+                      : launch_propagate_rs<R, true, false>(a, g, pdl, s, carveout);
+  if (a.variants) return launch_propagate_rs<R, false, true>(a, g, pdl, s, carveout);
+  return launch_propagate_rs<R, false, false>(a, g, pdl, s, carveout);
 }
 
-cudaError_t launch_propagate(const K1Args& a, int R, int grid, bool pdl, cudaStream_t s) {
+cudaError_t launch_propagate(const K1Args& a, int R, int grid, bool pdl, cudaStream_t s, int carveout) {
   const dim3 g(grid);
   switch (R) {
-    case 1: return launch_propagate_r<1>(a, g, pdl, s);
-    case 2: return launch_propagate_r<2>(a, g, pdl, s);
-    case 3: return launch_propagate_r<3>(a, g, pdl, s);
-    case 4: return launch_propagate_r<4>(a, g, pdl, s);
-    case 5: return launch_propagate_r<5>(a, g, pdl, s);
-    case 6: return launch_propagate_r<6>(a, g, pdl, s);
-    case 7: return launch_propagate_r<7>(a, g, pdl, s);
+    case 1: return launch_propagate_r<1>(a, g, pdl, s, carveout);
+    case 2: return launch_propagate_r<2>(a, g, pdl, s, carveout);
+    case 3: return launch_propagate_r<3>(a, g, pdl, s, carveout);
+    case 4: return launch_propagate_r<4>(a, g, pdl, s, carveout);
+    case 5: return launch_propagate_r<5>(a, g, pdl, s, carveout);
+    case 6: return launch_propagate_r<6>(a, g, pdl, s, carveout);
+    case 7: return launch_propagate_r<7>(a, g, pdl, s, carveout);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -3071,27 +3077,41 @@ static cudaError_t launch_resample_t(const ResampleArgs& a, int n_groups, int cl
   return launch_ex(k_resample<NTR, ITEMS, LEAN, EXTRA>, dim3((unsigned)(clusters * cluster)), dim3(NTR), cluster, pdl, s, a, smem);
 }
 
-cudaError_t launch_resample(const ResampleArgs& a0, int n_groups, int cluster, bool pdl, cudaStream_t s, int threads) {
-  // the lean instances while every CTA's chunk fits their registers: 8 items
-  // per thread, 16 for the largest groups (65536 particles on a cluster of 8).
-  // Room for groups off the 16-byte grid is given up where it alone would
-  // take the larger instance (the step of 64 groups of 32767: 132 us with it,
-  // 104 by single loads and stores; of 4 groups of 65535: 45 and 31).
-  ResampleArgs a = a0;
+// Items per thread of the lean instance that a launch takes (0: the general
+// instance), and in `pad` the room for groups off the 16-byte grid.  Lean
+// while every CTA's chunk fits its registers: 8 items per thread, 16 for the
+// largest groups (65536 particles on a cluster of 8).  The room is given up
+// where it alone would take the larger instance (the step of 64 groups of
+// 32767: 132 us with it, 104 by single loads and stores; of 4 groups of 65535:
+// 45 and 31).
+static int lean_items(const ResampleArgs& a, int cluster, int threads, int& pad) {
+  const bool wide = threads == RS_THREADS && a.lean && !a.q_out;
+  pad = a.pad;
   for (int items = RS_ITEMS; items <= 2 * RS_ITEMS; items *= 2)
-    if (rs_chunk_lean(a.max_np, cluster, 0) <= threads * items && rs_chunk_lean(a.max_np, cluster, a.pad) > threads * items)
-      a.pad = 0;
-  const long long chunk = rs_chunk_lean(a.max_np, cluster, a.pad);
+    if (rs_chunk_lean(a.max_np, cluster, 0) <= threads * items && rs_chunk_lean(a.max_np, cluster, pad) > threads * items)
+      pad = 0;
+  const long long chunk = rs_chunk_lean(a.max_np, cluster, pad);
+  if (chunk <= (long long)threads * RS_ITEMS) return RS_ITEMS;
+  return wide && chunk <= (long long)threads * 2 * RS_ITEMS ? 2 * RS_ITEMS : 0;
+}
+
+bool resample_is_lean(const ResampleArgs& a, int cluster, int threads) {
+  int pad;
+  return lean_items(a, cluster, threads, pad) != 0;
+}
+
+cudaError_t launch_resample(const ResampleArgs& a0, int n_groups, int cluster, bool pdl, cudaStream_t s, int threads) {
+  ResampleArgs a = a0;
+  const int items = lean_items(a0, cluster, threads, a.pad);
   const bool small = threads == RS_THREADS_SMALL, extra = !a.lean || a.q_out;
-  if (chunk <= (long long)threads * RS_ITEMS) {
+  if (items == RS_ITEMS) {
     if (small)
       return extra ? launch_resample_t<RS_THREADS_SMALL, RS_ITEMS, true, true>(a, n_groups, cluster, pdl, s)
                    : launch_resample_t<RS_THREADS_SMALL, RS_ITEMS, true, false>(a, n_groups, cluster, pdl, s);
     return extra ? launch_resample_t<RS_THREADS, RS_ITEMS, true, true>(a, n_groups, cluster, pdl, s)
                  : launch_resample_t<RS_THREADS, RS_ITEMS, true, false>(a, n_groups, cluster, pdl, s);
   }
-  if (!small && !extra && chunk <= (long long)RS_THREADS * 2 * RS_ITEMS)
-    return launch_resample_t<RS_THREADS, 2 * RS_ITEMS, true, false>(a, n_groups, cluster, pdl, s);
+  if (items != 0) return launch_resample_t<RS_THREADS, 2 * RS_ITEMS, true, false>(a, n_groups, cluster, pdl, s);
   if (small) return launch_resample_t<RS_THREADS_SMALL, RS_ITEMS, false, true>(a, n_groups, cluster, pdl, s);
   return launch_resample_t<RS_THREADS, RS_ITEMS, false, true>(a, n_groups, cluster, pdl, s);
 }

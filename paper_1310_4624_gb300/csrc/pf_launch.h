@@ -268,7 +268,8 @@ cudaError_t launch_init(const InitArgs& a, int grid, cudaStream_t s);
 // that kernel's completion and memory before touching any buffer.
 cudaError_t launch_frame_prep(const FrameArgs& a, int nt, int blocks_x, bool pdl, cudaStream_t s);
 cudaError_t launch_frame_prep_table(const FrameTableArgs& a, int blocks_x, bool pdl, cudaStream_t s);
-cudaError_t launch_propagate(const K1Args& a, int R, int grid, bool pdl, cudaStream_t s);
+// carveout: shared memory's preferred part of the SM's memory (percent), or -1
+cudaError_t launch_propagate(const K1Args& a, int R, int grid, bool pdl, cudaStream_t s, int carveout = -1);
 // The fused step: propagate + weight tiles, the per-group resampling and the
 // global step in one persistent launch.
 cudaError_t launch_fused_step(const K1Args& a, int R, int grid, bool pdl, cudaStream_t s);
@@ -276,6 +277,8 @@ cudaError_t fused_occupancy(int R, int* blocks_per_sm);
 // threads: RS_THREADS, or RS_THREADS_SMALL (eight CTAs per SM, for batches of small groups)
 cudaError_t launch_resample(const ResampleArgs& a, int n_groups, int cluster, bool pdl, cudaStream_t s,
                             int threads = RS_THREADS);
+// Whether a launch takes a lean instance.
+bool resample_is_lean(const ResampleArgs& a, int cluster, int threads);
 // Largest cluster that the general 512-thread resampler can be launched with:
 // 16 if the device has room for several, else the portable 8.
 int resample_max_cluster();
