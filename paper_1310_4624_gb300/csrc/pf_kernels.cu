@@ -3083,9 +3083,23 @@ static cudaError_t launch_resample_t(const ResampleArgs& a, int n_groups, int cl
 // largest groups (65536 particles on a cluster of 8).  The room is given up
 // where it alone would take the larger instance (the step of 64 groups of
 // 32767: 132 us with it, 104 by single loads and stores; of 4 groups of 65535:
-// 45 and 31).
+// 45 and 31).  The larger lean instance has one CTA an SM, the general one two:
+// it wins while its waves are few, and where the general one just spills into
+// a second wave (n CTAs; groups of 40000, the larger lean instance and the
+// general one: the step of 24, n = 192, 60 and 63 us; of 40, 90 and 101; of 64,
+// 148 and 139.  pf_resample, whose launch nothing overlaps: 24, 30 and 35 us;
+// 32, n = 256, 41 and 36; 40, 42 and 53; 64, 65 and 62).
 static int lean_items(const ResampleArgs& a, int cluster, int threads, int& pad) {
-  const bool wide = threads == RS_THREADS && a.lean && !a.q_out;
+  static const int sms = [] {
+    int dev = 0, n = 0;
+    return cudaGetDevice(&dev) == cudaSuccess &&
+                   cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess
+               ? n
+               : 152;
+  }();
+  const int n = a.n_groups * cluster;
+  const bool few = n <= sms + sms / 2 || (n <= 2 * sms ? a.tile_part != nullptr : n <= 2 * sms + sms / 5);
+  const bool wide = threads == RS_THREADS && a.lean && !a.q_out && few;
   pad = a.pad;
   for (int items = RS_ITEMS; items <= 2 * RS_ITEMS; items *= 2)
     if (rs_chunk_lean(a.max_np, cluster, 0) <= threads * items && rs_chunk_lean(a.max_np, cluster, pad) > threads * items)

@@ -64,3 +64,20 @@ def test_ragged_groups_cost_what_aligned_ones_cost(G, Np):
     ge.build()
     ragged, aligned = _resample_ms(G, Np), _resample_ms(G, (Np + 3) // 4 * 4)
     assert ragged <= 1.4 * aligned, (ragged, aligned)
+
+
+@pytest.mark.parametrize("G", [27, 28, 29, 32, 38, 39, 41, 42, 60])
+@pytest.mark.parametrize("Np", [33001, 65536])
+def test_either_side_of_the_larger_lean_instance(G, Np):
+    """Groups of more than 8 items a thread, as many as take the larger lean
+    instance (one block an SM) or the general one (two), without codes."""
+    import __graft_entry__ as ge
+    from paper_1310_4624_gb300.filter import resample
+    ge.build()
+    rng = np.random.default_rng(G)
+    lw = rng.uniform(-20.0, 0.0, size=(G, Np)).astype(np.float32)
+    u = rng.integers(0, 2 ** 32, size=G, dtype=np.uint64).astype(np.uint32)
+    anc = resample(torch.from_numpy(lw.ravel()).cuda(), torch.from_numpy(u.view(np.int32)).cuda(), G, Np)
+    anc = anc.cpu().numpy().reshape(G, Np)
+    for g in (0, 1, G // 2, G - 1):
+        assert np.array_equal(anc[g], ora.resample(ora.quantize(lw[g]), int(u[g]))), (G, Np, g)
