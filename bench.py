@@ -19,7 +19,7 @@ stepped one by one), the adjoint form (forward with ancestry recording plus
 pf_backward, against the plain forward), the information-sharing start
 (steps until every group mean is within 2 px, PE_eff / G per step) and the
 tracking accuracy over 10 sequences (RMSE, ARNA against RNA 10 %).
---no-extras skips them.
+--no-extras skips them.  Their curves are in the full record on stderr only.
 
 Usage: python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference] [--no-extras]
 Under torchrun each rank runs an independent replica (its own seed and
@@ -712,6 +712,19 @@ def bench_accuracy(dev, n_seq: int = 10):
     return out
 
 
+def short_line(x):
+    """The record without the studies' lists of more than nine values (curves,
+    errors per sequence), and its extra figures to six digits."""
+    def strip(v):
+        if isinstance(v, dict):
+            return {k: strip(w) for k, w in v.items() if not (isinstance(w, list) and len(w) > 9)}
+        if isinstance(v, list):
+            return [strip(w) for w in v]
+        return float("%.6g" % v) if isinstance(v, float) else v
+    exact = ("value", "ms_per_step")
+    return {k: v if k in exact or isinstance(v, str) else strip(v) for k, v in x.items()}
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -892,7 +905,10 @@ def main():
         if not args.no_extras:
             line["oracle_by_config"] = bench_oracle_configs()
     if rank == 0:
-        print(json.dumps(line))
+        # the whole record on stderr, the line itself without long curves: a
+        # reader that keeps only the last few KB of stdout gets all of it
+        print(json.dumps(line), file=sys.stderr)
+        print(json.dumps(short_line(line), separators=(",", ":")))
     if ws > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
