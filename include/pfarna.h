@@ -182,7 +182,14 @@ int32_t pf_abi_version(void);
  * and the per-group and per-step quantities of Alg. 3, sized here
  * for `history` steps of statistics (>= 1; the last `history` steps stay
  * readable through pf_exchange_stats / pf_history).  With record_ancestors
- * set, `history` is also the longest sequence pf_backward can differentiate.
+ * set, `history` is also the longest sequence pf_backward can differentiate,
+ * and the workspace holds, whether or not a gradient is taken, 4 bytes per
+ * particle and step of recorded parents, about 40 bytes per particle and
+ * sqrt(history) of replay states and checkpoints, and 24 bytes per particle
+ * and step for the derivatives that pf_backward keeps: of the whole history up
+ * to 4 GiB, beyond that of as many steps as 4 GiB hold, and of
+ * ceil(sqrt(history)) steps at least.  Handles that never take a gradient
+ * leave record_ancestors 0.
  * Errors: PF_ERR_ARG for invalid configs or NULL pointers. */
 pf_status pf_query_workspace(const pf_track_config* cfg, int32_t n_tracks, int32_t history,
                              size_t* bytes);
@@ -258,7 +265,7 @@ pf_status pf_step_host(pf_handle* h, const float* const* frames_host, void* stag
 pf_status pf_step_table(pf_handle* h, const float* const* table_dev, int32_t T_table, void* stream);
 
 /* pf_step_table through a CUDA graph: the first call (and the first after
- * the table, T_table or the autotuned shapes change) captures the step's
+ * the table, T_table, the autotuned shapes or theta change) captures the step's
  * launches into a graph; every call launches it on `stream`.
  * Errors: as pf_step_table. */
 pf_status pf_graph_step(pf_handle* h, const float* const* table_dev, int32_t T_table, void* stream);
@@ -266,10 +273,14 @@ pf_status pf_graph_step(pf_handle* h, const float* const* table_dev, int32_t T_t
 /* One pf_step that also chooses the launch shapes of the handle's later
  * steps: the propagate kernel's grid (SM count x resident CTAs per SM, 1 ..
  * the occupancy limit) and the resampler's thread-block cluster size
- * (1, 2, 4, 8) and CTA size (512 or 128 threads), each the fastest of the candidates timed with CUDA events
+ * (1, 2, 4, 8; 16 where the handle's own choice is) and CTA size (512 or 128
+ * threads), or with several tracks one CTA per group by class of size
+ * (cluster_out 1), each the fastest of the candidates timed with CUDA events
  * on this step's data (the propagate candidates first: it is idempotent
  * until a resampler replaces the ancestors it reads).  Results
- * are cached per problem shape for the process.  Synchronises the stream.
+ * are cached per problem shape (the device, the patch radius, every track's
+ * groups, their size and method variants) for the process.  Synchronises the
+ * stream.
  * k1_grid_out / cluster_out (may be NULL) receive the choices.
  * Errors: PF_ERR_ARG, PF_ERR_STATE, PF_ERR_CUDA. */
 pf_status pf_autotune(pf_handle* h, const float* const* frames_host, int32_t* k1_grid_out, int32_t* cluster_out,
@@ -443,10 +454,12 @@ pf_status pf_reset(pf_handle* h, void* stream);
  * (every track must have record_ancestors; T = steps run <= history).  The
  * forward pass is replayed from the initial population (drawn again with
  * the current theta) through the recorded parents and the same Philox
- * streams, keeping states only at checkpoints every ceil(sqrt(T)) steps;
- * the reverse sweep recomputes each segment's states and back-propagates
- * through the group log-weights (Alg. 3 steps 4-10), the likelihood and the
- * NCV dynamics.  frames_host: T x n_tracks device pointers, frame k of track
+ * streams, and keeps each step's log-weights and likelihood derivatives, from
+ * which the reverse sweep back-propagates through the likelihood, the NCV
+ * dynamics and the group log-weights (Alg. 3 steps 4-10).  Where the workspace
+ * does not hold the derivatives of T steps, the states are kept at checkpoints
+ * every ceil(sqrt(T)) steps and each segment is replayed again from its
+ * checkpoint.  frames_host: T x n_tracks device pointers, frame k of track
  * t at index k * n_tracks + t (the frames of the forward run).
  * dlogZ_host: n_tracks upstream derivatives.  grad_dev: n_tracks x 5 floats,
  * dlogZ * d log Z / d theta.  logZ_dev: optional n_tracks doubles, the
@@ -476,7 +489,9 @@ pf_status pf_set_replay(pf_handle* h, const uint32_t* parents_dev, int32_t T, vo
 
 /* Checkpoint and resume.  A filter's whole state lives in its workspace
  * and a few host counters, and every random draw is a counter-based Philox
- * word, so a restored filter continues exactly as the saved one would.
+ * word, so a restored filter continues exactly as the saved one would, with
+ * the launch shapes that decide orders of summation and the parameters last
+ * set by pf_set_theta.
  * pf_checkpoint_bytes: the size of a checkpoint of `h`.
  * pf_save: waits for the handle's work on `stream` and copies its state to
  * `host` (bytes >= pf_checkpoint_bytes).

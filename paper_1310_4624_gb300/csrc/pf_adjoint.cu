@@ -231,10 +231,13 @@ __device__ __noinline__ float2 replay_off_box(const ReplayArgs& a, const TrackPa
 // twice (the copy shifted by one float makes every patch row a row of aligned
 // pairs), a tile whose patches do not fit reads the frame through L1.  Bound
 // by FP32 issue (the two patch sums are ~1200 instructions a particle) and the
-// latency of the gathers before them.  Derivatives by column sums in packed
-// pairs took 55 us a million particles, but moved the gradient by up to 2e-5
-// (their error was smaller; results are held to the older order: gradient of
-// 16 x 65536 particles over 20 frames 7.7 -> 4.2 ms, 3.5 with the packed sums).
+// latency of the gathers before them: 84 us a million particles, a gradient of
+// 16 x 65536 particles over 20 frames 7.7 ms when each step's patches were
+// summed by the replay and again by the reverse sweep, 4.1 now.  Derivatives
+// by column sums in packed pairs would take 55 us.  They are in another order,
+// which moves the gradient by up to 2e-5 of its largest component (and nearer
+// to the 64-bit value): a library update would then change the iterates of a
+// parameter fit, so the order of the sums is kept as part of the result.
 // SINGLE: one track, its parameters and round keys in the constant bank.
 template <int R, bool SINGLE>
 __global__ void __launch_bounds__(K1_THREADS, 4) k_replay(const __grid_constant__ ReplayArgs a) {

@@ -20,6 +20,9 @@
 //                       reduction (steps 9-10), the weight carry (step 8),
 //                       the next ring order (step 1) and exchange count
 //                       (step 2, Eq. 3/4) -- once every group has reported
+// A handle of several tracks resamples by k_resample_groups, one CTA (or one
+// warp) per group in a launch per class of group size; a few large groups of
+// it take k_resample's clusters beside them.
 // A batch of tracks given device frames first pads them (k_frame_prep);
 // k_global prepares step 0; k_finish / k_finish_out complete the last
 // step's statistics when the host reads them.  The step index lives on the
